@@ -23,6 +23,8 @@ using namespace bridges;
 namespace {
 
 constexpr size_t kMiscBytes = 1024;  // status word, device counts of bridges_from_forest, spare output
+constexpr size_t kClearBytes = kMiscBytes + 256;  // cleared at a call's start: the misc area and the
+                                                  // certificate's control words, which follow it
 constexpr size_t kSpareAt = 512;     // the spare output slot: where a call that has no pairs or points
                                      // to write (V <= 1, null output) points the stages
 
@@ -69,6 +71,8 @@ Carved carve(bridges_ctx* c, const CertPlan& p) {
   k.cert = carve_cert(base + kMiscBytes, p);
   k.cert.status = k.status;
   k.fin = carve_final(base + kMiscBytes + align_up(cert_bytes(p), 256), p.V, k.status);
+  k.cert.hook = reinterpret_cast<unsigned long long*>(k.fin.sr);
+  k.cert.roots = k.fin.sr2;
   return k;
 }
 
@@ -215,10 +219,10 @@ int64_t run_path(bridges_ctx* c, cudaStream_t s, const int32_t* u, const int32_t
   c->last_cfg[4] = p.cache ? p.warm : -1;
   cudaEvent_t* ev = next_event_slot(c);
   if (ev) cudaEventRecord(ev[7], s);
-  cudaMemsetAsync(k.status, 0, sizeof(int32_t), s);
+  cudaMemsetAsync(k.status, 0, kClearBytes, s);
   cert_init(L, p, k.cert);
   cert_leaves(L, p, k.cert, u, v, ev);
-  if (ev && E == 0)
+  if (ev && E == 0 && !p.sampled)
     for (int i = 0; i < 4; i++) cudaEventRecord(ev[i], s);
   cert_merge(L, p, k.cert);
   if (ev) cudaEventRecord(ev[4], s);
@@ -349,8 +353,9 @@ static int64_t issue_chunks(bridges_ctx* c, cudaStream_t s, const int32_t* hu, c
 int64_t run_path_host(bridges_ctx* c, cudaStream_t s, const int32_t* hu, const int32_t* hv, int32_t* du, int32_t* dv,
                       int64_t E, int32_t V, int32_t M, int32_t* out, Carved* kout, bool bridges_only) {
   Range range("bridges: pipelined host input");
-  const CertPlan p = plan_for(c, E, V, M);
+  CertPlan p = plan_for(c, E, V, M);
   if (p.M != 1 || !p.cache) return 1;
+  p.stride = 0;  // a prefix, not a sample of the whole list: it has to be on the device first
   int64_t C = 0;
   int K = 0;
   if (!chunk_plan(E, p.warm, &C, &K)) return 1;
@@ -367,7 +372,7 @@ int64_t run_path_host(bridges_ctx* c, cudaStream_t s, const int32_t* hu, const i
   if (rc != BRIDGES_OK) return rc;
   cudaEvent_t* ev = next_event_slot(c);
   if (ev) cudaEventRecord(ev[7], s);
-  cudaMemsetAsync(k.status, 0, sizeof(int32_t), s);
+  cudaMemsetAsync(k.status, 0, kClearBytes, s);
   cert_init(L, p, k.cert);
   cudaStreamWaitEvent(s, c->chunk_ev[0], 0);  // the first chunk holds the warm-up prefix (C >= warm)
   if (ev) cudaEventRecord(ev[0], s);
@@ -1310,6 +1315,17 @@ static CertPlan block_pass_plan(const bridges_ctx* c, int64_t E, int32_t V) {
   return q;
 }
 
+// The plan of the articulation-point path's certificate: as for the bridges alone, but with a
+// snapshot also for a list that the bridge path would certify whole (its one read of the list then
+// serves both passes).
+static CertPlan ap_plan(const bridges_ctx* c, int64_t E, int32_t V, int32_t M) {
+  const CertPlan p = plan_for(c, E, V, M);
+  if (!p.sampled || p.cache || c->opts.warm_edges >= 0) return p;
+  const bridges_opts& o = c->opts;
+  return make_plan(E, V, p.M, o.fan_in, o.block, o.ctas_per_sm, 8 * (int64_t)V + 4096, c->num_sms, c->smem_optin,
+                   o.warm_block);
+}
+
 // One read of the list for both passes: one partition with a 16-bit label snapshot.
 static bool fused_eligible(const bridges_ctx* c, const CertPlan& p, int64_t E, int32_t V) {
   return c->opts.ap_fused >= 0 && p.M == 1 && p.cache && p.mode == 1 && V >= 2 && E > p.warm;
@@ -1323,7 +1339,7 @@ static size_t fused_ws_bytes(const CertPlan& p, int32_t V) {
 
 // The fused form.  With host edges (hu, hv) not yet on the device, (u, v) is their device
 // staging: the copy runs in chunks and the stream follows it chunk by chunk.
-static int64_t articulation_fused_run(bridges_ctx* c, cudaStream_t s, const Launch& L, const CertPlan& p,
+static int64_t articulation_fused_run(bridges_ctx* c, cudaStream_t s, const Launch& L, CertPlan p,
                                       const int32_t* u, const int32_t* v, int64_t E, int32_t V, int32_t* out_points,
                                       int32_t* out_bridges, int64_t* out_counts_device, const int32_t* hu,
                                       const int32_t* hv) {
@@ -1361,6 +1377,7 @@ static int64_t articulation_fused_run(bridges_ctx* c, cudaStream_t s, const Laun
       rc = issue_chunks(c, s, hu, hv, const_cast<int32_t*>(u), const_cast<int32_t*>(v), E, C, K);
       if (rc) return rc;
       chunks = ChunkSchedule{c->chunk_ev, C, K};
+      p.stride = 0;  // a prefix, not a sample of the whole list: it has to be on the device first
     } else if (E > 0 &&
                (cudaMemcpyAsync(const_cast<int32_t*>(u), hu, sizeof(int32_t) * (size_t)E, cudaMemcpyHostToDevice, s) !=
                     cudaSuccess ||
@@ -1369,7 +1386,7 @@ static int64_t articulation_fused_run(bridges_ctx* c, cudaStream_t s, const Laun
       return cuda_fail(cudaGetLastError());
     }
   }
-  cudaMemsetAsync(k.status, 0, sizeof(int32_t), s);
+  cudaMemsetAsync(k.status, 0, kClearBytes, s);
   cert_init(L, p, k.cert);
   articulation_fused(L, p, k.cert, k.fin, b0, b1, fb, u, v, out_points, out_bridges, b1.count, bev, aev, chunks);
   if (bev) c->calls++;
@@ -1394,7 +1411,7 @@ static int64_t articulation_fused_run(bridges_ctx* c, cudaStream_t s, const Laun
 static int64_t articulation_run(bridges_ctx* c, cudaStream_t s, const int32_t* u, const int32_t* v, int64_t E, int32_t V,
                          int32_t M, int32_t* out_points, int32_t* out_bridges, int64_t* out_counts_device,
                          const int32_t* hu, const int32_t* hv) {
-  const CertPlan p0 = plan_for(c, E, V, M);
+  const CertPlan p0 = ap_plan(c, E, V, M);
   const size_t ap_at = align_up(total_bytes(p0), 256);
   Launch L = launch_for(c, s);
   // the fused form when it applies and its larger workspace fits the caller's limits, else two passes
@@ -1493,7 +1510,7 @@ extern "C" int64_t bridges_articulation_points_host(bridges_ctx* c, struct CUstr
 
 extern "C" int64_t bridges_articulation_workspace_bytes(const bridges_ctx* c, int64_t E, int32_t V, int32_t M) {
   if (!c || E < 0 || V < 0) return 0;
-  const CertPlan p = plan_for(c, E, V, M);
+  const CertPlan p = ap_plan(c, E, V, M);
   const size_t two_pass = align_up(total_bytes(p), 256) + ap_bytes(V);
   if (!fused_eligible(c, p, E, V)) return (int64_t)two_pass;
   return (int64_t)std::max(two_pass, fused_ws_bytes(p, V));

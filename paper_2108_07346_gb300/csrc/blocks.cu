@@ -450,6 +450,7 @@ struct FusedArgs {
   const int32_t* u;
   const int32_t* v;
   int64_t s, t;           // edge range of this launch
+  uint32_t stride;        // > 1: every stride-th group of the list is in the certificate already
   const uint16_t* lab;    // combined labels (Vpad entries)
   int64_t Vpad;
 };
@@ -460,7 +461,7 @@ template <bool FOREST>
 __device__ __forceinline__ void fused_edge(const FusedArgs& F, bool go, int32_t a, int32_t b, int64_t i) {
   int r = 0;
   if (FOREST) {
-    r = go ? offer(F.J, a, b) : 0;
+    r = go && !excluded(i, F.stride) ? offer(F.J, a, b) : 0;
     warp_append(r == 1, a, b, F.J.cnt + 0, F.J.f1u, F.J.f1v, F.A.V, F.A.status);
     warp_append(r == 2, a, b, F.J.cnt + 1, F.J.f2u, F.J.f2v, F.A.V, F.A.status);
   }
@@ -802,15 +803,20 @@ void articulation_fused(const Launch& L, const CertPlan& p, const CertBufs& cb, 
   const int grid = (int)std::max<int64_t>(1, (int64_t)p.G);
   const Job J{cb.P1, cb.P2, cb.f1u, cb.f1v, cb.f2u, cb.f2v, cnt};
   FusedArgs a{ApArgs{f.pre, b0.Q, b0.PP, b0.LAST, V, f.status, b0.hooks}, J, f.root, fb.keep, fb.top, u, v, 0,
-              p.warm, cb.lab, cb.Vpad};
-  if (vec)
-    launch_fused<false, true>(L, a, grid, p.block);
-  else
-    launch_fused<false, false>(L, a, grid, p.block);
+              p.warm, p.sampled && p.stride > 1 ? (uint32_t)p.stride : 0u, cb.lab, cb.Vpad};
+  // a certified prefix has only the block pass left; a certified sample is passed over by the
+  // stream's forest half
+  const int64_t first = a.stride > 1 ? 0 : p.warm;
+  if (first > 0) {
+    if (vec)
+      launch_fused<false, true>(L, a, grid, p.block);
+    else
+      launch_fused<false, false>(L, a, grid, p.block);
+  }
   const int K = chunks.ev ? chunks.K : 1;
   for (int i = 0; i < K; i++) {  // the rest of the list, chunk by chunk behind a host copy
     if (i > 0) cudaStreamWaitEvent(L.stream, chunks.ev[i], 0);
-    a.s = chunks.ev ? std::max<int64_t>(p.warm, chunks.C * i) : p.warm;
+    a.s = chunks.ev ? std::max<int64_t>(first, chunks.C * i) : first;
     a.t = chunks.ev ? std::min<int64_t>(p.E, chunks.C * (i + 1)) : p.E;
     if (a.t <= a.s) continue;
     if (vec)

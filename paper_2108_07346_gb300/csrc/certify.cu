@@ -68,7 +68,8 @@ __device__ __forceinline__ void scalar_slot(const Job& J, bool valid, int32_t a,
 // Kept out of line so the streaming loop stays small; the edges are re-read (they are still in
 // L1/L2).
 __device__ __noinline__ void offer_misses(const Job& J, uint32_t m, const int32_t* __restrict__ u,
-                                          const int32_t* __restrict__ v, int64_t base, int32_t V, int32_t* status) {
+                                          const int32_t* __restrict__ v, int64_t base, int32_t V, int32_t* status,
+                                          int64_t first, uint32_t stride) {
   while (__any_sync(kFull, m != 0)) {
     int32_t a = 0, b = 0;
     bool go = false;
@@ -78,7 +79,7 @@ __device__ __noinline__ void offer_misses(const Job& J, uint32_t m, const int32_
       const int64_t e = miss_edge(bit, base);
       a = u[e];
       b = v[e];
-      go = checked(a, b, V, status);
+      go = checked(a, b, V, status) && !excluded(first + e, stride);
     }
     const int r = go ? offer(J, a, b) : 0;
     warp_append(r == 1, a, b, J.cnt + 0, J.f1u, J.f1v, V, status);
@@ -91,11 +92,13 @@ struct ForestSink {
   const Job& J;
   int32_t V;
   int32_t* status;
-  __device__ __forceinline__ void slot(bool need, int32_t a, int32_t b, int64_t) const {
-    settle(J, need && checked(a, b, V, status), a, b, V, status);
+  const int32_t* u;  // the list's start, and the stride of the sample already certified
+  uint32_t stride;
+  __device__ __forceinline__ void slot(bool need, int32_t a, int32_t b, int64_t i) const {
+    settle(J, need && checked(a, b, V, status) && !excluded(i, stride), a, b, V, status);
   }
   __device__ __forceinline__ void misses(uint32_t m, const int32_t* ub, const int32_t* vb, int64_t base) const {
-    offer_misses(J, m, ub, vb, base, V, status);
+    offer_misses(J, m, ub, vb, base, V, status, ub - u, stride);
   }
 };
 
@@ -112,6 +115,7 @@ struct LeafArgs {
   int32_t mode;  // 0: warm-up prefix of each chunk, 1: the rest of each chunk
   int32_t Vb;    // bitmap snapshot: vertices it covers
   int64_t r0, r1;  // mode 1: only edges [r0, r1) of the rest (r1 <= r0: all of it)
+  uint32_t stride;  // > 1: every stride-th group was certified before (a sample of the whole chunk)
   CertBufs b;
 };
 
@@ -122,9 +126,13 @@ struct LeafArgs {
 template <int MODE, bool VEC>
 __global__ void __launch_bounds__(1024, 1) leaf_kernel(LeafArgs A) {
   extern __shared__ __align__(16) uint16_t slab[];
+  __shared__ int32_t stop;
+  if (threadIdx.x == 0) stop = A.mode == 1 ? ld_relaxed(A.b.status) : 0;
+  __syncthreads();
+  if (stop) return;  // an earlier step failed: its labels and union-finds may be unset
   const int64_t j = blockIdx.x / A.G, m = blockIdx.x % A.G;
   const int64_t lo = A.E * j / A.M, hi = A.E * (j + 1) / A.M;
-  const int64_t w = min(A.warm, hi - lo);
+  const int64_t w = A.stride > 1 ? 0 : min(A.warm, hi - lo);
   int64_t a = A.mode == 0 ? lo : lo + w;
   int64_t z = A.mode == 0 ? lo + w : hi;
   if (A.mode == 1 && A.r1 > A.r0) {
@@ -134,7 +142,7 @@ __global__ void __launch_bounds__(1024, 1) leaf_kernel(LeafArgs A) {
   if (MODE == 1) load_labels(slab, A.b.lab + j * A.b.Vpad, A.b.Vpad);
   if (MODE == 2) load_words(slab, A.b.lab + j * A.b.Vpad, (A.Vb / 32 + 4) / 4);
   const Job J = job_of(A.b, A.V, j);
-  const ForestSink S{J, A.V, A.b.status};
+  const ForestSink S{J, A.V, A.b.status, A.u, A.mode == 1 ? A.stride : 0};
   const uint32_t clampv = MODE == 2 ? (uint32_t)A.Vb : (uint32_t)A.V;
   if (A.mode == 1 && use_tiles(a, z, A.G, blockDim.x, kUnroll)) {
     stream_range<MODE, VEC, kUnroll>(S, A.u, A.v, a, z, clampv, slab, m, A.G);
@@ -415,6 +423,27 @@ CertPlan make_plan(int64_t E, int32_t V, int32_t M, int32_t fan_in, int32_t bloc
   p.G = (int32_t)std::max<int64_t>(1, ((int64_t)num_sms * cps) / p.M);
   p.warm_block = p.block;
   const int64_t chunk = ceil_div(std::max<int64_t>(E, 1), p.M);
+  p.sampled = p.M == 1 && labels_fit && warm != 0;
+  if (p.sampled) {
+    // One partition: the sample of cert_sample.  8V edges leave a vertex of a random dense graph
+    // out of F' (fewer than two sampled edges) with probability 2e-6, and every such vertex sends
+    // all its edges down the stream's slow path; a list of at most twice that is certified whole.
+    // With too many vertices for labels the prefix below stays: a round visits every vertex
+    // (R-MAT, 2^20 vertices, 1.05 M edges: 227 us for prefix and bitmap, 245 us in rounds).
+    const int64_t cap = sample_capacity(num_sms);
+    if (warm < 0) {
+      warm = 8 * (int64_t)V + 4096;
+      if (E <= 2 * warm) warm = E;
+    }
+    warm = std::min(warm, cap);
+    const int64_t groups = ceil_div(E, 1 << kSampleShift);
+    p.stride = E <= warm ? 1 : ceil_div(groups, std::max<int64_t>(warm >> kSampleShift, 1));
+    p.cache = E > warm;
+    p.warm = warm;
+    p.warm_block = p.block;
+    return p;
+  }
+  // Several partitions, or no labels: each partition certifies its own prefix.
   // Twice the edges after which F' holds a giant component in a dense random partition: at about
   // 0.6 V ln V the snapshot still misses a few vertices whose edges then all take the union-find
   // path (measured on the large workload: 41 k such edges and a 2.3x slower forest pass at
@@ -443,7 +472,7 @@ size_t cert_bytes(const CertPlan& p) {
   const size_t MV = (size_t)p.M * (size_t)std::max(p.V, 1);
   const size_t Vpad = align_up((size_t)p.V + 1, 8);
   size_t s = 0;
-  s += 256;                                         // status
+  s += 256;                                         // ctl
   s += align_up(sizeof(int32_t) * 2 * p.M, 256);    // cnt
   s += align_up(sizeof(int32_t) * p.M, 256);        // nlab
   s += align_up(sizeof(unsigned long long) * p.M, 256);  // giant
@@ -457,7 +486,7 @@ CertBufs carve_cert(void* base, const CertPlan& p) {
   char* c = static_cast<char*>(base);
   const size_t MV = (size_t)p.M * (size_t)std::max(p.V, 1);
   const size_t Vpad = align_up((size_t)p.V + 1, 8);
-  b.status = reinterpret_cast<int32_t*>(c);
+  b.ctl = reinterpret_cast<unsigned*>(c);
   c += 256;
   b.cnt = reinterpret_cast<int32_t*>(c);
   c += align_up(sizeof(int32_t) * 2 * p.M, 256);
@@ -476,13 +505,18 @@ CertBufs carve_cert(void* base, const CertPlan& p) {
 }
 
 void cert_init(const Launch& L, const CertPlan& p, const CertBufs& b) {
+  if (p.sampled) return;  // cert_sample initialises what it uses
   init_kernel<<<grid_for(L, (int64_t)p.M * p.V, 256), 256, 0, L.stream>>>(b, p.V, p.M);
   *L.launches += 1;
 }
 
 void cert_warm(const Launch& L, const CertPlan& p, const CertBufs& b, const int32_t* u, const int32_t* v) {
+  if (p.sampled) {
+    cert_sample(L, p, b, u, v);
+    return;
+  }
   if (p.E == 0) return;
-  const LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 0, p.Vb, 0, 0, b};
+  const LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 0, p.Vb, 0, 0, 0, b};
   if (((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v)) & 15) == 0)
     launch_leaf<0, true>(L, p, a, 0);
   else
@@ -490,7 +524,7 @@ void cert_warm(const Launch& L, const CertPlan& p, const CertBufs& b, const int3
 }
 
 void cert_snapshot(const Launch& L, const CertPlan& p, const CertBufs& b) {
-  if (p.E == 0 || !p.cache) return;
+  if (p.E == 0 || !p.cache || p.sampled) return;
   if (p.mode == 1)
     snapshot(L, p, b, 1, p.M);
   else
@@ -500,7 +534,7 @@ void cert_snapshot(const Launch& L, const CertPlan& p, const CertBufs& b) {
 void cert_stream(const Launch& L, const CertPlan& p, const CertBufs& b, const int32_t* u, const int32_t* v, int64_t r0,
                  int64_t r1) {
   if (p.E == 0 || !p.cache) return;
-  const LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 1, p.Vb, r0, r1, b};
+  const LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 1, p.Vb, r0, r1, p.sampled ? (uint32_t)p.stride : 0u, b};
   const bool vec = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v)) & 15) == 0;
   if (p.mode == 1) {
     const size_t smem = (size_t)b.Vpad * 2;
@@ -519,7 +553,7 @@ void cert_stream(const Launch& L, const CertPlan& p, const CertBufs& b, const in
 
 void cert_leaves(const Launch& L, const CertPlan& p, const CertBufs& b, const int32_t* u, const int32_t* v,
                  cudaEvent_t* ev) {
-  if (p.E == 0) return;
+  if (p.E == 0 && !p.sampled) return;
   if (ev) cudaEventRecord(ev[0], L.stream);
   cert_warm(L, p, b, u, v);
   if (ev) cudaEventRecord(ev[1], L.stream);

@@ -35,7 +35,7 @@
 // barrier.
 #include <algorithm>
 
-#include "common.cuh"
+#include "grid.cuh"
 
 namespace bridges {
 
@@ -50,7 +50,6 @@ constexpr int kMaxSup = 1024;        // superchunks covered by the shared-memory
 constexpr int kSupLevels = 11;       // log2(kMaxSup) + 1
 constexpr int64_t kRankMax = 16384;  // up to this many bridges: slice sort + merge ranking
 constexpr int kSortSlice = 256;      // keys per sorted slice at most (the small-n sort)
-constexpr unsigned kSpinCap = 1u << 22;
 constexpr int kHopsLog = 2;  // pointer-jumping hops per round: 4 (8 was slower: longer load chains)
 constexpr int kHops = 1 << kHopsLog;
 constexpr int kMaxBlocks = 1024;
@@ -78,58 +77,14 @@ struct FinArgs {
   int32_t hold_polls;  // > 0: the last block sleeps this many ~100 ns polls before its first barrier
 };
 
-__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
-__device__ __forceinline__ void red_add_release(unsigned* p, unsigned v) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// Grid-wide barrier for a cooperative launch, on a counter that only grows within the launch
-// (cleared before it): barrier k ends once the counter reaches k * gridDim.  Thread 0 of each
-// block counts its barriers in shared memory (*epoch), arrives with one release add that returns
-// nothing, and polls the counter with acquire loads -- one round trip to memory per poll and
-// none for the arrival (against about 3 us per barrier for an acquire-release add that returns,
-// a generation word and its release store).  The block's writes are ordered before its thread 0
-// by the block barrier, the release add publishes them, and the acquire that sees the count
-// carries everyone's to the block.  Returns false if the wait gave up: the status word then holds
-// BRIDGES_ETIMEDOUT (or an earlier error) and the caller must leave the kernel.  Every other
-// block then gives up at its next barrier, so the block that would write the count after the
-// last phase never gets there; the count is set to that first error here instead, so that a
-// caller never reads the count of an earlier call.
-__device__ __noinline__ bool grid_barrier(const FinalBufs& f, unsigned polls, unsigned* epoch) {
-  __shared__ int ok;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    ok = 1;
-    const unsigned target = (*epoch += 1) * gridDim.x;
-    red_add_release(f.bar_count, 1u);
-    if (!bounded_poll([&] { return (int)(ld_acquire(f.bar_count) - target) >= 0; }, polls)) {
-      const int32_t first = atomicCAS(f.status, 0, BRIDGES_ETIMEDOUT_CODE);
-      *f.count = (int64_t)(first != 0 ? first : BRIDGES_ETIMEDOUT_CODE);
-      ok = 0;
-    }
-  }
-  __syncthreads();
-  return ok != 0;
+__device__ __forceinline__ bool grid_barrier(const FinalBufs& f, unsigned polls, unsigned* epoch) {
+  return bridges::grid_barrier(f.bar_count, f.status, f.count, polls, epoch);
 }
 
 #define BARRIER()                                         \
   do {                                                    \
     if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return; \
   } while (0)
-
-__device__ __forceinline__ int64_t gtid() { return (int64_t)blockIdx.x * blockDim.x + threadIdx.x; }
-__device__ __forceinline__ int64_t gstride() { return (int64_t)gridDim.x * blockDim.x; }
-// This thread's index among all threads with the warps dealt round-robin over the blocks (warp w
-// of block b is global warp w * gridDim + b): a loop over fewer items than threads still spreads
-// them over every SM, and each warp still takes 32 consecutive items.
-__device__ __forceinline__ int64_t gspread() {
-  return (((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) << 5) + (threadIdx.x & 31);
-}
 
 // Block-wide sum (every thread gets the result).
 __device__ __forceinline__ int32_t block_sum(int32_t v, int32_t* red) {
@@ -347,6 +302,13 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
   const int32_t nx = min(*A.d_nx, A.cx);
   const int64_t na = 2 * (int64_t)nt;  // tree arcs
   const int64_t nchunks = (V + kChunk - 1) / kChunk;
+
+  // an earlier stage failed: its lists and union-finds may be unset (nothing sets the status between
+  // a block's start here and the first barrier, so every block sees the same)
+  if (ld_relaxed(f.status) != 0) {
+    if (gtid() == 0) *f.count = (int64_t)ld_relaxed(f.status);
+    return;
+  }
 
   // a test knob: hold the last block back (a bounded sleep) so that the others' first barrier
   // gives up; never set in normal use

@@ -15,6 +15,9 @@ namespace bridges {
 // Sentinel label: "no class", never equal to another vertex's label.
 constexpr uint16_t kNoLabel = 0xffff;
 
+// The sample of a plan is taken in groups of 2^kSampleShift edges.
+constexpr int kSampleShift = 3;
+
 // One launch context: the stream and the context's launch counter.
 struct Launch {
   cudaStream_t stream;
@@ -38,6 +41,9 @@ struct CertPlan {
   int32_t block;   // threads per block in the forest pass
   int32_t warm_block;  // threads per block of its warm-up launch
   int64_t warm;    // edges per partition certified before the snapshot (>= partition: no cache)
+  bool sampled;    // one partition: those edges advance in rounds together (cert_sample) ...
+  int64_t stride;  // ... and are every stride-th group of the list (0: its first `warm` edges;
+                   // 1: the whole list)
   bool cache;      // a snapshot is taken after the warm-up
   int32_t mode;    // its form: 1 = 16-bit F' labels (2V bytes fit in shared memory), 2 = bitmap
                    // of the largest F' component (for larger V)
@@ -48,6 +54,9 @@ struct CertPlan {
 // slices [j*V, (j+1)*V) of P1, P2, f1u, f1v, f2u, f2v, tmp and lab (lab stride Vpad).
 struct CertBufs {
   int32_t* status;  // [1] device status word
+  unsigned* ctl;    // [64] the sampled certificate's barrier word and counters (cleared by every call)
+  unsigned long long* hook;  // [2V] its hooks and
+  int2* roots;               // [V] its roots in both forests (scratch of the final stage, idle until then)
   int32_t* cnt;     // [2*M] forest sizes |F|, |F'| per job
   int32_t* nlab;    // [M] labels handed out per job
   unsigned long long* giant;  // [M] bitmap snapshot: (size << 32 | ~root) of the largest F' component
@@ -146,6 +155,14 @@ void cert_warm(const Launch& L, const CertPlan& p, const CertBufs& b, const int3
 void cert_snapshot(const Launch& L, const CertPlan& p, const CertBufs& b);
 void cert_stream(const Launch& L, const CertPlan& p, const CertBufs& b, const int32_t* u, const int32_t* v, int64_t r0,
                  int64_t r1);
+// ---- sample.cu ----
+// The first steps of a sampled plan in one cooperative launch: initialises the union-finds and the
+// lists, certifies the sample and writes the snapshot (none when the sample is the whole list).
+void cert_sample(const Launch& L, const CertPlan& p, const CertBufs& b, const int32_t* u, const int32_t* v);
+// Edges a sample may hold.
+int64_t sample_capacity(int num_sms);
+
+// ---- certify.cu, continued ----
 // Merge tree (Sec. 3 phases): fan-in f until one certificate remains in job 0.
 void cert_merge(const Launch& L, const CertPlan& p, const CertBufs& b);
 // Plan for (E, V, M) on this device.

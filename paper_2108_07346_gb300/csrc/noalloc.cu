@@ -88,15 +88,18 @@ extern "C" int64_t bridges_find_noalloc(struct CUstream_st* stream, const int32_
   CertBufs cb = carve_cert(base + kMiscBytes, p);
   cb.status = status;
   FinalBufs fb = carve_final(base + kMiscBytes + cert, p.V, status);
+  cb.hook = reinterpret_cast<unsigned long long*>(fb.sr);
+  cb.roots = fb.sr2;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   Launch L{s, &S->launches, S->num_sms, S->smem_optin};
   // a graph of at most one vertex has no pairs to write; its output pointer may be null, so the
   // stage gets a slot of the scratch array instead (a device address, never a host one)
   int32_t* spare_out = reinterpret_cast<int32_t*>(base + kSpareOut);
 
-  // The array keeps whatever the previous call left: the status word is cleared here, and every
+  // The array keeps whatever the previous call left: the status word and the certificate's control
+  // words (which follow the misc area) are cleared here, and every
   // other buffer that must start at zero is initialised by the stages themselves.
-  if (cudaMemsetAsync(status, 0, sizeof(int32_t), s) != cudaSuccess) {
+  if (cudaMemsetAsync(status, 0, kMiscBytes + 256, s) != cudaSuccess) {
     cudaGetLastError();
     return BRIDGES_ECUDA;
   }

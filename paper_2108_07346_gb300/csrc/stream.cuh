@@ -137,6 +137,12 @@ __device__ __forceinline__ void stream_range(const Sink& S, const int32_t* __res
   }
 }
 
+// Whether list index i belongs to the sample that was certified before the stream: every
+// stride-th group of 8 edges (stride < 2: no sample, or one that the stream does not read).
+__device__ __forceinline__ bool excluded(int64_t i, uint32_t stride) {
+  return stride > 1 && (uint32_t)(i >> kSampleShift) % stride == 0;
+}
+
 // Whether `members` blocks of nt threads share [s, t) in interleaved tiles (true) or take one
 // slice each (false): tiles only when every block gets at least 16 of them -- a tile is 4U edges
 // per thread, so on a short list tiles would leave blocks idle (a 1 M-edge list has 61 tiles of

@@ -1,0 +1,98 @@
+"""The sampled certificate (sample.cu) at the sizes where it can go wrong: one and several edges a
+thread, label and bitmap limits, lists certified whole and lists with a stream behind the sample,
+long chains, hubs, parallel edges, lists sorted by their ends, unaligned starts -- against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def _er(rng, V, E):
+    return rng.integers(0, V, E).astype(np.int32), rng.integers(0, V, E).astype(np.int32)
+
+
+def _check(pb, u, v, V, **opts):
+    import torch
+
+    du, dv = torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda()
+    ctx = pb.Context(device="cuda:0", **opts)
+    ref = oracle.dfs_bridges(u, v, V) if hasattr(oracle, "dfs_bridges") else oracle.bridges(u, v, V, 1)
+    for _ in range(2):  # the second call finds the first one's workspace
+        got = ctx.find(du, dv, V).cpu().numpy()
+        assert got.tolist() == np.asarray(ref).reshape(-1, 2).tolist()
+    cu, cv, ct = (t.cpu().numpy() for t in ctx.certificate(du, dv, V))
+    # F spans what the list spans, F' lies inside F's sets, and neither holds a cycle
+    comps = oracle.components(u, v, V)[1]
+    assert int(ct.sum()) == V - len(np.unique(comps))
+    f, f2 = (cu[ct], cv[ct]), (cu[~ct], cv[~ct])
+    assert np.array_equal(oracle.components(f[0].copy(), f[1].copy(), V)[1], comps)
+    c2 = oracle.components(f2[0].copy(), f2[1].copy(), V)[1]
+    assert len(f2[0]) == V - len(np.unique(c2))
+
+
+@pytest.mark.parametrize("V,E", [(1, 3), (2, 1), (33, 20), (1000, 999), (5000, 2 * (8 * 5000 + 4096)),
+                                 (5000, 2 * (8 * 5000 + 4096) + 1), (20011, 900_001), (65_534, 400_000),
+                                 (65_535, 1_300_000), (65_536, 1_300_001), (90_000, 3_000_000), (120_001, 2_500_000)])
+def test_random_lists(cuda_lib, V, E):
+    rng = np.random.default_rng(V * 7 + E)
+    _check(cuda_lib, *_er(rng, V, E), V)
+
+
+@pytest.mark.parametrize("V", [4097, 60_000, 130_000])
+@pytest.mark.parametrize("shape", ["path", "reversed path", "star", "doubled path", "two hubs"])
+def test_chains_and_hubs(cuda_lib, V, shape):
+    x = np.arange(V - 1, dtype=np.int32)
+    if shape == "path":
+        u, v = x, x + 1
+    elif shape == "reversed path":
+        u, v = x[::-1].copy() + 1, x[::-1].copy()
+    elif shape == "star":
+        u, v = np.full(V - 1, V - 1, np.int32), x
+    elif shape == "doubled path":
+        u, v = np.concatenate([x, x + 1]), np.concatenate([x + 1, x])
+    else:
+        u = np.concatenate([np.full(V - 1, V - 1, np.int32), np.full(V - 1, V // 2, np.int32)])
+        v = np.concatenate([x, x])
+    _check(cuda_lib, u.astype(np.int32), v.astype(np.int32), V)
+
+
+@pytest.mark.parametrize("V,E,warm", [(3000, 300_000, -1), (70_000, 2_000_000, -1), (70_000, 2_000_000, 5000),
+                                      (3000, 300_000, 64), (130_000, 3_000_000, 200_000)])
+def test_sorted_lists(cuda_lib, V, E, warm):
+    rng = np.random.default_rng(E + warm)
+    u, v = _er(rng, V, E)
+    lo, hi = np.minimum(u, v), np.maximum(u, v)
+    order = np.lexsort((hi, lo))
+    u, v = lo[order].copy(), hi[order].copy()
+    u = np.concatenate([u, np.arange(V, V + 40, dtype=np.int32)])  # a pendant path at the end
+    v = np.concatenate([v, np.arange(V - 1, V + 39, dtype=np.int32)])
+    _check(cuda_lib, u, v, V + 40, warm_edges=warm)
+
+
+@pytest.mark.parametrize("skip", [1, 2, 3])
+def test_unaligned_slices(cuda_lib, skip):
+    import torch
+
+    rng = np.random.default_rng(skip)
+    V, E = 2500, 200_003
+    u, v = _er(rng, V, E)
+    du, dv = torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda()
+    got = cuda_lib.Context(device="cuda:0").find(du[skip:], dv[skip:], V).cpu().numpy()
+    assert got.tolist() == oracle.bridges(u[skip:].copy(), v[skip:].copy(), V, 1).tolist()
+
+
+@pytest.mark.parametrize("E,at", [(500, 499), (300_000, 0), (300_000, 299_999), (300_000, 150_001)])
+def test_ids_out_of_range(cuda_lib, E, at):
+    import torch
+
+    rng = np.random.default_rng(at)
+    V = 5000
+    u, v = _er(rng, V, E)
+    u[at] = V
+    v[at] = V  # a loop out of range is an error all the same
+    ctx = cuda_lib.Context(device="cuda:0")
+    with pytest.raises(cuda_lib.BridgesError) as err:
+        ctx.find(torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda(), V)
+    assert err.value.code == -2

@@ -23,6 +23,7 @@ using namespace bridges;
 namespace {
 
 constexpr size_t kMiscBytes = 1024;  // status word, device counts of bridges_from_forest, spare output
+constexpr int64_t kSmallCallEdges = 22528;  // a whole call on one block up to this many edges
 constexpr size_t kClearBytes = kMiscBytes + 256;  // cleared at a call's start: the misc area and the
                                                   // certificate's control words, which follow it
 constexpr size_t kSpareAt = 512;     // the spare output slot: where a call that has no pairs or points
@@ -184,28 +185,39 @@ int init_ctx(bridges_ctx* c, int device, const bridges_opts* opts) {
   return 0;
 }
 
-// The final stage of a call that wants only the sorted bridges and their count (none of the
-// rooted forest's arrays): a graph of 2..kBatchVmax vertices runs it on one block in shared
-// memory (small_final_launch: block barriers only, against the grid stage's 19 grid barriers),
-// a larger one on the grid.  The grid barrier's test knobs keep the grid form.
-void final_bridges(const Launch& L, const Carved& k, int32_t V, int32_t* out) {
-  if (V >= 2 && V <= kBatchVmax && L.bar_polls == 0 && L.hold_polls == 0) {
-    const SmallFinalArgs a{V, k.cert.P1, k.cert.f1u, k.cert.f1v, k.cert.cnt + 0, k.cert.f2u, k.cert.f2v,
-                           k.cert.cnt + 1, k.fin.status, k.fin.count, out};
+// What a call reads after the path: the certificate alone; the sorted bridges and their count; those and
+// which F edges they are (2-edge-connected components, incremental sets); the rooted forest's arrays
+// (articulation points).
+enum class Want { certificate, bridges, components, rooted };
+
+// The final stage of a call, pairs to out.  The bridges alone of a graph of 2..kBatchVmax vertices run on
+// one block in shared memory (small_final_launch), unless the grid barrier's test knobs are set; what
+// needs no rooted forest takes the reduced graph.
+void final_for(const Launch& L, const Carved& k, int32_t V, int32_t* out, Want want) {
+  if (want == Want::bridges && V >= 2 && V <= kBatchVmax && L.bar_polls == 0 && L.hold_polls == 0) {
+    const SmallFinalArgs a{V, k.cert.P2, k.cert.f1u, k.cert.f1v, k.cert.cnt + 0, k.fin.status, k.fin.count, out};
     small_final_launch(L.stream, a);  // a launch error is caught by the caller's error check
     *L.launches += 1;
-    return;
+  } else if (want == Want::bridges || want == Want::components) {
+    reduced_stage(L, k.fin, k.cert, V, out);
+  } else if (want == Want::rooted) {
+    // job 0 holds the final certificate: F (tree) and F' (extra); its UF1 roots the trees
+    final_stage(L, k.fin, V, k.cert.f1u, k.cert.f1v, k.cert.cnt + 0, V, k.cert.f2u, k.cert.f2v, k.cert.cnt + 1, V,
+                k.cert.P1, out);
   }
-  final_stage(L, k.fin, V, k.cert.f1u, k.cert.f1v, k.cert.cnt + 0, V, k.cert.f2u, k.cert.f2v, k.cert.cnt + 1, V,
-              k.cert.P1, out);
 }
 
-// The whole path on device-resident edges.  Leaves the count on the device (fin.count).  With
-// with_final false it stops after the certificate; otherwise the sorted pairs go to out, or to
-// the final stage's own dscan array (free by the time it sorts) when out is null.  With
-// bridges_only the caller reads nothing of the final stage but the pairs and the count.
+// Whether a call that wants only the bridges runs whole on one block (small_call_launch).
+bool small_call(const bridges_ctx* c, const CertPlan& p) {
+  return p.sampled && p.V >= 2 && p.V <= kBatchVmax && p.E <= kSmallCallEdges && c->opts.test_barrier_polls <= 0 &&
+         c->opts.test_hold_polls <= 0;
+}
+
+// The whole path on device-resident edges.  Leaves the count on the device (fin.count); the sorted
+// pairs go to out, or to the final stage's own dscan array (free by the time it sorts) when out is
+// null.
 int64_t run_path(bridges_ctx* c, cudaStream_t s, const int32_t* u, const int32_t* v, int64_t E, int32_t V, int32_t M,
-                 int32_t* out, Carved* kout, CertPlan* pout, bool with_final = true, bool bridges_only = false) {
+                 int32_t* out, Carved* kout, CertPlan* pout, Want want) {
   Range range("bridges: certificate + final stage");
   CertPlan p = plan_for(c, E, V, M);
   int64_t rc = ensure_ws(c, total_bytes(p), s);
@@ -219,6 +231,21 @@ int64_t run_path(bridges_ctx* c, cudaStream_t s, const int32_t* u, const int32_t
   c->last_cfg[4] = p.cache ? p.warm : -1;
   cudaEvent_t* ev = next_event_slot(c);
   if (ev) cudaEventRecord(ev[7], s);
+  if (want == Want::bridges && small_call(c, p)) {
+    if (ev)
+      for (int i = 0; i < 5; i++) cudaEventRecord(ev[i], s);
+    small_call_launch(s, u, v, E, V, k.fin.count, out ? out : k.fin.dscan);
+    c->launches += 1;
+    if (ev) {
+      cudaEventRecord(ev[5], s);
+      cudaEventRecord(ev[6], s);
+      c->calls++;
+    }
+    if (cudaGetLastError() != cudaSuccess) return BRIDGES_ECUDA;
+    if (kout) *kout = k;
+    if (pout) *pout = p;
+    return BRIDGES_OK;
+  }
   cudaMemsetAsync(k.status, 0, kClearBytes, s);
   cert_init(L, p, k.cert);
   cert_leaves(L, p, k.cert, u, v, ev);
@@ -226,14 +253,7 @@ int64_t run_path(bridges_ctx* c, cudaStream_t s, const int32_t* u, const int32_t
     for (int i = 0; i < 4; i++) cudaEventRecord(ev[i], s);
   cert_merge(L, p, k.cert);
   if (ev) cudaEventRecord(ev[4], s);
-  if (with_final) {
-    // job 0 holds the final certificate: F (tree) and F' (extra); its UF1 roots the trees
-    if (bridges_only)
-      final_bridges(L, k, V, out ? out : k.fin.dscan);
-    else
-      final_stage(L, k.fin, V, k.cert.f1u, k.cert.f1v, k.cert.cnt + 0, V, k.cert.f2u, k.cert.f2v, k.cert.cnt + 1,
-                  V, k.cert.P1, out ? out : k.fin.dscan);
-  }
+  final_for(L, k, V, out ? out : k.fin.dscan, want);
   if (ev) {
     cudaEventRecord(ev[5], s);
     cudaEventRecord(ev[6], s);
@@ -351,7 +371,7 @@ static int64_t issue_chunks(bridges_ctx* c, cudaStream_t s, const int32_t* hu, c
 }
 
 int64_t run_path_host(bridges_ctx* c, cudaStream_t s, const int32_t* hu, const int32_t* hv, int32_t* du, int32_t* dv,
-                      int64_t E, int32_t V, int32_t M, int32_t* out, Carved* kout, bool bridges_only) {
+                      int64_t E, int32_t V, int32_t M, int32_t* out, Carved* kout, Want want) {
   Range range("bridges: pipelined host input");
   CertPlan p = plan_for(c, E, V, M);
   if (p.M != 1 || !p.cache) return 1;
@@ -387,11 +407,7 @@ int64_t run_path_host(bridges_ctx* c, cudaStream_t s, const int32_t* hu, const i
   if (ev) cudaEventRecord(ev[3], s);
   cert_merge(L, p, k.cert);
   if (ev) cudaEventRecord(ev[4], s);
-  if (bridges_only)
-    final_bridges(L, k, V, out);
-  else
-    final_stage(L, k.fin, V, k.cert.f1u, k.cert.f1v, k.cert.cnt + 0, V, k.cert.f2u, k.cert.f2v, k.cert.cnt + 1, V,
-                k.cert.P1, out);
+  final_for(L, k, V, out, want);
   if (ev) {
     cudaEventRecord(ev[5], s);
     cudaEventRecord(ev[6], s);
@@ -476,7 +492,7 @@ int64_t bridges_find_ctx(bridges_ctx* c, struct CUstream_st* stream, const int32
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (cudaSetDevice(c->device) != cudaSuccess) return cuda_fail(cudaGetLastError());
   Carved k{};
-  rc = run_path(c, s, u, v, E, V, M, out, &k, nullptr, true, true);
+  rc = run_path(c, s, u, v, E, V, M, out, &k, nullptr, Want::bridges);
   if (rc) return rc;
   if (out_count_device) {
     if (cudaMemcpyAsync(out_count_device, k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
@@ -518,7 +534,7 @@ int64_t bridges_find_host(bridges_ctx* c, struct CUstream_st* stream, const int3
   Carved k{};
   rc = 1;
   if (deferred)  // copies not issued yet: overlap them with the forest pass if the plan allows
-    rc = run_path_host(c, s, hu, hv, const_cast<int32_t*>(ru), const_cast<int32_t*>(rv), E, V, M, dout, &k, true);
+    rc = run_path_host(c, s, hu, hv, const_cast<int32_t*>(ru), const_cast<int32_t*>(rv), E, V, M, dout, &k, Want::bridges);
   if (rc < 0) return rc;
   if (rc == 1) {
     if (deferred && E > 0 &&
@@ -527,7 +543,7 @@ int64_t bridges_find_host(bridges_ctx* c, struct CUstream_st* stream, const int3
          cudaMemcpyAsync(const_cast<int32_t*>(rv), hv, sizeof(int32_t) * (size_t)E, cudaMemcpyHostToDevice, s) !=
              cudaSuccess))
       return cuda_fail(cudaGetLastError());
-    rc = run_path(c, s, ru, rv, E, V, M, dout, &k, nullptr, true, true);
+    rc = run_path(c, s, ru, rv, E, V, M, dout, &k, nullptr, Want::bridges);
     if (rc) return rc;
   }
   if (cudaMemcpyAsync(c->h_pinned, k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)
@@ -552,7 +568,7 @@ int64_t bridges_certificate(bridges_ctx* c, struct CUstream_st* stream, const in
   if (cudaSetDevice(c->device) != cudaSuccess) return cuda_fail(cudaGetLastError());
   Carved k{};
   CertPlan p{};
-  rc = run_path(c, s, u, v, E, V, M, nullptr, &k, &p, false);
+  rc = run_path(c, s, u, v, E, V, M, nullptr, &k, &p, Want::certificate);
   if (rc) return rc;
   if (V > 1) cert_export(launch_for(c, s), p, k.cert, cu, cv, ct);
   // counts and status
@@ -906,7 +922,7 @@ int64_t default_split(const bridges_ctx* c, int64_t total_e) {
 int64_t run_single(bridges_ctx* c, cudaStream_t s, const int32_t* u, const int32_t* v, int64_t E, int32_t V, int32_t M,
                    int32_t* out, int64_t* count_dev) {
   Carved k{};
-  int64_t rc = run_path(c, s, u, v, E, V, M, out, &k, nullptr, true, true);
+  int64_t rc = run_path(c, s, u, v, E, V, M, out, &k, nullptr, Want::bridges);
   if (rc) return rc;
   if (cudaMemcpyAsync(count_dev, k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
     return cuda_fail(cudaGetLastError());
@@ -1161,13 +1177,13 @@ extern "C" int32_t bridges_autotune(bridges_ctx* c, struct CUstream_st* stream, 
           // one untimed run (workspace growth, first-touch), then reps timed runs
           int64_t r = BRIDGES_OK;
           Carved k{};
-          r = run_path(c, s, u, v, E, V, 0, out, &k, nullptr, true, true);
+          r = run_path(c, s, u, v, E, V, 0, out, &k, nullptr, Want::bridges);
           if (r) {
             rc = (int32_t)r;
             break;
           }
           cudaEventRecord(e0, s);
-          for (int i = 0; i < reps && !r; i++) r = run_path(c, s, u, v, E, V, 0, out, &k, nullptr, true, true);
+          for (int i = 0; i < reps && !r; i++) r = run_path(c, s, u, v, E, V, 0, out, &k, nullptr, Want::bridges);
           cudaEventRecord(e1, s);
           if (r || cudaEventSynchronize(e1) != cudaSuccess) {
             rc = r ? (int32_t)r : (int32_t)BRIDGES_ECUDA;
@@ -1195,9 +1211,9 @@ extern "C" int32_t bridges_autotune(bridges_ctx* c, struct CUstream_st* stream, 
     o.profile = 0;
     c->opts = o;
     Carved k{};
-    int64_t r = run_path(c, s, u, v, E, V, 0, out, &k, nullptr, true, true);
+    int64_t r = run_path(c, s, u, v, E, V, 0, out, &k, nullptr, Want::bridges);
     cudaEventRecord(e0, s);
-    for (int i = 0; i < reps && !r; i++) r = run_path(c, s, u, v, E, V, 0, out, &k, nullptr, true, true);
+    for (int i = 0; i < reps && !r; i++) r = run_path(c, s, u, v, E, V, 0, out, &k, nullptr, Want::bridges);
     cudaEventRecord(e1, s);
     if (r || cudaEventSynchronize(e1) != cudaSuccess) {
       rc = r ? (int32_t)r : (int32_t)BRIDGES_ECUDA;
@@ -1280,10 +1296,10 @@ extern "C" int64_t bridges_two_edge_components(bridges_ctx* c, struct CUstream_s
   // the bridges go to the caller's buffer or to the (then unused) workspace key area
   Carved k{};
   CertPlan p{};
-  rc = run_path(c, s, u, v, E, V, M, out_bridges, &k, &p);
+  rc = run_path(c, s, u, v, E, V, M, out_bridges, &k, &p, Want::components);
   if (rc) return rc;
   Launch L = launch_for(c, s);
-  two_edge_components(L, k.fin, V, k.cert.f2u, k.cert.f2v, k.cert.cnt + 1, V, labels, k.fin.count);
+  two_edge_components(L, k.fin, k.cert, V, labels, k.fin.count);
   if (cudaMemcpyAsync(c->h_pinned, k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return cuda_fail(cudaGetLastError());
@@ -1427,7 +1443,7 @@ static int64_t articulation_run(bridges_ctx* c, cudaStream_t s, const int32_t* u
     // free by the time the final stage sorts
     const Carved k0 = carve(c, p0);
     rc = run_path_host(c, s, hu, hv, const_cast<int32_t*>(u), const_cast<int32_t*>(v), E, V, M,
-                       out_bridges ? out_bridges : k0.fin.dscan, &k, false);
+                       out_bridges ? out_bridges : k0.fin.dscan, &k, Want::rooted);
     if (rc < 0) return rc;
     if (rc == 1 && E > 0 &&
         (cudaMemcpyAsync(const_cast<int32_t*>(u), hu, sizeof(int32_t) * (size_t)E, cudaMemcpyHostToDevice, s) !=
@@ -1437,7 +1453,7 @@ static int64_t articulation_run(bridges_ctx* c, cudaStream_t s, const int32_t* u
       return cuda_fail(cudaGetLastError());
   }
   if (rc == 1) {
-    rc = run_path(c, s, u, v, E, V, M, out_bridges, &k, nullptr);
+    rc = run_path(c, s, u, v, E, V, M, out_bridges, &k, nullptr, Want::rooted);
     if (rc) return rc;
   }
   if (!out_points) out_points = k.spare;  // V <= 1: no point is written
@@ -1572,7 +1588,7 @@ extern "C" int64_t bridges_inc_reset(bridges_inc* I, struct CUstream_st* stream,
   if (V > (1 << 30)) return BRIDGES_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (cudaSetDevice(I->ctx->device) != cudaSuccess) return cuda_fail(cudaGetLastError());
-  rc = run_path(I->ctx, s, u, v, E, V, M, out_bridges, &I->k, &I->p);
+  rc = run_path(I->ctx, s, u, v, E, V, M, out_bridges, &I->k, &I->p, Want::components);
   if (rc) return rc;
   if (cudaMemcpyAsync(I->ctx->h_pinned, I->k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
@@ -1594,8 +1610,7 @@ extern "C" int64_t bridges_inc_add(bridges_inc* I, struct CUstream_st* stream, c
   const int32_t V = I->V;
   if (cudaMemsetAsync(k.status, 0, sizeof(int32_t), s) != cudaSuccess) return cuda_fail(cudaGetLastError());
   cert_offer(L, I->p, k.cert, yu, yv, n);
-  final_stage(L, k.fin, V, k.cert.f1u, k.cert.f1v, k.cert.cnt + 0, V, k.cert.f2u, k.cert.f2v, k.cert.cnt + 1, V,
-              k.cert.P1, out_bridges ? out_bridges : k.spare);
+  reduced_stage(L, k.fin, k.cert, V, out_bridges ? out_bridges : k.spare);
   if (cudaMemcpyAsync(c->h_pinned, k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return cuda_fail(cudaGetLastError());
@@ -1609,7 +1624,7 @@ extern "C" int64_t bridges_inc_two_edge_components(bridges_inc* I, struct CUstre
   if (cudaSetDevice(c->device) != cudaSuccess) return cuda_fail(cudaGetLastError());
   Launch L = launch_for(c, s);
   const Carved& k = I->k;
-  two_edge_components(L, k.fin, I->V, k.cert.f2u, k.cert.f2v, k.cert.cnt + 1, I->V, labels, k.fin.count);
+  two_edge_components(L, k.fin, k.cert, I->V, labels, k.fin.count);
   if (cudaMemcpyAsync(c->h_pinned, k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return cuda_fail(cudaGetLastError());

@@ -4,6 +4,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "internal.h"
+
 namespace bridges {
 
 constexpr int kBatchVmax = 4096;  // graphs up to this many vertices are handled in shared memory
@@ -60,29 +62,57 @@ inline int batch_min_class(int32_t V, int32_t nparts) {
 // smallest it fits; never a smaller one).
 inline int batch_task_class(const BatchTask& t) { return t.cls; }
 
-// Words of a task's certificate slot: [nF, nF', F (V words), F' (V words), the root of each
-// vertex's F tree (V u16, padded to a word), the root of each vertex's F' tree (likewise)]; the
-// roots are written by a graph's first task (the F' roots only when more tasks follow).  A
-// graph's slots are consecutive.
+// Words of a task's certificate slot: [nF, nF', F (V words), F' (V words), the root of each vertex's
+// F' tree (V u16, padded to a word), the root of each vertex's F tree (likewise)]; the roots are
+// written by a graph's first task (the F roots only when more tasks follow).  A graph's slots are
+// consecutive.
 __host__ __device__ inline int64_t batch_slot_words(int32_t V) { return 2 + 2 * (int64_t)V + 2 * (((int64_t)V + 1) / 2); }
 
 // One graph's final stage on one block (small_final_launch): the final certificate as the forest
 // pass and the merge tree leave it in global memory, for a graph of 2..kBatchVmax vertices.
 struct SmallFinalArgs {
   int32_t V;
-  const int32_t* P;     // F's union-find (P[x] <= x; a root is its set's minimum vertex)
+  const int32_t* P2;    // the union-find of F' (P2[x] <= x)
   const int32_t* tu;    // F: tree edges, *d_nt of them
   const int32_t* tv;
   const int32_t* d_nt;
-  const int32_t* xu;    // F': the other certificate edges, *d_nx of them
-  const int32_t* xv;
-  const int32_t* d_nx;
   const int32_t* status;  // the call's status word (0, or the first error of an earlier stage)
   int64_t* count;       // receives the bridge count, or the status when it is set
   int32_t* out;         // receives the sorted (a, b) pairs, capacity 2 (V - 1)
 };
 
+// The sampled certificate on one block (block_certify_launch): edges [0, n) of the list, `groups`
+// groups of 2^kSampleShift edges, every stride-th one.
+struct BlockCertArgs {
+  const int32_t* u;
+  const int32_t* v;
+  int64_t n;
+  int64_t stride;
+  int32_t groups;
+  int32_t V;
+  int32_t snap;  // whether the labels are wanted (V < kNoLabel then)
+  CertBufs b;
+};
+
+// A whole call on one block (small_call_launch).
+struct SmallCallArgs {
+  const int32_t* u;
+  const int32_t* v;
+  int64_t E;
+  int64_t stride;  // the sample: every stride-th group (1: the whole list)
+  int32_t groups;
+  int32_t V;
+  int64_t* count;  // receives the bridge count, or a negative status
+  int32_t* out;    // receives the sorted (a, b) pairs, capacity 2 (V - 1)
+};
+
 size_t batched_smem_bytes();
+// Launches the sampled certificate on one block (V <= kBatchVmax, at most kBlockCertSlots edges).
+constexpr int64_t kBlockCertSlots = 8 * kBatchVmax + 4096;
+bool block_certify_launch(cudaStream_t s, const BlockCertArgs& a);
+// Launches a whole call (2 <= V <= kBatchVmax, bridges and count only) on one block.
+bool small_call_launch(cudaStream_t s, const int32_t* u, const int32_t* v, int64_t E, int32_t V, int64_t* count,
+                       int32_t* out);
 // Launches the one-block final stage (bridges and count only) on stream s.
 bool small_final_launch(cudaStream_t s, const SmallFinalArgs& a);
 // Launches the two persistent kernels (one block per SM each: certification, then the bridge

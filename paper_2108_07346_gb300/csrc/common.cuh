@@ -74,6 +74,17 @@ __device__ __forceinline__ int32_t uf_find_static(int32_t* P, int32_t x) {
   return x;
 }
 
+// Root of x, under the same condition, without a write: for passes that leave every entry at its root
+// (a halving store may put an ancestor back over a root that another thread has just written).
+__device__ __forceinline__ int32_t uf_root_static(const int32_t* P, int32_t x) {
+  int32_t p = __ldca(P + x);
+  while (p != x) {
+    x = p;
+    p = __ldca(P + x);
+  }
+  return x;
+}
+
 // Joins the sets of a and b.  Returns true iff they were different (the edge is a forest edge).
 //
 // Walks up from both ends comparing PARENTS, not roots: equal parents prove a common set, so in

@@ -36,6 +36,7 @@
 #include <algorithm>
 
 #include "grid.cuh"
+#include "smem.cuh"
 
 namespace bridges {
 
@@ -69,7 +70,11 @@ struct FinArgs {
   const int32_t* d_nx;
   int32_t cx;             // capacity of the extra list
   const int32_t* P_tree;  // union-find of T, or null: built here in f.P
+  const int32_t* orig;    // reduced graph: the place of each tree edge's original in (ou, ov) (null: its own)
+  const int32_t* ou;
+  const int32_t* ov;
   int32_t* out;
+  int32_t key_cap;  // bridges that the key array holds (the graph's vertices)
   int kbits;
   int32_t sup_log;  // chunks per superchunk = kSuperChunks << sup_log
   int32_t ordered;  // trees in increasing order of their roots
@@ -81,9 +86,10 @@ __device__ __forceinline__ bool grid_barrier(const FinalBufs& f, unsigned polls,
   return bridges::grid_barrier(f.bar_count, f.status, f.count, polls, epoch);
 }
 
-#define BARRIER()                                         \
-  do {                                                    \
-    if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return; \
+// in a device function that returns whether the kernel may go on
+#define BARRIER()                                               \
+  do {                                                          \
+    if (!grid_barrier(f, A.bar_polls, bar_epoch)) return false; \
   } while (0)
 
 // Block-wide sum (every thread gets the result).
@@ -287,13 +293,26 @@ __device__ __forceinline__ int32_t lower_rank(const uint64_t* s, int32_t n, uint
   return lo;
 }
 
-__global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
-  extern __shared__ __align__(16) int32_t sm[];  // superchunk sparse tables, then sort staging
-  __shared__ int32_t red[kWarps];
-  __shared__ uint32_t wcnt[kWarps][256];
-  __shared__ uint32_t run[256];
-  __shared__ unsigned bar_epoch;  // grid barriers passed (thread 0's count)
-  if (threadIdx.x == 0) bar_epoch = 0;
+// A bridge's sort key: its smaller end above its larger one.
+__device__ __forceinline__ uint64_t key_of(int32_t a, int32_t b, int kbits) {
+  return (uint64_t)(uint32_t)min(a, b) << kbits | (uint32_t)max(a, b);
+}
+
+// The reduced stage lists a bridge by its slot among the kept edges until the sort, when every block
+// reads its share of the edges' ends.
+constexpr uint64_t kSlotTag = 1ull << 63;
+
+__device__ __forceinline__ uint64_t resolved(const FinArgs& A, const int32_t* ko, uint64_t key) {
+  if (!(key & kSlotTag)) return key;
+  const int32_t o = ko[(uint32_t)key];
+  A.f.bflag[o] = 1;
+  return key_of(A.tu[o], A.tv[o], A.kbits);
+}
+
+// Phases 0 to 7: the bridges of T u X appended to f.keys.  RED: the graph is a reduced one (below),
+// whose tree edges stand for edges of the caller's.
+template <bool RED>
+__device__ bool forest_bridges(const FinArgs& A, int32_t* sm, int32_t* red, unsigned* bar_epoch) {
   const FinalBufs& f = A.f;
   const int32_t V = A.V;
   const bool own = A.P_tree == nullptr;
@@ -302,18 +321,6 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
   const int32_t nx = min(*A.d_nx, A.cx);
   const int64_t na = 2 * (int64_t)nt;  // tree arcs
   const int64_t nchunks = (V + kChunk - 1) / kChunk;
-
-  // an earlier stage failed: its lists and union-finds may be unset (nothing sets the status between
-  // a block's start here and the first barrier, so every block sees the same)
-  if (ld_relaxed(f.status) != 0) {
-    if (gtid() == 0) *f.count = (int64_t)ld_relaxed(f.status);
-    return;
-  }
-
-  // a test knob: hold the last block back (a bounded sleep) so that the others' first barrier
-  // gives up; never set in normal use
-  if (A.hold_polls > 0 && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0)
-    for (int32_t i = 0; i < A.hold_polls; i++) __nanosleep(100);
 
   // 0: clear
   for (int64_t x = gspread(); x < V; x += gstride()) {
@@ -328,10 +335,7 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
     f.cmin[c] = INT32_MAX;
     f.cmax[c] = INT32_MIN;
   }
-  if (gtid() == 0) {
-    *f.nkeys = 0;
-    *f.nroots = 0;
-  }
+  if (gtid() == 0) *f.nroots = 0;
   BARRIER();
 
   // 1: arc lists (and the forest's union-find when it is ours to build); with a given
@@ -381,7 +385,7 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
   }
   BARRIER();
   if (A.ordered) {
-    if (!grid_scan(f, A.bar_polls, &bar_epoch, f.sz, f.rslot, nullptr, nullptr, V, red)) return;
+    if (!grid_scan(f, A.bar_polls, bar_epoch, f.sz, f.rslot, nullptr, nullptr, V, red)) return false;
     BARRIER();
     for (int64_t x = gspread(); x < V; x += gstride()) {
       if (f.root[x] == x)
@@ -399,7 +403,7 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
       const int32_t first = atomicCAS(f.status, 0, BRIDGES_EINTERNAL_CODE);
       *f.count = (int64_t)(first != 0 ? first : BRIDGES_EINTERNAL_CODE);
     }
-    return;  // every block leaves here
+    return false;  // every block leaves here
   }
 
   // 2: successors.  Arc i = (x -> y): the arc after its twin in y's list; at the end of y's list
@@ -500,6 +504,7 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
       f.dflag[g] = down ? 1 : 0;
       if (down) {
         f.par[y] = x;
+        if (RED) f.root[y] = (int32_t)(i >> 1);  // y's tree edge (root is free by now)
         f.slo[y] = (int32_t)g;  // tour position of y's down arc (slo serves as scratch until the test)
         f.sz[y] = (ri - rt + 1) / 2;
       }
@@ -518,7 +523,7 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
     }
   }
   BARRIER();
-  if (!grid_scan(f, A.bar_polls, &bar_epoch, f.dflag, f.dscan, nullptr, nullptr, N, red)) return;
+  if (!grid_scan(f, A.bar_polls, bar_epoch, f.dflag, f.dscan, nullptr, nullptr, N, red)) return false;
   BARRIER();
 
   // 5: preorder numbers (the down arcs and entries before the vertex's own tour position), and in
@@ -725,7 +730,7 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
     const int64_t y = base + (threadIdx.x & 31);
     bool is_bridge = false;
     uint64_t key = 0;
-    if (y < V) f.bflag[y] = 0;
+    if (!RED && y < V) f.bflag[y] = 0;
     if (y < V && f.par[y] >= 0) {
       const int64_t l = f.pre[y];
       const int64_t r = min((int64_t)V, l + max(f.sz[y], 1));
@@ -734,10 +739,17 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
       f.slo[y] = min(mn, (int32_t)l);
       f.shi[y] = max(mx, (int32_t)(r - 1));
       if (mn >= l && mx < r) {
-        const uint32_t a = (uint32_t)min((int32_t)y, f.par[y]), b = (uint32_t)max((int32_t)y, f.par[y]);
-        key = ((uint64_t)a << A.kbits) | b;
+        int32_t a = (int32_t)y, b = f.par[y];
+        if (RED) {
+          const int32_t o = A.orig ? A.orig[f.root[y]] : f.root[y];
+          a = A.ou[o];
+          b = A.ov[o];
+          f.bflag[o] = 1;
+        } else {
+          f.bflag[y] = 1;
+        }
+        key = key_of(a, b, A.kbits);
         is_bridge = true;
-        f.bflag[y] = 1;
       }
     }
     const unsigned m = __ballot_sync(kFull, is_bridge);
@@ -748,18 +760,24 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
       at = __shfl_sync(kFull, at, leader);
       if (is_bridge) {
         const int32_t i = at + __popc(m & lanemask_lt());
-        if (i < V)
+        if (i < A.key_cap)
           f.keys[i] = key;
         else
           set_status(f.status, BRIDGES_EINTERNAL_CODE);
       }
     }
   }
-  BARRIER();
+  return true;
+}
 
-  // 8: sort the keys; write (a, b) pairs
-  const int32_t cap = max(V - 1, 0);
-  const int32_t n = min(*f.nkeys, cap);
+// Phase 8, after a barrier: sorts the keys and writes the pairs.  ko: the kept edges' places in F, for keys
+// still listed by slot (at most kRankMax of them); listed >= 0: the keys are the slots [0, listed) and not
+// in f.keys (with ko null, they are there by value).
+__device__ bool sort_keys(const FinArgs& A, const int32_t* ko, int32_t listed, int32_t* sm, int32_t* red,
+                          unsigned* bar_epoch) {
+  const FinalBufs& f = A.f;
+  const int32_t cap = max(A.key_cap - 1, 0);
+  const int32_t n = min(listed >= 0 ? listed : *f.nkeys, cap);
   const uint64_t mask = (1ULL << A.kbits) - 1;
   const int64_t per = (n + gridDim.x - 1) / gridDim.x;
   if (n <= kRankMax) {
@@ -773,7 +791,7 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
     const int32_t ps = nsl > 0 ? (n32 + nsl - 1) / nsl : 0;  // slice length
     for (int32_t b = blockIdx.x; b < nsl; b += gridDim.x) {  // small grids take several slices
       const int32_t s0 = ps * b, m = min(n32, s0 + ps) - s0;
-      for (int i = threadIdx.x; i < m; i += blockDim.x) S[i] = f.keys[s0 + i];
+      for (int i = threadIdx.x; i < m; i += blockDim.x) S[i] = resolved(A, ko, listed >= 0 && ko ? kSlotTag | (uint64_t)(s0 + i) : f.keys[s0 + i]);
       __syncthreads();
       for (int q = threadIdx.x; q < m; q += blockDim.x) {
         const uint64_t key = S[q];
@@ -806,6 +824,8 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
       }
     }
   } else {
+    uint32_t(*const wcnt)[256] = reinterpret_cast<uint32_t(*)[256]>(sm);  // [kWarps][256]
+    uint32_t* const run = reinterpret_cast<uint32_t*>(sm) + kWarps * 256;   // [256]
     const int passes = (2 * A.kbits + 7) / 8;
     const int64_t lo = min((int64_t)n, per * (int64_t)blockIdx.x), hi = min((int64_t)n, lo + per);
     uint64_t* src = f.keys;
@@ -819,7 +839,7 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
       __syncthreads();
       if (threadIdx.x < 256) f.hist[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = (int32_t)run[threadIdx.x];
       BARRIER();
-      if (!grid_scan(f, A.bar_polls, &bar_epoch, f.hist, f.hist, nullptr, nullptr, (int64_t)256 * gridDim.x, red)) return;
+      if (!grid_scan(f, A.bar_polls, bar_epoch, f.hist, f.hist, nullptr, nullptr, (int64_t)256 * gridDim.x, red)) return false;
       BARRIER();
       if (threadIdx.x < 256) {
         run[threadIdx.x] = (uint32_t)f.hist[(int64_t)threadIdx.x * gridDim.x + blockIdx.x];
@@ -867,17 +887,428 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
       dst = t;
     }
   }
+  return true;
+}
 
-  // 9: the count, or the first error
+// The count, or the first error.
+__device__ __forceinline__ void write_count(const FinArgs& A) {
+  const FinalBufs& f = A.f;
   if (gtid() == 0) {
     int32_t st = *f.status;
     const int32_t nk = *f.nkeys;
-    if (st == 0 && nk > cap) st = BRIDGES_EINTERNAL_CODE;  // a forest has at most V-1 edges
+    if (st == 0 && nk > max(A.key_cap - 1, 0)) st = BRIDGES_EINTERNAL_CODE;  // a forest has at most V-1 edges
     *f.count = st != 0 ? (int64_t)st : (int64_t)nk;
   }
 }
 
+// The first block's checks of a final stage: an earlier stage's error ends it (its lists and union-finds
+// may be unset; nothing sets the status between a block's start here and the first barrier, so every
+// block sees the same).
+__device__ __forceinline__ bool may_start(const FinArgs& A) {
+  const int32_t st = ld_relaxed(A.f.status);
+  if (st != 0) {
+    if (gtid() == 0) *A.f.count = (int64_t)st;
+    return false;
+  }
+  // a test knob: hold the last block back (a bounded sleep) so that the others' first barrier
+  // gives up; never set in normal use
+  if (A.hold_polls > 0 && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0)
+    for (int32_t i = 0; i < A.hold_polls; i++) __nanosleep(100);
+  return true;
+}
+
+__global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
+  extern __shared__ __align__(16) int32_t sm[];  // superchunk sparse tables, then sort staging
+  __shared__ int32_t red[kWarps];
+  __shared__ unsigned bar_epoch;  // grid barriers passed (thread 0's count)
+  if (threadIdx.x == 0) bar_epoch = 0;
+  if (!may_start(A)) return;
+  if (gtid() == 0) *A.f.nkeys = 0;
+  if (!forest_bridges<false>(A, sm, red, &bar_epoch)) return;
+  if (!grid_barrier(A.f, A.bar_polls, &bar_epoch)) return;
+  if (!sort_keys(A, nullptr, -1, sm, red, &bar_epoch)) return;
+  write_count(A);
+}
+
+// ---- the bridges alone: on the reduced graph ----
+//
+// Two ends of an F' edge are joined by F as well, so the edge lies on a cycle, and each F' component in
+// one 2-edge-connected component: contracting the F' components changes no bridge, and the edges that are
+// left all come from F (s_contract, smem.cuh, does the same for small graphs).  Dense graphs keep only
+// their sparse fringe: 4,443 vertices of 37,147, 8.3 k of 73,719.
+//   1  P2 flattened: every vertex's F' root.
+//   2  F edges between two roots are kept; the roots are numbered as they are met, and the trees of F that
+//      kept edges lie in counted.  If the kept edges number the roots less the trees, the reduced graph is
+//      a forest and all of them are bridges.  If they are many more than the roots (a sparse graph with
+//      cycles throughout), the reduction gained little and the phases above run on F and F' as they are.
+//   3  Else leaves are stripped.  The one edge of a vertex of degree 1 is a bridge; without it its other
+//      end may be the next leaf, and the thread goes on there (at most kStripSteps times, so that a long
+//      path does not run in one thread; vertices of kHub edges and more keep their degree, so that their
+//      leaves do not queue on them).
+//   4  What is left, the cycles and what joins them, is solved by block 0 in shared memory when it has at
+//      most kCoreMax vertices, else by every block: a spanning forest of it, then the phases above.
+//   5  The keys are sorted, as above.
+// 2.5 M edges on 37,147 vertices: 79 us with the phases above on the whole forest, 27 us so; 16.8 M
+// R-MAT edges on 2^20 vertices (141 k kept edges, 140.1 k of them bridges): 417 and 177 us.
+
+struct ReducedArgs {
+  FinArgs a;          // a.V: the graph's vertices; tu, tv, d_nt: F; kbits, sup_log, bar_polls, hold_polls
+  int32_t* P1;        // union-find of F
+  int32_t* P2;        // union-find of F'
+  const int32_t* xu;  // F'
+  const int32_t* xv;
+  const int32_t* d_nx;
+  int32_t* tmp;       // [V] scratch
+};
+
+// counters behind f.nroots (one page)
+constexpr int kCntVerts = 1;  // reduced vertices
+constexpr int kCntKept = 2;   // kept edges
+constexpr int kCntTrees = 3;  // trees of F with kept edges
+constexpr int kCoreVerts = 4;
+constexpr int kCoreEdges = 5;
+constexpr int kCntTree = 6;
+constexpr int kCntRest = 7;
+constexpr int32_t kCyclicMin = 4096;  // kept edges above which a graph with many cycles is not reduced
+constexpr int kStripSteps = 8;
+constexpr int32_t kHub = 64;
+constexpr int32_t kCoreMax = 5632;  // the largest layout that fits a block's shared memory
+using CoreLayout = Layout<kCoreMax>;
+static_assert(kCoreMax % 32 == 0 && CoreLayout::kBytes + 3072 <= 227 * 1024, "the core's layout fits a block");
+
+// Appends one item per lane that has one; the place of each, counted in *n per warp.
+__device__ __forceinline__ int32_t warp_place(bool has, int32_t* n) {
+  const unsigned m = __ballot_sync(kFull, has);
+  if (!m) return 0;
+  const int lane = threadIdx.x & 31;
+  int32_t at = 0;
+  if (lane == __ffs(m) - 1) at = atomicAdd(n, __popc(m));
+  return __shfl_sync(kFull, at, __ffs(m) - 1) + __popc(m & lanemask_lt());
+}
+
+// Numbers the entries r[k] of number[k] (all -1 before) as they are met, counted in *n[k]: the first lane
+// that brings an entry numbers it.  Lanes of a warp with one entry send one of them, so that an entry that
+// every edge shares is not read by each; the N entries' accesses run side by side.
+template <int N>
+__device__ __forceinline__ void number_once(bool has, const int32_t (&r)[N], int32_t* const (&number)[N],
+                                            int32_t* const (&n)[N]) {
+  const int lane = threadIdx.x & 31;
+  bool mine[N];
+  int32_t at[N];
+  unsigned m[N];
+#pragma unroll
+  for (int k = 0; k < N; k++) {
+    const unsigned peers = __match_any_sync(kFull, has ? r[k] : -1 - lane);
+    mine[k] = has && lane == __ffs(peers) - 1;
+    at[k] = mine[k] ? __ldca(number[k] + r[k]) : 0;
+  }
+#pragma unroll
+  for (int k = 0; k < N; k++) {
+    mine[k] = mine[k] && at[k] == -1;
+    at[k] = mine[k] ? atomicCAS(number[k] + r[k], -1, -2) : 0;
+  }
+#pragma unroll
+  for (int k = 0; k < N; k++) {
+    mine[k] = mine[k] && at[k] == -1;
+    m[k] = __ballot_sync(kFull, mine[k]);
+    at[k] = m[k] && lane == __ffs(m[k]) - 1 ? atomicAdd(n[k], __popc(m[k])) : 0;
+  }
+#pragma unroll
+  for (int k = 0; k < N; k++) {
+    if (!m[k]) continue;
+    at[k] = __shfl_sync(kFull, at[k], __ffs(m[k]) - 1) + __popc(m[k] & lanemask_lt());
+    if (mine[k]) number[k][r[k]] = at[k];
+  }
+}
+
+// Adds edge `slot` to its end x's degree and to the xor of x's edges (lanes with one end together).
+__device__ __forceinline__ void add_edge_end(bool has, int32_t x, int32_t slot, int32_t* deg, int32_t* inc) {
+  const int lane = threadIdx.x & 31;
+  const unsigned peers = __match_any_sync(kFull, has ? x : -1 - lane);
+  if (!has) return;
+  const uint32_t all = __reduce_xor_sync(peers, (uint32_t)slot);
+  if (lane == __ffs(peers) - 1) {
+    atomicAdd(deg + x, __popc(peers));
+    atomicXor(reinterpret_cast<uint32_t*>(inc + x), all);
+  }
+}
+
+// Step 4 by block 0: the core's edges i < mc, between id2[cu[cs[i]]] and id2[cv[cs[i]]], VC <= kCoreMax
+// vertices.  Its bridges are appended to f.keys as slots.
+__device__ void solve_core(const ReducedArgs& R, char* smem, GroupShared& gs, const int32_t* id2, const int32_t* cu,
+                           const int32_t* cv, const int32_t* cs, int32_t VC, int32_t mc) {
+  const FinArgs& A = R.a;
+  const int tid = threadIdx.x;
+  const Smem S = carve_smem<kCoreMax>(smem);
+  for (int x = tid; x < VC; x += kThreads) {
+    S.P1[x] = x;
+    S.P2[x] = x;
+  }
+  if (tid == 0) gs.n1 = 0;
+  __syncthreads();
+  // a spanning forest (its edges' slots in R.tmp) and the components of the other edges: the core is
+  // reduced by them once more, as the graph was by those of F'
+  constexpr int kAhead = 4;
+  const int base0 = tid & ~31;
+  for (int base = base0; base < mc; base += kAhead * kThreads) {
+    int32_t slot[kAhead], a[kAhead], b[kAhead];
+#pragma unroll
+    for (int k = 0; k < kAhead; k++) {
+      const int i = base + k * kThreads + (tid & 31);
+      slot[k] = i < mc ? __ldcg(cs + i) : -1;
+    }
+#pragma unroll
+    for (int k = 0; k < kAhead; k++) {
+      a[k] = slot[k] >= 0 ? __ldcg(cu + slot[k]) : 0;
+      b[k] = slot[k] >= 0 ? __ldcg(cv + slot[k]) : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kAhead; k++) {
+      a[k] = slot[k] >= 0 ? __ldcg(id2 + a[k]) : 0;
+      b[k] = slot[k] >= 0 ? __ldcg(id2 + b[k]) : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kAhead; k++) {
+      const bool live = slot[k] >= 0;
+      const bool tree = live && s_link(S.P1, a[k], b[k]);
+      const int32_t at = warp_place(tree, &gs.n1);
+      if (tree) {
+        S.F1[at] = (uint32_t)a[k] | ((uint32_t)b[k] << 16);
+        R.tmp[at] = slot[k];
+      } else if (live) {
+        s_link(S.P2, a[k], b[k]);
+      }
+    }
+  }
+  const Grp<kThreads> G{tid, 0};
+  s_flatten(G, S.P2, VC);
+  const int32_t* slots = R.tmp;
+  int32_t nt2, nx2, n = 0;
+  const int32_t VH = s_contract<kThreads, kCoreMax>(G, S, VC, gs.n1, gs, &nt2, &nx2,
+                                                    [&](int32_t e) { return (uint32_t)slots[e]; });
+  if (VH > 0)
+    n = s_bridges<kThreads, kCoreMax>(G, S, VH, nt2, nx2, gs.red, gs.red_b, &gs.sh, [&](int32_t e) { return S.F2[e]; });
+  const int32_t found = *A.f.nkeys;
+  __syncthreads();
+  for (int i = tid; i < n; i += kThreads)
+    if (found + i < A.key_cap) A.f.keys[found + i] = kSlotTag | orig_of<kCoreMax>(S, (int32_t)S.keys[i]);
+  if (tid == 0) *A.f.nkeys = found + n;
+}
+
+__global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
+  extern __shared__ __align__(16) int32_t sm[];
+  __shared__ int32_t red[kWarps];
+  __shared__ GroupShared gs;
+  __shared__ unsigned bar_epoch;
+  if (threadIdx.x == 0) bar_epoch = 0;
+  const FinArgs& A = R.a;
+  const FinalBufs& f = A.f;
+  const int32_t V = A.V;
+  const int lane = threadIdx.x & 31;
+  if (!may_start(A)) return;
+  int32_t* const id = f.pre;    // a root's number
+  int32_t* const tree = f.head; // a tree's (its root's in F)
+  int32_t* const deg = f.sz;    // by number
+  int32_t* const inc = f.slo;
+  int32_t* const id2 = f.hi;    // a core vertex's number
+  int32_t* const gone = f.shi;  // by kept edge: stripped
+  int32_t* const ku = reinterpret_cast<int32_t*>(f.sr);
+  int32_t* const kv = ku + V;
+  int32_t* const ko = kv + V;  // the kept edges' places in F
+  int32_t* const cu = reinterpret_cast<int32_t*>(f.sr2);
+  int32_t* const cv = cu + V;
+  int32_t* const cs = cv + V;
+  // 1: flat F' roots
+  for (int64_t x = gspread(); x < V; x += gstride()) {
+    R.P2[x] = uf_root_static(R.P2, (int32_t)x);
+    id[x] = -1;
+    tree[x] = -1;
+    id2[x] = -1;
+    deg[x] = 0;
+    inc[x] = 0;
+    gone[x] = 0;
+    f.P[x] = (int32_t)x;
+    f.bflag[x] = 0;
+  }
+  if (gtid() < 8) f.nroots[gtid()] = 0;
+  if (gtid() == 8) *f.nkeys = 0;
+  if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
+  // 2: kept edges.  With more F edges than two per thread they are listed first and numbered after a
+  // barrier, one per thread: the numbering is a chain of accesses, and a thread's edges would queue.
+  const int32_t nt = min(*A.d_nt, A.ct);
+  const bool list_first = nt > 2 * gstride();
+  auto number = [&](bool has, int32_t ra, int32_t rb, int32_t t) {
+    number_once<3>(has, {ra, rb, t}, {id, id, tree}, {f.nroots + kCntVerts, f.nroots + kCntVerts, f.nroots + kCntTrees});
+  };
+  for (int64_t base = gspread() & ~31LL; base < nt; base += gstride()) {
+    const int64_t e = base + lane;
+    int32_t ra = -1, rb = -1, t = -1;
+    if (e < nt) {
+      const int32_t a = A.tu[e], b = A.tv[e];
+      if ((uint32_t)a >= (uint32_t)V || (uint32_t)b >= (uint32_t)V) {
+        set_status(f.status, BRIDGES_EINTERNAL_CODE);
+      } else {
+        ra = R.P2[a];
+        rb = R.P2[b];
+        if (ra != rb && !list_first) t = uf_root_static(R.P1, a);
+      }
+    }
+    const bool keep = ra != rb;
+    if (!__any_sync(kFull, keep)) continue;
+    const int32_t at = warp_place(keep, f.nroots + kCntKept);
+    if (keep) {
+      ku[at] = ra;
+      kv[at] = rb;
+      ko[at] = (int32_t)e;
+    }
+    if (!list_first) number(keep, ra, rb, t);
+  }
+  if (list_first) {
+    if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
+    const int32_t m = f.nroots[kCntKept];
+    for (int64_t base = gspread() & ~31LL; base < m; base += gstride()) {
+      const int64_t i = base + lane;
+      const bool in = i < m;
+      number(in, in ? ku[i] : 0, in ? kv[i] : 0, in ? uf_root_static(R.P1, A.tu[ko[i]]) : 0);
+    }
+  }
+  if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
+  const int32_t kept = f.nroots[kCntKept], verts = f.nroots[kCntVerts];
+  if (kept == verts - f.nroots[kCntTrees]) {
+    // a forest: every kept edge is a bridge, listed by its place
+    if (kept <= kRankMax) {
+      if (!sort_keys(A, ko, kept, sm, red, &bar_epoch)) return;
+    } else {
+      for (int64_t i = gspread(); i < kept; i += gstride()) f.keys[i] = resolved(A, ko, kSlotTag | (uint64_t)i);
+      if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
+      if (!sort_keys(A, nullptr, kept, sm, red, &bar_epoch)) return;
+    }
+    if (gtid() == 0) *f.nkeys = kept;  // (read by this thread alone, below)
+    write_count(A);
+    return;
+  }
+  if (kept > kCyclicMin && kept > verts + verts / 4) {
+    FinArgs B = A;
+    B.orig = nullptr;
+    B.ou = A.tu;
+    B.ov = A.tv;
+    B.xu = R.xu;
+    B.xv = R.xv;
+    B.d_nx = R.d_nx;
+    B.cx = V;
+    B.P_tree = R.P1;
+    if (!forest_bridges<true>(B, sm, red, &bar_epoch)) return;
+    if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
+    if (!sort_keys(A, nullptr, -1, sm, red, &bar_epoch)) return;
+    write_count(A);
+    return;
+  }
+  // 3: degrees, then the strip
+  for (int64_t base = gspread() & ~31LL; base < kept; base += gstride()) {
+    const int64_t i = base + lane;
+    const bool in = i < kept;
+    const int32_t a = in ? id[ku[i]] : 0, b = in ? id[kv[i]] : 0;
+    if (in) {
+      cu[i] = a;
+      cv[i] = b;
+    }
+    add_edge_end(in, a, (int32_t)i, deg, inc);
+    add_edge_end(in, b, (int32_t)i, deg, inc);
+  }
+  if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
+  for (int64_t x0 = gspread(); x0 < verts; x0 += gstride()) {
+    int32_t x = (int32_t)x0;
+    for (int step = 0; step < kStripSteps && ld_relaxed(deg + x) == 1; step++) {
+      // x's one live edge; if its other end's thread is taking it, the word read here may be any edge:
+      // one that does not touch x, or one that is gone
+      const int32_t i = ld_relaxed(inc + x);
+      if ((uint32_t)i >= (uint32_t)kept) break;
+      const int32_t a = cu[i], b = cv[i];
+      if ((a != x && b != x) || atomicExch(gone + i, 1) != 0) break;
+      const int32_t y = a ^ b ^ x;
+      st_relaxed(deg + x, 0);
+      if (ld_relaxed(deg + y) >= kHub) break;
+      atomicXor(reinterpret_cast<uint32_t*>(inc + y), (uint32_t)i);
+      __threadfence();  // whoever sees y's new degree sees its edges without this one
+      if (atomicSub(deg + y, 1) != 2) break;
+      x = y;
+    }
+  }
+  if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
+  for (int64_t base = gspread() & ~31LL; base < kept; base += gstride()) {
+    const int64_t i = base + lane;
+    const bool in = i < kept, bridge = in && gone[i] != 0, core = in && !bridge;
+    const int32_t at = warp_place(bridge, f.nkeys);
+    if (bridge) f.keys[at] = kSlotTag | (uint64_t)i;
+    if (!__any_sync(kFull, core)) continue;
+    const int32_t ct = warp_place(core, f.nroots + kCoreEdges);
+    if (core) cs[ct] = (int32_t)i;
+    number_once<2>(core, {core ? cu[i] : 0, core ? cv[i] : 0}, {id2, id2},
+                   {f.nroots + kCoreVerts, f.nroots + kCoreVerts});
+  }
+  if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
+  // 4
+  const int32_t VC = f.nroots[kCoreVerts], mc = f.nroots[kCoreEdges];
+  if (mc > 0 && VC <= kCoreMax) {
+    if (blockIdx.x == 0) solve_core(R, reinterpret_cast<char*>(sm), gs, id2, cu, cv, cs, VC, mc);
+    if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
+  }
+  const bool on_grid = mc > 0 && VC > kCoreMax;
+  if (on_grid || *f.nkeys > kRankMax) {  // the keys so far by value: the sort of many, and the phases, need the room
+    const int32_t found = *f.nkeys;
+    for (int64_t i = gspread(); i < found; i += gstride()) f.keys[i] = resolved(A, ko, f.keys[i]);
+  }
+  if (on_grid) {
+    // a spanning forest of the core, in keys2 (its tree edges from the front, the others from the back)
+    // and R.tmp (the tree edges' places in F)
+    int32_t* const tu = reinterpret_cast<int32_t*>(f.keys2);
+    int32_t* const tv = tu + V;
+    for (int64_t base = gspread() & ~31LL; base < mc; base += gstride()) {
+      const int64_t i = base + lane;
+      const bool live = i < mc;
+      int32_t a = 0, b = 0, slot = 0;
+      if (live) {
+        slot = cs[i];
+        a = id2[cu[slot]];
+        b = id2[cv[slot]];
+      }
+      const bool joins = live && uf_link(f.P, a, b);
+      const int32_t at = warp_place(joins, f.nroots + kCntTree);
+      const int32_t xt = warp_place(live && !joins, f.nroots + kCntRest);
+      if (joins) {
+        tu[at] = a;
+        tv[at] = b;
+        R.tmp[at] = ko[slot];
+      } else if (live) {
+        tu[V - 1 - xt] = a;
+        tv[V - 1 - xt] = b;
+      }
+    }
+    if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
+    FinArgs B = A;
+    const int32_t nx = f.nroots[kCntRest];
+    B.V = VC;
+    B.orig = R.tmp;
+    B.ou = A.tu;
+    B.ov = A.tv;
+    B.tu = tu;
+    B.tv = tv;
+    B.d_nt = f.nroots + kCntTree;
+    B.xu = tu + (V - nx);
+    B.xv = tv + (V - nx);
+    B.d_nx = f.nroots + kCntRest;
+    B.cx = V;
+    B.P_tree = f.P;
+    if (!forest_bridges<true>(B, sm, red, &bar_epoch)) return;
+  }
+  if (on_grid || *f.nkeys > kRankMax)
+    if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
+  if (!sort_keys(A, ko, -1, sm, red, &bar_epoch)) return;
+  write_count(A);
+}
+
 #undef BARRIER
+
 
 int bits_for(int32_t V) {
   int k = 1;
@@ -885,21 +1316,21 @@ int bits_for(int32_t V) {
   return k;
 }
 
-// ---- 2-edge-connected components: union-find over the certificate minus its bridges ----
-__global__ void tecc_init_kernel(FinalBufs f, int32_t V) {
-  for (int64_t x = gtid(); x < V; x += gstride()) f.P[x] = (int32_t)x;
+// ---- 2-edge-connected components: the F' components (P2, flat) joined over the F edges between them that
+// are no bridges ----
+__global__ void tecc_init_kernel(FinalBufs f, const int32_t* P2, int32_t V) {
+  for (int64_t x = gtid(); x < V; x += gstride()) f.P[x] = P2[x];
   if (gtid() == 0) *f.nkeys = 0;
 }
 
-__global__ void tecc_link_kernel(FinalBufs f, int32_t V, const int32_t* xu, const int32_t* xv, const int32_t* d_nx,
-                                 int32_t cx) {
+__global__ void tecc_link_kernel(FinalBufs f, const int32_t* P2, int32_t V, const int32_t* tu, const int32_t* tv,
+                                 const int32_t* d_nt) {
   if (*f.status) return;  // the bridge stage failed: labels are left untouched
-  for (int64_t y = gtid(); y < V; y += gstride())
-    if (f.par[y] >= 0 && !f.bflag[y]) uf_link(f.P, (int32_t)y, f.par[y]);
-  const int32_t nx = min(*d_nx, cx);
-  for (int64_t e = gtid(); e < nx; e += gstride()) {
-    const int32_t a = xu[e], b = xv[e];
-    if ((uint32_t)a < (uint32_t)V && (uint32_t)b < (uint32_t)V && a != b) uf_link(f.P, a, b);
+  const int32_t nt = min(*d_nt, V);
+  for (int64_t e = gtid(); e < nt; e += gstride()) {
+    if (f.bflag[e]) continue;
+    const int32_t a = P2[tu[e]], b = P2[tv[e]];
+    if (a != b) uf_link(f.P, a, b);
   }
 }
 
@@ -925,20 +1356,16 @@ __global__ void tecc_count_kernel(FinalBufs f, int64_t* count) {
 
 }  // namespace
 
-void two_edge_components(const Launch& L, const FinalBufs& f, int32_t V, const int32_t* xu, const int32_t* xv,
-                         const int32_t* d_nx, int64_t cap_extra, int32_t* labels, int64_t* count_dev) {
+void two_edge_components(const Launch& L, const FinalBufs& f, const CertBufs& c, int32_t V, int32_t* labels,
+                         int64_t* count_dev) {
   const int bs = 256;
   const int g = (int)std::min<int64_t>(ceil_div(std::max(V, 1), bs), (int64_t)L.num_sms * 16);
-  const int32_t cx = (int32_t)std::min<int64_t>(cap_extra, INT32_MAX);
-  tecc_init_kernel<<<g, bs, 0, L.stream>>>(f, V);
-  tecc_link_kernel<<<g, bs, 0, L.stream>>>(f, V, xu, xv, d_nx, cx);
+  tecc_init_kernel<<<g, bs, 0, L.stream>>>(f, c.P2, V);
+  tecc_link_kernel<<<g, bs, 0, L.stream>>>(f, c.P2, V, c.f1u, c.f1v, c.cnt);
   tecc_label_kernel<<<g, bs, 0, L.stream>>>(f, V, labels, count_dev);
   tecc_count_kernel<<<1, 1, 0, L.stream>>>(f, count_dev);
   *L.launches += 4;
 }
-
-namespace {
-}  // namespace
 
 size_t final_bytes(int32_t V) {
   const size_t Vs = (size_t)std::max(V, 1);
@@ -998,9 +1425,11 @@ FinalBufs carve_final(void* base, int32_t V, int32_t* status) {
   return f;
 }
 
-void final_stage(const Launch& L, const FinalBufs& f, int32_t V, const int32_t* tu, const int32_t* tv,
-                 const int32_t* d_nt, int64_t cap_tree, const int32_t* xu, const int32_t* xv, const int32_t* d_nx,
-                 int64_t cap_extra, const int32_t* P_tree, int32_t* out, bool ordered) {
+namespace {
+
+// What both forms of the final stage share: the arguments, and the shared memory of the phases on the
+// grid (the superchunk sparse tables, [2][levels][nsup], and later the sort's staging).
+FinArgs final_args(const Launch& L, const FinalBufs& f, int32_t V, int32_t* out, size_t* smem) {
   // superchunk size: the shared-memory table covers at most kMaxSup superchunks
   const int64_t nch = ceil_div(std::max(V, 1), kChunk);
   int slg = 0;
@@ -1008,44 +1437,76 @@ void final_stage(const Launch& L, const FinalBufs& f, int32_t V, const int32_t* 
   const int64_t nsup = ceil_div(nch, (int64_t)kSuperChunks << slg);
   int levels = 1;
   while ((1LL << levels) <= nsup) levels++;
-  // shared memory: the superchunk sparse tables, [2][levels][nsup], and later the sort's
-  // staging of up to min(V - 1, kRankMax) keys and a slice's ranks
-  const size_t tables = sizeof(int32_t) * 2 * (size_t)levels * (size_t)nsup;
-  const size_t sort = kSmemSort;
-  const size_t smem = std::max(tables, sort);
-  // function attributes are per device: set on every call (a host-side call, no launch)
-  cudaFuncSetAttribute(final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)std::max(kSmemTables, kSmemSort));
-  int occ = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, final_kernel, kThreads, smem);
+  *smem = std::max(sizeof(int32_t) * 2 * (size_t)levels * (size_t)nsup, kSmemSort);
   FinArgs A{};
   A.f = f;
   A.V = V;
+  A.ct = std::max(V, 1);  // <= V tree edges keep the arcs in bounds
+  A.out = out;
+  A.key_cap = std::max(V, 1);
+  A.kbits = bits_for(std::max(V, 1));
+  A.sup_log = slg;
+  A.bar_polls = L.bar_polls > 0 ? L.bar_polls : kSpinCap;
+  A.hold_polls = L.hold_polls;
+  return A;
+}
+
+// Launches a final stage of a graph of V vertices: one block per SM at most (more blocks make every
+// grid barrier slower than they make the phases faster); small forests take fewer, one thread per
+// element of the tour (2V), which makes every grid barrier cheaper and leaves SMs free for work on
+// other streams (the server).
+void launch_final(const Launch& L, const FinalBufs& f, const void* kernel, int32_t V, size_t smem, size_t smem_max,
+                  void** args) {
+  // function attributes are per device: set on every call (a host-side call, no launch)
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
+  int occ = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kThreads, smem);
+  const int64_t want = ceil_div(2 * (int64_t)std::max(V, 1), kThreads);
+  const int blocks = (int)std::min<int64_t>({(int64_t)kMaxBlocks, (int64_t)std::max(occ, 1) * L.num_sms, want,
+                                             (int64_t)L.num_sms});
+  cudaMemsetAsync(f.bar_count, 0, sizeof(unsigned), L.stream);
+  cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(kThreads), args, smem, L.stream);
+  *L.launches += 1;
+}
+
+}  // namespace
+
+void final_stage(const Launch& L, const FinalBufs& f, int32_t V, const int32_t* tu, const int32_t* tv,
+                 const int32_t* d_nt, int64_t cap_tree, const int32_t* xu, const int32_t* xv, const int32_t* d_nx,
+                 int64_t cap_extra, const int32_t* P_tree, int32_t* out, bool ordered) {
+  size_t smem = 0;
+  FinArgs A = final_args(L, f, V, out, &smem);
   A.tu = tu;
   A.tv = tv;
   A.d_nt = d_nt;
-  A.ct = (int32_t)std::min<int64_t>(cap_tree, std::max(V, 1));  // <= V tree edges keep the arcs in bounds
+  A.ct = (int32_t)std::min<int64_t>(cap_tree, A.ct);
   A.xu = xu;
   A.xv = xv;
   A.d_nx = d_nx;
   A.cx = (int32_t)std::min<int64_t>(cap_extra, INT32_MAX);
   A.P_tree = P_tree;
-  A.out = out;
-  A.kbits = bits_for(std::max(V, 1));
-  A.sup_log = slg;
   A.ordered = ordered ? 1 : 0;
-  A.bar_polls = L.bar_polls > 0 ? L.bar_polls : kSpinCap;
-  A.hold_polls = L.hold_polls;
-  // one block per SM at most (more blocks make every grid barrier slower than they make the
-  // phases faster); small forests take fewer, one thread per element of the tour (2V), which
-  // makes every grid barrier cheaper and leaves SMs free for work on other streams (the server)
-  const int64_t want = ceil_div(2 * (int64_t)std::max(V, 1), kThreads);
-  const int blocks = (int)std::min<int64_t>({(int64_t)kMaxBlocks, (int64_t)std::max(occ, 1) * L.num_sms, want,
-                                             (int64_t)L.num_sms});
-  cudaMemsetAsync(f.bar_count, 0, sizeof(unsigned), L.stream);
   void* args[] = {&A};
-  cudaLaunchCooperativeKernel((void*)final_kernel, dim3(blocks), dim3(kThreads), args, smem, L.stream);
-  *L.launches += 1;
+  launch_final(L, f, (const void*)final_kernel, V, smem, std::max(kSmemTables, kSmemSort), args);
+}
+
+void reduced_stage(const Launch& L, const FinalBufs& f, const CertBufs& c, int32_t V, int32_t* out) {
+  size_t smem = 0;
+  ReducedArgs R{};
+  R.a = final_args(L, f, V, out, &smem);
+  R.a.tu = c.f1u;
+  R.a.tv = c.f1v;
+  R.a.d_nt = c.cnt;
+  R.P1 = c.P1;
+  R.xu = c.f2u;
+  R.xv = c.f2v;
+  R.d_nx = c.cnt + 1;
+  R.P2 = c.P2;
+  R.tmp = c.tmp;
+  smem = std::max(smem, (size_t)CoreLayout::kBytes);
+  void* args[] = {&R};
+  launch_final(L, f, (const void*)reduced_kernel, V, smem,
+               std::max({kSmemTables, kSmemSort, (size_t)CoreLayout::kBytes}), args);
 }
 
 }  // namespace bridges

@@ -91,7 +91,7 @@ struct FinalBufs {
   int32_t* pre;    // [V]
   int32_t* sz;     // [V]
   int32_t* par;    // [V] parent in the rooted tree (-1 for roots)
-  int32_t* bflag;  // [V] 1 if the tree edge (par[y], y) is a bridge
+  int32_t* bflag;  // [V] 1 if the tree edge (par[y], y) is a bridge (reduced_stage: if F edge e is one)
   int32_t* slo;    // [V] by vertex y (non-roots): min of lo over y's subtree range (at most pre y)
   int32_t* shi;    // [V] by vertex y (non-roots): max of hi over y's subtree range (at least its end)
   int32_t* lo;     // [V] indexed by preorder: smallest preorder among the X-neighbours
@@ -177,10 +177,10 @@ void cert_export(const Launch& L, const CertPlan& p, const CertBufs& b, int32_t*
 // ---- final.cu ----
 size_t final_bytes(int32_t V);
 FinalBufs carve_final(void* base, int32_t V, int32_t* status);
-// 2-edge-connected components after final_stage: labels[x] = minimum vertex of x's component
-// (the components of T u X minus its bridges); count_dev receives their number.
-void two_edge_components(const Launch& L, const FinalBufs& fb, int32_t V, const int32_t* xu, const int32_t* xv,
-                         const int32_t* d_nx, int64_t cap_extra, int32_t* labels, int64_t* count_dev);
+// 2-edge-connected components after reduced_stage: labels[x] = minimum vertex of x's component;
+// count_dev receives their number.
+void two_edge_components(const Launch& L, const FinalBufs& fb, const CertBufs& c, int32_t V, int32_t* labels,
+                         int64_t* count_dev);
 // Offers n extra edges to partition 0's union-finds (its certificate grows to a certificate of
 // the union).  Ids are range-checked first; on ERANGE nothing is changed.
 void cert_offer(const Launch& L, const CertPlan& p, const CertBufs& b, const int32_t* u, const int32_t* v, int64_t n);
@@ -192,6 +192,10 @@ void final_stage(const Launch& L, const FinalBufs& fb, int32_t V, const int32_t*
                  const int32_t* d_ntree, int64_t cap_tree, const int32_t* xu, const int32_t* xv,
                  const int32_t* d_nextra, int64_t cap_extra, const int32_t* P_tree, int32_t* out,
                  bool ordered = false);
+
+// The bridges of job 0's certificate alone, sorted to out, their number to fb.count: the final stage of
+// calls that need no rooted forest.  Flattens P2; fb.bflag[e] tells whether F edge e is a bridge.
+void reduced_stage(const Launch& L, const FinalBufs& fb, const CertBufs& c, int32_t V, int32_t* out);
 
 // ---- blocks.cu ----
 size_t ap_bytes(int32_t V);

@@ -106,7 +106,7 @@ extern "C" int64_t bridges_find_noalloc(struct CUstream_st* stream, const int32_
   cert_init(L, p, cb);
   cert_leaves(L, p, cb, u, v, nullptr);
   cert_merge(L, p, cb);
-  final_stage(L, fb, V, cb.f1u, cb.f1v, cb.cnt + 0, V, cb.f2u, cb.f2v, cb.cnt + 1, V, cb.P1, out ? out : spare_out);
+  reduced_stage(L, fb, cb, V, out ? out : spare_out);
   if (cudaGetLastError() != cudaSuccess) return BRIDGES_ECUDA;
   if (out_count_device) {
     if (cudaMemcpyAsync(out_count_device, fb.count, sizeof(int64_t), cudaMemcpyDeviceToDevice, s) != cudaSuccess) {

@@ -41,6 +41,7 @@
 // longer than the sample is certified here whole.
 #include <algorithm>
 
+#include "batched.h"
 #include "grid.cuh"
 #include "forest.cuh"
 
@@ -276,7 +277,7 @@ __global__ void __launch_bounds__(kThreads, 1) sample_kernel(SampleArgs A) {
   }
   for (int64_t x = gspread(); x < V; x += gstride()) {
     int2 r = R[x];
-    if (left != 0) r = make_int2(uf_find_static(J.P1, (int32_t)x), uf_find_static(J.P2, (int32_t)x));
+    if (left != 0) r = make_int2(uf_root_static(J.P1, (int32_t)x), uf_root_static(J.P2, (int32_t)x));
     J.P1[x] = r.x;
     J.P2[x] = r.y;
   }
@@ -372,6 +373,13 @@ void cert_sample(const Launch& L, const CertPlan& p, const CertBufs& b, const in
   a.H2 = b.hook + std::max(p.V, 1);
   a.R = b.roots;
   a.b = b;
+  const int64_t slots = a.groups * kGroup;
+  if (slots <= kBlockCertSlots && p.V <= kBatchVmax) {
+    const BlockCertArgs ba{u, v, a.n, a.stride, (int32_t)a.groups, p.V, a.snap, b};
+    block_certify_launch(L.stream, ba);  // a launch error is caught by the caller's error check
+    *L.launches += 1;
+    return;
+  }
   // one thread per sampled edge and per vertex, at most one block per SM (fewer blocks make the
   // barriers cheaper), at most 8 edges a thread (the plan keeps the sample below that)
   const int64_t work = std::max<int64_t>({a.groups * kGroup, (int64_t)p.V, 1});

@@ -234,8 +234,8 @@ __global__ void __launch_bounds__(1024, 1) ap_pass_kernel(PassArgs P) {
 }
 
 // ---- label snapshot: each vertex takes the largest class it belongs to ----
-// 1) flatten the classes; reset sizes, proposals and label ids
-__global__ void ap_flatten_kernel(ApBufs b, int32_t V, const int32_t* status) {
+// 1) flatten the classes; reset sizes, proposals and label ids (and the fused form's pairs)
+__global__ void ap_flatten_kernel(ApBufs b, int32_t V, const int32_t* status, unsigned long long* pairs) {
   if (*status) return;  // T is not valid: its arrays may be partly unset
   for (int64_t i = gtid(); i < V; i += gstride()) {
     int32_t r = (int32_t)i, p = __ldca(b.Q + i);
@@ -247,6 +247,10 @@ __global__ void ap_flatten_kernel(ApBufs b, int32_t V, const int32_t* status) {
     b.csize[i] = 0;
     b.tmp[i] = -1;
     b.best[i] = 0;
+    if (pairs) {
+      pairs[2 * i] = ~0ull;
+      pairs[2 * i + 1] = ~0ull;
+    }
   }
   if (gtid() == 0) {
     *b.nlab = 0;
@@ -431,8 +435,8 @@ __global__ void ap_scatter_kernel(ApBufs b, int32_t V, int64_t ntiles, const int
 // vertex, and F only grows: T_0 is a subforest of the final T.  So T_0 is rooted and numbered
 // right after the warm-up (the final stage on the partial certificate), its classes are seeded
 // (the blocks of T_0 u F'), and one stream then serves both passes: an edge is dropped from
-// shared memory when both ends carry the same combined label (same F' component, both in the
-// largest class), otherwise it is offered to the union-finds and, unless it just became a tree
+// shared memory when both ends carry the same combined label (same F' component, same class),
+// otherwise it is offered to the union-finds and, unless it just became a tree
 // edge, its cycle is merged on T_0 -- its path in the final T is its path in T_0 whenever both
 // ends lie in one tree of T_0.  Edges between two trees of T_0 are marked in a bitmap over the
 // list and walked once the final T is known, after the classes are renamed from T_0's edges to
@@ -528,15 +532,63 @@ __global__ void __launch_bounds__(1024, 1) ap_fused_kernel(FusedArgs F) {
   }
 }
 
-// The combined snapshot, in place over the certificate's F' labels: a vertex keeps its F' label
-// only if it lies in the largest class (whose label id the class root's tmp entry holds).
-__global__ void ap_combine_kernel(uint16_t* flab, ApBufs b, int64_t Vpad, int32_t V, const int32_t* status) {
+// The combined snapshot: one 16-bit label per distinct pair of F' label and largest class, so that two
+// vertices share it exactly when they share both.  (With the F' labels of the one largest class only, a
+// graph of 64 dense clusters, each a class of its own at this point, sent 1.89 M of its 2.5 M edges down
+// the slow path: 412 us for the stream, 36 us so.)  The pairs go into a hash table of 2V slots
+// (linear probing, never more than V pairs); the lane that places a pair numbers it.
+constexpr unsigned long long kNoPair = ~0ull;
+
+struct PairTable {
+  unsigned long long* key;  // [2V], kNoPair before
+  int32_t* id;              // [2V] the pair's number
+  int32_t* slot;            // [V] by vertex: its pair's slot, -1 for none
+};
+
+__global__ void ap_pair_kernel(const uint16_t* flab, ApBufs b, PairTable t, const int32_t* pre, int32_t V,
+                               const int32_t* status) {
   if (*status) return;
-  const unsigned long long g = *b.giant;
-  const int32_t gid = g ? b.tmp[(int32_t)(uint32_t)g] : -1;
-  for (int64_t x = gtid(); x < Vpad; x += gstride()) {
-    const bool keep = x < V && gid >= 0 && gid < (int32_t)kNoLabel && b.lab[x] == (uint16_t)gid;
-    if (!keep) flab[x] = kNoLabel;
+  const int lane = threadIdx.x & 31;
+  const uint32_t slots = 2 * (uint32_t)V;
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < V; base += gstride()) {
+    const int64_t x = base + threadIdx.x;
+    const uint64_t cls = x < V ? b.best[pre[x]] : 0;
+    const uint16_t f = x < V ? flab[x] : kNoLabel;
+    const bool has = cls != 0 && f != kNoLabel;
+    const unsigned long long key = (unsigned long long)(uint32_t)cls << 16 | f;
+    const unsigned peers = __match_any_sync(kFull, has ? key : kNoPair - 1 - lane);
+    const int leader = __ffs(peers) - 1;
+    int32_t at = -1;
+    if (has && lane == leader) {
+      const uint64_t h = (key * 0x9e3779b97f4a7c15ull) >> 32;
+      uint32_t s = (uint32_t)((h * slots) >> 32);
+      for (uint32_t k = 0; k < slots; k++) {
+        unsigned long long old = __ldca(t.key + s);  // (a placed pair never changes)
+        if (old == kNoPair) {
+          old = atomicCAS(t.key + s, kNoPair, key);
+          if (old == kNoPair) {
+            t.id[s] = atomicAdd(b.nlab, 1);
+            old = key;
+          }
+        }
+        if (old == key) {
+          at = (int32_t)s;
+          break;
+        }
+        s = s + 1 == slots ? 0 : s + 1;
+      }
+    }
+    at = __shfl_sync(kFull, at, leader);
+    if (x < V) t.slot[x] = has ? at : -1;
+  }
+}
+
+__global__ void ap_pair_label_kernel(ApBufs b, PairTable t, int32_t V, const int32_t* status) {
+  if (*status) return;
+  for (int64_t x = gtid(); x < b.Vpad; x += gstride()) {
+    const int32_t s = x < V ? t.slot[x] : -1;
+    const int32_t id = s >= 0 ? t.id[s] : -1;
+    b.lab[x] = (id >= 0 && id < (int32_t)kNoLabel) ? (uint16_t)id : kNoLabel;
   }
 }
 
@@ -659,14 +711,23 @@ void ap_seed(const Launch& L, const FinalBufs& f, const ApBufs& b, int32_t V, co
 }
 
 // The snapshot of the classes: mode 1, 16-bit labels (each vertex labelled with the largest
-// class containing it); mode 2, the bitmap of the largest class over vertices [0, Vb).
-void ap_snapshot(const Launch& L, const FinalBufs& f, const ApBufs& b, int32_t V, int32_t mode, int32_t Vb) {
+// class containing it; with flab, the F' labels, with the pair of both); mode 2, the bitmap of the
+// largest class over vertices [0, Vb).
+void ap_snapshot(const Launch& L, const FinalBufs& f, const ApBufs& b, int32_t V, int32_t mode, int32_t Vb,
+                 const uint16_t* flab = nullptr) {
   const int bs = 256;
   const int g = grid_of(L, V, bs);
-  ap_flatten_kernel<<<g, bs, 0, L.stream>>>(b, V, f.status);
+  // (the tour's successor words are free between the final stages)
+  const PairTable t{reinterpret_cast<unsigned long long*>(f.sr), reinterpret_cast<int32_t*>(f.sr2),
+                    reinterpret_cast<int32_t*>(f.sr2) + 2 * (int64_t)V};
+  ap_flatten_kernel<<<g, bs, 0, L.stream>>>(b, V, f.status, flab ? t.key : nullptr);
   ap_count_kernel<<<g, bs, 0, L.stream>>>(b, V, f.status);
   ap_propose_kernel<<<g, bs, 0, L.stream>>>(b, V, f.status);
-  if (mode == 2)
+  if (flab) {
+    ap_pair_kernel<<<g, bs, 0, L.stream>>>(flab, b, t, f.pre, V, f.status);
+    ap_pair_label_kernel<<<grid_of(L, b.Vpad, bs), bs, 0, L.stream>>>(b, t, V, f.status);
+    *L.launches += 1;
+  } else if (mode == 2)
     ap_bitmap_kernel<<<grid_of(L, Vb / 32 + 4, bs), bs, 0, L.stream>>>(b, f.pre, V, Vb, f.status);
   else
     ap_label_kernel<<<grid_of(L, b.Vpad, bs), bs, 0, L.stream>>>(b, f.pre, V, f.status);
@@ -793,17 +854,14 @@ void articulation_fused(const Launch& L, const CertPlan& p, const CertBufs& cb, 
   ap_seed(L, f, b0, V, cb.f2u, cb.f2v, cnt + 1);
   if (aev) cudaEventRecord(aev[1], L.stream);
   cert_snapshot(L, p, cb);
-  ap_snapshot(L, f, b0, V, 1, 0);
-  const int bs = 256;
-  ap_combine_kernel<<<grid_of(L, cb.Vpad, bs), bs, 0, L.stream>>>(cb.lab, b0, cb.Vpad, V, f.status);
-  *L.launches += 1;
+  ap_snapshot(L, f, b0, V, 1, 0, cb.lab);
   if (bev) cudaEventRecord(bev[2], L.stream);
   if (aev) cudaEventRecord(aev[2], L.stream);
   const bool vec = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v)) & 15) == 0;
   const int grid = (int)std::max<int64_t>(1, (int64_t)p.G);
   const Job J{cb.P1, cb.P2, cb.f1u, cb.f1v, cb.f2u, cb.f2v, cnt};
   FusedArgs a{ApArgs{f.pre, b0.Q, b0.PP, b0.LAST, V, f.status, b0.hooks}, J, f.root, fb.keep, fb.top, u, v, 0,
-              p.warm, p.sampled && p.stride > 1 ? (uint32_t)p.stride : 0u, cb.lab, cb.Vpad};
+              p.warm, p.sampled && p.stride > 1 ? (uint32_t)p.stride : 0u, b0.lab, b0.Vpad};
   // a certified prefix has only the block pass left; a certified sample is passed over by the
   // stream's forest half
   const int64_t first = a.stride > 1 ? 0 : p.warm;
@@ -833,6 +891,7 @@ void articulation_fused(const Launch& L, const CertPlan& p, const CertBufs& cb, 
   final_stage(L, f, V, cb.f1u, cb.f1v, cnt + 0, V, cb.f2u, cb.f2v, cnt + 1, V, cb.P1,
               out_bridges ? out_bridges : f.dscan);
   if (bev) cudaEventRecord(bev[5], L.stream);
+  const int bs = 256;
   const int g = grid_of(L, V, bs);
   ap_init_kernel<<<g, bs, 0, L.stream>>>(f, b1, V);
   ap_rename_min_kernel<<<g, bs, 0, L.stream>>>(f, b0, b1, V);

@@ -103,11 +103,11 @@ __device__ __forceinline__ void offer_edge(const ApArgs& A, int32_t a, int32_t b
 }
 
 __device__ __noinline__ void cycle_misses(const ApArgs& A, uint32_t m, const int32_t* __restrict__ u,
-                                          const int32_t* __restrict__ v, int64_t base) {
+                                          const int32_t* __restrict__ v, int64_t unit, int64_t step) {
   while (m) {
     const int bit = __ffs(m) - 1;
     m &= m - 1;
-    const int64_t e = miss_edge(bit, base);
+    const int64_t e = miss_edge(bit, unit, step);
     offer_edge(A, u[e], v[e]);
   }
 }
@@ -118,8 +118,9 @@ struct CycleSink {
   __device__ __forceinline__ void slot(bool need, int32_t a, int32_t b, int64_t) const {
     if (need) offer_edge(A, a, b);
   }
-  __device__ __forceinline__ void misses(uint32_t m, const int32_t* ub, const int32_t* vb, int64_t base) const {
-    cycle_misses(A, m, ub, vb, base);
+  __device__ __forceinline__ void misses(uint32_t m, const int32_t* ub, const int32_t* vb, int64_t unit,
+                                         int64_t step) const {
+    cycle_misses(A, m, ub, vb, unit, step);
   }
 };
 
@@ -455,6 +456,7 @@ struct FusedArgs {
   const int32_t* v;
   int64_t s, t;           // edge range of this launch
   uint32_t stride;        // > 1: every stride-th group of the list is in the certificate already
+  unsigned* queue;        // the stream's claims (stream_range), one launch over the whole list; else null
   const uint16_t* lab;    // combined labels (Vpad entries)
   int64_t Vpad;
 };
@@ -484,7 +486,7 @@ __device__ __forceinline__ void fused_edge(const FusedArgs& F, bool go, int32_t 
 
 template <bool FOREST>
 __device__ __noinline__ void fused_misses(const FusedArgs& F, uint32_t m, const int32_t* __restrict__ u,
-                                          const int32_t* __restrict__ v, int64_t base) {
+                                          const int32_t* __restrict__ v, int64_t unit, int64_t step) {
   while (__any_sync(kFull, m != 0)) {
     int32_t a = 0, b = 0;
     int64_t e = 0;
@@ -492,7 +494,7 @@ __device__ __noinline__ void fused_misses(const FusedArgs& F, uint32_t m, const 
     if (m) {
       const int bit = __ffs(m) - 1;
       m &= m - 1;
-      e = miss_edge(bit, base);
+      e = miss_edge(bit, unit, step);
       a = u[e];
       b = v[e];
       go = checked_edge(F.A, a, b);
@@ -507,8 +509,9 @@ struct FusedSink {
   __device__ __forceinline__ void slot(bool need, int32_t a, int32_t b, int64_t i) const {
     fused_edge<FOREST>(F, need && checked_edge(F.A, a, b), a, b, i);
   }
-  __device__ __forceinline__ void misses(uint32_t m, const int32_t* ub, const int32_t* vb, int64_t base) const {
-    fused_misses<FOREST>(F, m, ub, vb, base);
+  __device__ __forceinline__ void misses(uint32_t m, const int32_t* ub, const int32_t* vb, int64_t unit,
+                                         int64_t step) const {
+    fused_misses<FOREST>(F, m, ub, vb, unit, step);
   }
 };
 
@@ -524,7 +527,8 @@ __global__ void __launch_bounds__(1024, 1) ap_fused_kernel(FusedArgs F) {
   load_labels(slab, F.lab, F.Vpad);
   const FusedSink<FOREST> S{F};
   if (FOREST && use_tiles(F.s, F.t, gridDim.x, blockDim.x, kUnroll)) {  // the stream after the prefix, in tiles
-    stream_range<1, VEC, kUnroll>(S, F.u, F.v, F.s, F.t, (uint32_t)F.A.V, slab, blockIdx.x, gridDim.x);
+    stream_range<1, VEC, kUnroll>(S, F.u, F.v, F.s, F.t, (uint32_t)F.A.V, slab, blockIdx.x, gridDim.x,
+                                 F.queue);
   } else {  // the prefix (or a short list), a slice per block
     const int64_t n = F.t - F.s;
     const int64_t s = F.s + n * blockIdx.x / gridDim.x, t = F.s + n * (blockIdx.x + 1) / gridDim.x;
@@ -861,7 +865,8 @@ void articulation_fused(const Launch& L, const CertPlan& p, const CertBufs& cb, 
   const int grid = (int)std::max<int64_t>(1, (int64_t)p.G);
   const Job J{cb.P1, cb.P2, cb.f1u, cb.f1v, cb.f2u, cb.f2v, cnt};
   FusedArgs a{ApArgs{f.pre, b0.Q, b0.PP, b0.LAST, V, f.status, b0.hooks}, J, f.root, fb.keep, fb.top, u, v, 0,
-              p.warm, p.sampled && p.stride > 1 ? (uint32_t)p.stride : 0u, b0.lab, b0.Vpad};
+              p.warm, p.sampled && p.stride > 1 ? (uint32_t)p.stride : 0u,
+              chunks.ev ? nullptr : cb.ctl + kCtlQueue, b0.lab, b0.Vpad};
   // a certified prefix has only the block pass left; a certified sample is passed over by the
   // stream's forest half
   const int64_t first = a.stride > 1 ? 0 : p.warm;

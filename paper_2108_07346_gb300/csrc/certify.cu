@@ -68,15 +68,15 @@ __device__ __forceinline__ void scalar_slot(const Job& J, bool valid, int32_t a,
 // Kept out of line so the streaming loop stays small; the edges are re-read (they are still in
 // L1/L2).
 __device__ __noinline__ void offer_misses(const Job& J, uint32_t m, const int32_t* __restrict__ u,
-                                          const int32_t* __restrict__ v, int64_t base, int32_t V, int32_t* status,
-                                          int64_t first, uint32_t stride) {
+                                          const int32_t* __restrict__ v, int64_t unit, int64_t step, int32_t V,
+                                          int32_t* status, int64_t first, uint32_t stride) {
   while (__any_sync(kFull, m != 0)) {
     int32_t a = 0, b = 0;
     bool go = false;
     if (m) {
       const int bit = __ffs(m) - 1;
       m &= m - 1;
-      const int64_t e = miss_edge(bit, base);
+      const int64_t e = miss_edge(bit, unit, step);
       a = u[e];
       b = v[e];
       go = checked(a, b, V, status) && !excluded(first + e, stride);
@@ -97,8 +97,9 @@ struct ForestSink {
   __device__ __forceinline__ void slot(bool need, int32_t a, int32_t b, int64_t i) const {
     settle(J, need && checked(a, b, V, status) && !excluded(i, stride), a, b, V, status);
   }
-  __device__ __forceinline__ void misses(uint32_t m, const int32_t* ub, const int32_t* vb, int64_t base) const {
-    offer_misses(J, m, ub, vb, base, V, status, ub - u, stride);
+  __device__ __forceinline__ void misses(uint32_t m, const int32_t* ub, const int32_t* vb, int64_t unit,
+                                         int64_t step) const {
+    offer_misses(J, m, ub, vb, unit, step, V, status, ub - u, stride);
   }
 };
 
@@ -116,6 +117,7 @@ struct LeafArgs {
   int32_t Vb;    // bitmap snapshot: vertices it covers
   int64_t r0, r1;  // mode 1: only edges [r0, r1) of the rest (r1 <= r0: all of it)
   uint32_t stride;  // > 1: every stride-th group was certified before (a sample of the whole chunk)
+  unsigned* queue;  // mode 1, one launch over one partition: the stream's claims (stream_range); else null
   CertBufs b;
 };
 
@@ -145,7 +147,7 @@ __global__ void __launch_bounds__(1024, 1) leaf_kernel(LeafArgs A) {
   const ForestSink S{J, A.V, A.b.status, A.u, A.mode == 1 ? A.stride : 0};
   const uint32_t clampv = MODE == 2 ? (uint32_t)A.Vb : (uint32_t)A.V;
   if (A.mode == 1 && use_tiles(a, z, A.G, blockDim.x, kUnroll)) {
-    stream_range<MODE, VEC, kUnroll>(S, A.u, A.v, a, z, clampv, slab, m, A.G);
+    stream_range<MODE, VEC, kUnroll>(S, A.u, A.v, a, z, clampv, slab, m, A.G, A.queue);
   } else {
     const int64_t n = z - a;
     const int64_t s = a + n * m / A.G, t = a + n * (m + 1) / A.G;
@@ -414,13 +416,19 @@ CertPlan make_plan(int64_t E, int32_t V, int32_t M, int32_t fan_in, int32_t bloc
   p.mode = labels_fit ? 1 : 2;
   p.Vb = (int32_t)std::min<int64_t>(align_up((size_t)std::max(V, 1), 128), std::max<int64_t>(bm_cap, 128));
   const bool fits = labels_fit || bm_cap >= 128;
+  // Blocks per SM: 1,024 threads of the stream fit (64 registers each), as one block of 1,024 or two of
+  // 512; a second wave would wait for the first (2.5 M edges, 16-bit labels of 74 KB: 26 us with three
+  // blocks of 512 per SM, 24 with two).
   int cps = ctas_per_sm;
   if (cps <= 0) {
     const size_t snap_bytes = labels_fit ? lab_bytes : (size_t)(p.Vb / 32 + 4) * 4;
-    cps = fits ? (int)std::max<size_t>(1, std::min<size_t>(4, (228 * 1024) / (snap_bytes + 2048))) : 2;
+    cps = fits ? (int)std::max<size_t>(1, std::min<size_t>(2, (228 * 1024) / (snap_bytes + 2048))) : 2;
   }
-  p.block = block > 0 ? block : (cps <= 2 ? 1024 : 512);
+  p.block = block > 0 ? block : (cps < 2 || !fits ? 1024 : 512);
   p.G = (int32_t)std::max<int64_t>(1, ((int64_t)num_sms * cps) / p.M);
+  // a short list takes fewer blocks, one 16-byte unit of each array per thread (130 k edges: 18 us with
+  // 608 blocks, 12 with 64)
+  if (p.M == 1) p.G = (int32_t)std::max<int64_t>(1, std::min<int64_t>(p.G, ceil_div(E, 4 * (int64_t)p.block)));
   p.warm_block = p.block;
   const int64_t chunk = ceil_div(std::max<int64_t>(E, 1), p.M);
   p.sampled = p.M == 1 && labels_fit && warm != 0;
@@ -516,7 +524,7 @@ void cert_warm(const Launch& L, const CertPlan& p, const CertBufs& b, const int3
     return;
   }
   if (p.E == 0) return;
-  const LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 0, p.Vb, 0, 0, 0, b};
+  const LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 0, p.Vb, 0, 0, 0, nullptr, b};
   if (((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v)) & 15) == 0)
     launch_leaf<0, true>(L, p, a, 0);
   else
@@ -534,7 +542,8 @@ void cert_snapshot(const Launch& L, const CertPlan& p, const CertBufs& b) {
 void cert_stream(const Launch& L, const CertPlan& p, const CertBufs& b, const int32_t* u, const int32_t* v, int64_t r0,
                  int64_t r1) {
   if (p.E == 0 || !p.cache) return;
-  const LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 1, p.Vb, r0, r1, p.sampled ? (uint32_t)p.stride : 0u, b};
+  const LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 1, p.Vb, r0, r1, p.sampled ? (uint32_t)p.stride : 0u,
+                   p.M == 1 && r1 <= r0 ? b.ctl + kCtlQueue : nullptr, b};
   const bool vec = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v)) & 15) == 0;
   if (p.mode == 1) {
     const size_t smem = (size_t)b.Vpad * 2;

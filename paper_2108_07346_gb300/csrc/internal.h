@@ -15,6 +15,11 @@ namespace bridges {
 // Sentinel label: "no class", never equal to another vertex's label.
 constexpr uint16_t kNoLabel = 0xffff;
 
+// Control words of a call (CertBufs::ctl), cleared at its start: the sampled certificate's 64-bit barrier
+// word and label counter, and the stream's queue on a line of its own.
+constexpr int kCtlLabels = 2;
+constexpr int kCtlQueue = 32;
+
 // The sample of a plan is taken in groups of 2^kSampleShift edges.
 constexpr int kSampleShift = 3;
 

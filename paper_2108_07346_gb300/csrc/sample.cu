@@ -54,9 +54,6 @@ constexpr int kMaxRounds = 24;  // rounds before the remaining edges take the un
 constexpr unsigned kFewLive = 8192;  // live edges (and at most V / 4) that take the union-finds one by one
 constexpr int kGroup = 8;       // edges per group of the sample (kSampleShift)
 static_assert(kGroup == 1 << kSampleShift, "the stream's test of a sampled edge");
-// control words (CertBufs::ctl), cleared before the launch: the 64-bit barrier word, then the labels
-// handed out
-constexpr int kCtlLabels = 2;
 
 struct SampleArgs {
   const int32_t* u;

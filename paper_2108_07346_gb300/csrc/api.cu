@@ -26,6 +26,7 @@ constexpr size_t kMiscBytes = 1024;  // status word, device counts of bridges_fr
 constexpr int64_t kSmallCallEdges = 22528;  // a whole call on one block up to this many edges
 constexpr size_t kClearBytes = kMiscBytes + 256;  // cleared at a call's start: the misc area and the
                                                   // certificate's control words, which follow it
+constexpr size_t kBarAt = 128;       // the final stage's barrier count
 constexpr size_t kSpareAt = 512;     // the spare output slot: where a call that has no pairs or points
                                      // to write (V <= 1, null output) points the stages
 
@@ -74,6 +75,7 @@ Carved carve(bridges_ctx* c, const CertPlan& p) {
   k.fin = carve_final(base + kMiscBytes + align_up(cert_bytes(p), 256), p.V, k.status);
   k.cert.hook = reinterpret_cast<unsigned long long*>(k.fin.sr);
   k.cert.roots = k.fin.sr2;
+  k.fin.bar_count = reinterpret_cast<unsigned*>(base + kBarAt);
   return k;
 }
 
@@ -172,6 +174,8 @@ int init_ctx(bridges_ctx* c, int device, const bridges_opts* opts) {
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
   c->smem_optin = (size_t)optin;
+  if (!certify_prepare(c->smem_optin) || !final_prepare() || !blocks_prepare(c->smem_optin) || !batched_prepare())
+    return -1;
   if (cudaMallocHost(&c->h_pinned, 64) != cudaSuccess) return -1;
   if (c->opts.profile) {
     for (auto& set : c->ev)
@@ -213,16 +217,18 @@ bool small_call(const bridges_ctx* c, const CertPlan& p) {
          c->opts.test_hold_polls <= 0;
 }
 
-// The whole path on device-resident edges.  Leaves the count on the device (fin.count); the sorted
-// pairs go to out, or to the final stage's own dscan array (free by the time it sorts) when out is
+// The whole path on device-resident edges.  The count goes to *count (device memory, or the context's
+// pinned host area: the last kernel then writes it where the host reads it once the stream has been waited
+// for), or with count null to the workspace's own; the sorted pairs go to out, or to the final stage's own dscan array (free by the time it sorts) when out is
 // null.
 int64_t run_path(bridges_ctx* c, cudaStream_t s, const int32_t* u, const int32_t* v, int64_t E, int32_t V, int32_t M,
-                 int32_t* out, Carved* kout, CertPlan* pout, Want want) {
+                 int32_t* out, int64_t* count, Carved* kout, CertPlan* pout, Want want) {
   Range range("bridges: certificate + final stage");
   CertPlan p = plan_for(c, E, V, M);
   int64_t rc = ensure_ws(c, total_bytes(p), s);
   if (rc != BRIDGES_OK) return rc;
   Carved k = carve(c, p);
+  if (count) k.fin.count = count;
   Launch L = launch_for(c, s);
   c->last_cfg[0] = p.M;
   c->last_cfg[1] = p.f;
@@ -371,7 +377,7 @@ static int64_t issue_chunks(bridges_ctx* c, cudaStream_t s, const int32_t* hu, c
 }
 
 int64_t run_path_host(bridges_ctx* c, cudaStream_t s, const int32_t* hu, const int32_t* hv, int32_t* du, int32_t* dv,
-                      int64_t E, int32_t V, int32_t M, int32_t* out, Carved* kout, Want want) {
+                      int64_t E, int32_t V, int32_t M, int32_t* out, int64_t* count, Carved* kout, Want want) {
   Range range("bridges: pipelined host input");
   CertPlan p = plan_for(c, E, V, M);
   if (p.M != 1 || !p.cache) return 1;
@@ -382,6 +388,7 @@ int64_t run_path_host(bridges_ctx* c, cudaStream_t s, const int32_t* hu, const i
   int64_t rc = ensure_ws(c, total_bytes(p), s);
   if (rc != BRIDGES_OK) return rc;
   Carved k = carve(c, p);
+  if (count) k.fin.count = count;
   Launch L = launch_for(c, s);
   c->last_cfg[0] = p.M;
   c->last_cfg[1] = p.f;
@@ -492,15 +499,8 @@ int64_t bridges_find_ctx(bridges_ctx* c, struct CUstream_st* stream, const int32
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (cudaSetDevice(c->device) != cudaSuccess) return cuda_fail(cudaGetLastError());
   Carved k{};
-  rc = run_path(c, s, u, v, E, V, M, out, &k, nullptr, Want::bridges);
-  if (rc) return rc;
-  if (out_count_device) {
-    if (cudaMemcpyAsync(out_count_device, k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-      return cuda_fail(cudaGetLastError());
-    return BRIDGES_OK;
-  }
-  if (cudaMemcpyAsync(c->h_pinned, k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-    return cuda_fail(cudaGetLastError());
+  rc = run_path(c, s, u, v, E, V, M, out, out_count_device ? out_count_device : c->h_pinned, &k, nullptr, Want::bridges);
+  if (rc || out_count_device) return rc;
   if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_fail(cudaGetLastError());
   return c->h_pinned[0];
 }
@@ -534,7 +534,7 @@ int64_t bridges_find_host(bridges_ctx* c, struct CUstream_st* stream, const int3
   Carved k{};
   rc = 1;
   if (deferred)  // copies not issued yet: overlap them with the forest pass if the plan allows
-    rc = run_path_host(c, s, hu, hv, const_cast<int32_t*>(ru), const_cast<int32_t*>(rv), E, V, M, dout, &k, Want::bridges);
+    rc = run_path_host(c, s, hu, hv, const_cast<int32_t*>(ru), const_cast<int32_t*>(rv), E, V, M, dout, c->h_pinned, &k, Want::bridges);
   if (rc < 0) return rc;
   if (rc == 1) {
     if (deferred && E > 0 &&
@@ -543,11 +543,9 @@ int64_t bridges_find_host(bridges_ctx* c, struct CUstream_st* stream, const int3
          cudaMemcpyAsync(const_cast<int32_t*>(rv), hv, sizeof(int32_t) * (size_t)E, cudaMemcpyHostToDevice, s) !=
              cudaSuccess))
       return cuda_fail(cudaGetLastError());
-    rc = run_path(c, s, ru, rv, E, V, M, dout, &k, nullptr, Want::bridges);
+    rc = run_path(c, s, ru, rv, E, V, M, dout, c->h_pinned, &k, nullptr, Want::bridges);
     if (rc) return rc;
   }
-  if (cudaMemcpyAsync(c->h_pinned, k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess)
-    return cuda_fail(cudaGetLastError());
   if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_fail(cudaGetLastError());
   const int64_t n = c->h_pinned[0];
   if (n > 0) {
@@ -568,7 +566,7 @@ int64_t bridges_certificate(bridges_ctx* c, struct CUstream_st* stream, const in
   if (cudaSetDevice(c->device) != cudaSuccess) return cuda_fail(cudaGetLastError());
   Carved k{};
   CertPlan p{};
-  rc = run_path(c, s, u, v, E, V, M, nullptr, &k, &p, Want::certificate);
+  rc = run_path(c, s, u, v, E, V, M, nullptr, nullptr, &k, &p, Want::certificate);
   if (rc) return rc;
   if (V > 1) cert_export(launch_for(c, s), p, k.cert, cu, cv, ct);
   // counts and status
@@ -602,7 +600,7 @@ int64_t bridges_from_forest(bridges_ctx* c, struct CUstream_st* stream, const in
   cudaStreamSynchronize(s);
   h[0] = (int32_t)n_tree;
   h[1] = (int32_t)n_extra;
-  cudaMemsetAsync(k.status, 0, sizeof(int32_t), s);
+  cudaMemsetAsync(k.status, 0, kClearBytes, s);
   cudaMemcpyAsync(k.counts, h, 2 * sizeof(int32_t), cudaMemcpyHostToDevice, s);
   final_stage(L, k.fin, V, tu, tv, k.counts, n_tree, xu, xv, k.counts + 1, n_extra, nullptr, out ? out : k.spare);
   if (cudaGetLastError() != cudaSuccess) return BRIDGES_ECUDA;
@@ -628,7 +626,7 @@ int64_t bridges_rooted_forest(bridges_ctx* c, struct CUstream_st* stream, const 
   cudaStreamSynchronize(s);  // the pinned scratch may still be read by an earlier copy
   h[0] = (int32_t)n_tree;
   h[1] = 0;
-  cudaMemsetAsync(k.status, 0, sizeof(int32_t), s);
+  cudaMemsetAsync(k.status, 0, kClearBytes, s);
   cudaMemcpyAsync(k.counts, h, 2 * sizeof(int32_t), cudaMemcpyHostToDevice, s);
   // with no extra edges every tree edge is a bridge; the sorted list goes to dscan, which the
   // stage no longer reads once it sorts
@@ -922,11 +920,7 @@ int64_t default_split(const bridges_ctx* c, int64_t total_e) {
 int64_t run_single(bridges_ctx* c, cudaStream_t s, const int32_t* u, const int32_t* v, int64_t E, int32_t V, int32_t M,
                    int32_t* out, int64_t* count_dev) {
   Carved k{};
-  int64_t rc = run_path(c, s, u, v, E, V, M, out, &k, nullptr, Want::bridges);
-  if (rc) return rc;
-  if (cudaMemcpyAsync(count_dev, k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-    return cuda_fail(cudaGetLastError());
-  return BRIDGES_OK;
+  return run_path(c, s, u, v, E, V, M, out, count_dev, &k, nullptr, Want::bridges);
 }
 
 size_t single_workspace_bytes(const bridges_ctx* c, int64_t E, int32_t V) { return total_bytes(plan_for(c, E, V, 0)); }
@@ -1177,13 +1171,13 @@ extern "C" int32_t bridges_autotune(bridges_ctx* c, struct CUstream_st* stream, 
           // one untimed run (workspace growth, first-touch), then reps timed runs
           int64_t r = BRIDGES_OK;
           Carved k{};
-          r = run_path(c, s, u, v, E, V, 0, out, &k, nullptr, Want::bridges);
+          r = run_path(c, s, u, v, E, V, 0, out, nullptr, &k, nullptr, Want::bridges);
           if (r) {
             rc = (int32_t)r;
             break;
           }
           cudaEventRecord(e0, s);
-          for (int i = 0; i < reps && !r; i++) r = run_path(c, s, u, v, E, V, 0, out, &k, nullptr, Want::bridges);
+          for (int i = 0; i < reps && !r; i++) r = run_path(c, s, u, v, E, V, 0, out, nullptr, &k, nullptr, Want::bridges);
           cudaEventRecord(e1, s);
           if (r || cudaEventSynchronize(e1) != cudaSuccess) {
             rc = r ? (int32_t)r : (int32_t)BRIDGES_ECUDA;
@@ -1211,9 +1205,9 @@ extern "C" int32_t bridges_autotune(bridges_ctx* c, struct CUstream_st* stream, 
     o.profile = 0;
     c->opts = o;
     Carved k{};
-    int64_t r = run_path(c, s, u, v, E, V, 0, out, &k, nullptr, Want::bridges);
+    int64_t r = run_path(c, s, u, v, E, V, 0, out, nullptr, &k, nullptr, Want::bridges);
     cudaEventRecord(e0, s);
-    for (int i = 0; i < reps && !r; i++) r = run_path(c, s, u, v, E, V, 0, out, &k, nullptr, Want::bridges);
+    for (int i = 0; i < reps && !r; i++) r = run_path(c, s, u, v, E, V, 0, out, nullptr, &k, nullptr, Want::bridges);
     cudaEventRecord(e1, s);
     if (r || cudaEventSynchronize(e1) != cudaSuccess) {
       rc = r ? (int32_t)r : (int32_t)BRIDGES_ECUDA;
@@ -1296,12 +1290,11 @@ extern "C" int64_t bridges_two_edge_components(bridges_ctx* c, struct CUstream_s
   // the bridges go to the caller's buffer or to the (then unused) workspace key area
   Carved k{};
   CertPlan p{};
-  rc = run_path(c, s, u, v, E, V, M, out_bridges, &k, &p, Want::components);
+  rc = run_path(c, s, u, v, E, V, M, out_bridges, nullptr, &k, &p, Want::components);
   if (rc) return rc;
   Launch L = launch_for(c, s);
-  two_edge_components(L, k.fin, k.cert, V, labels, k.fin.count);
-  if (cudaMemcpyAsync(c->h_pinned, k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess)
+  two_edge_components(L, k.fin, k.cert, V, labels, c->h_pinned);
+  if (cudaStreamSynchronize(s) != cudaSuccess)
     return cuda_fail(cudaGetLastError());
   return c->h_pinned[0];
 }
@@ -1443,7 +1436,7 @@ static int64_t articulation_run(bridges_ctx* c, cudaStream_t s, const int32_t* u
     // free by the time the final stage sorts
     const Carved k0 = carve(c, p0);
     rc = run_path_host(c, s, hu, hv, const_cast<int32_t*>(u), const_cast<int32_t*>(v), E, V, M,
-                       out_bridges ? out_bridges : k0.fin.dscan, &k, Want::rooted);
+                       out_bridges ? out_bridges : k0.fin.dscan, nullptr, &k, Want::rooted);
     if (rc < 0) return rc;
     if (rc == 1 && E > 0 &&
         (cudaMemcpyAsync(const_cast<int32_t*>(u), hu, sizeof(int32_t) * (size_t)E, cudaMemcpyHostToDevice, s) !=
@@ -1453,7 +1446,7 @@ static int64_t articulation_run(bridges_ctx* c, cudaStream_t s, const int32_t* u
       return cuda_fail(cudaGetLastError());
   }
   if (rc == 1) {
-    rc = run_path(c, s, u, v, E, V, M, out_bridges, &k, nullptr, Want::rooted);
+    rc = run_path(c, s, u, v, E, V, M, out_bridges, nullptr, &k, nullptr, Want::rooted);
     if (rc) return rc;
   }
   if (!out_points) out_points = k.spare;  // V <= 1: no point is written
@@ -1588,10 +1581,9 @@ extern "C" int64_t bridges_inc_reset(bridges_inc* I, struct CUstream_st* stream,
   if (V > (1 << 30)) return BRIDGES_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (cudaSetDevice(I->ctx->device) != cudaSuccess) return cuda_fail(cudaGetLastError());
-  rc = run_path(I->ctx, s, u, v, E, V, M, out_bridges, &I->k, &I->p, Want::components);
+  rc = run_path(I->ctx, s, u, v, E, V, M, out_bridges, I->ctx->h_pinned, &I->k, &I->p, Want::components);
   if (rc) return rc;
-  if (cudaMemcpyAsync(I->ctx->h_pinned, I->k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess)
+  if (cudaStreamSynchronize(s) != cudaSuccess)
     return cuda_fail(cudaGetLastError());
   const int64_t n = I->ctx->h_pinned[0];
   I->V = V;
@@ -1608,11 +1600,11 @@ extern "C" int64_t bridges_inc_add(bridges_inc* I, struct CUstream_st* stream, c
   Launch L = launch_for(c, s);
   const Carved& k = I->k;
   const int32_t V = I->V;
-  if (cudaMemsetAsync(k.status, 0, sizeof(int32_t), s) != cudaSuccess) return cuda_fail(cudaGetLastError());
+  if (cudaMemsetAsync(k.status, 0, kClearBytes, s) != cudaSuccess) return cuda_fail(cudaGetLastError());
   cert_offer(L, I->p, k.cert, yu, yv, n);
-  reduced_stage(L, k.fin, k.cert, V, out_bridges ? out_bridges : k.spare);
-  if (cudaMemcpyAsync(c->h_pinned, k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess)
+  reduced_stage(L, k.fin, k.cert, V, out_bridges ? out_bridges : k.spare);  // (fin.count: the pinned area)
+  if (cudaGetLastError() != cudaSuccess) return BRIDGES_ECUDA;
+  if (cudaStreamSynchronize(s) != cudaSuccess)
     return cuda_fail(cudaGetLastError());
   return c->h_pinned[0];
 }
@@ -1624,9 +1616,9 @@ extern "C" int64_t bridges_inc_two_edge_components(bridges_inc* I, struct CUstre
   if (cudaSetDevice(c->device) != cudaSuccess) return cuda_fail(cudaGetLastError());
   Launch L = launch_for(c, s);
   const Carved& k = I->k;
-  two_edge_components(L, k.fin, k.cert, I->V, labels, k.fin.count);
-  if (cudaMemcpyAsync(c->h_pinned, k.fin.count, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess)
+  two_edge_components(L, k.fin, k.cert, I->V, labels, c->h_pinned);
+  if (cudaGetLastError() != cudaSuccess) return BRIDGES_ECUDA;
+  if (cudaStreamSynchronize(s) != cudaSuccess)
     return cuda_fail(cudaGetLastError());
   return c->h_pinned[0];
 }

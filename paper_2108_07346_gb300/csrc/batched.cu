@@ -424,8 +424,6 @@ __global__ void __launch_bounds__(kT, 1) small_call_kernel(const SmallCallArgs A
 
 bool block_certify_launch(cudaStream_t s, const BlockCertArgs& a) {
   const size_t smem = 3 * sizeof(uint32_t) * kVmax + sizeof(uint32_t) * ((size_t)a.groups << kSampleShift);
-  cudaFuncSetAttribute(block_certify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       3 * sizeof(uint32_t) * kVmax + sizeof(uint32_t) * kBlockCertSlots);
   block_certify_kernel<<<1, kT, smem, s>>>(a);
   return cudaPeekAtLastError() == cudaSuccess;
 }
@@ -440,25 +438,34 @@ bool small_call_launch(cudaStream_t s, const int32_t* u, const int32_t* v, int64
   const int64_t most = std::min<int64_t>(kRoom, E <= 2 * (4 * (int64_t)V + 2048) ? E + 7 : 4 * (int64_t)V + 2048) >> kSampleShift;
   const int64_t stride = std::max<int64_t>(1, ceil_div(groups, std::max<int64_t>(most, 1)));
   const SmallCallArgs a{u, v, E, stride, (int32_t)ceil_div(groups, stride), V, count, out};
-  cudaFuncSetAttribute(small_call_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kBytes);
   small_call_kernel<<<1, kT, L::kBytes, s>>>(a);
   return cudaPeekAtLastError() == cudaSuccess;
+}
+
+bool batched_prepare() {
+  const struct {
+    const void* kernel;
+    size_t bytes;
+  } most[] = {{(const void*)small_final_kernel, Layout<kVmax>::kBytes},
+              {(const void*)block_certify_kernel, sizeof(uint32_t) * (3 * kVmax + kBlockCertSlots)},
+              {(const void*)small_call_kernel, Layout<kVmax>::kBytes},
+              {(const void*)certify_kernel, kAGroups * kABytes},
+              {(const void*)bridge_kernel, kSmem}};
+  for (const auto& m : most)
+    if (cudaFuncSetAttribute(m.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)m.bytes) != cudaSuccess)
+      return false;
+  return true;
 }
 
 size_t batched_smem_bytes() { return (size_t)kSmem; }
 
 bool small_final_launch(cudaStream_t s, const SmallFinalArgs& a) {
   if (a.V < 2 || a.V > kVmax) return false;
-  cudaFuncSetAttribute(small_final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Layout<kVmax>::kBytes);
   small_final_kernel<<<1, kT, Layout<kVmax>::kBytes, s>>>(a);
   return cudaPeekAtLastError() == cudaSuccess;
 }
 
 bool batched_launch(cudaStream_t s, const BatchArgs* dev_args, int num_sms) {
-  // function attributes are per device: set on every launch (a host-side call; the launches are
-  // usually replayed from a CUDA graph anyway)
-  cudaFuncSetAttribute(certify_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAGroups * kABytes);
-  cudaFuncSetAttribute(bridge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   certify_kernel<<<num_sms, kT, kAGroups * kABytes, s>>>(dev_args);
   bridge_kernel<<<num_sms, kT, kSmem, s>>>(dev_args);
   return cudaGetLastError() == cudaSuccess;

@@ -106,6 +106,8 @@ struct SmallCallArgs {
   int32_t* out;    // receives the sorted (a, b) pairs, capacity 2 (V - 1)
 };
 
+// The kernels' shared-memory attributes on the current device (see prepare_kernels).
+bool batched_prepare();
 size_t batched_smem_bytes();
 // Launches the sampled certificate on one block (V <= kBatchVmax, at most kBlockCertSlots edges).
 constexpr int64_t kBlockCertSlots = 8 * kBatchVmax + 4096;

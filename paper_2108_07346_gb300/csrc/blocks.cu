@@ -682,7 +682,6 @@ int grid_of(const Launch& L, int64_t work, int block) {
 template <int MODE, bool VEC>
 void launch_pass(const Launch& L, const PassArgs& a, int grid, int block, size_t smem) {
   auto k = ap_pass_kernel<MODE, VEC>;
-  if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   k<<<grid, block, smem, L.stream>>>(a);
   *L.launches += 1;
 }
@@ -742,12 +741,21 @@ template <bool FOREST, bool VEC>
 void launch_fused(const Launch& L, const FusedArgs& a, int grid, int block) {
   auto k = ap_fused_kernel<FOREST, VEC>;
   const size_t smem = (size_t)a.Vpad * 2;
-  if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   k<<<grid, block, smem, L.stream>>>(a);
   *L.launches += 1;
 }
 
 }  // namespace
+
+bool blocks_prepare(size_t smem_optin) {
+  const int most = (int)(smem_optin - 1024);
+  for (const void* k : {(const void*)ap_pass_kernel<1, true>, (const void*)ap_pass_kernel<1, false>,
+                        (const void*)ap_pass_kernel<2, true>, (const void*)ap_pass_kernel<2, false>,
+                        (const void*)ap_fused_kernel<true, true>, (const void*)ap_fused_kernel<true, false>,
+                        (const void*)ap_fused_kernel<false, true>, (const void*)ap_fused_kernel<false, false>})
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess) return false;
+  return true;
+}
 
 size_t ap_bytes(int32_t V) {
   const size_t Vs = (size_t)std::max(V, 1);
@@ -892,7 +900,8 @@ void articulation_fused(const Launch& L, const CertPlan& p, const CertBufs& cb, 
     cudaEventRecord(bev[4], L.stream);
   }
   if (aev) cudaEventRecord(aev[3], L.stream);
-  // the final certificate: its bridges and the final T
+  // the final certificate: its bridges and the final T (the barrier's count starts over)
+  cudaMemsetAsync(f.bar_count, 0, sizeof(unsigned), L.stream);
   final_stage(L, f, V, cb.f1u, cb.f1v, cnt + 0, V, cb.f2u, cb.f2v, cnt + 1, V, cb.P1,
               out_bridges ? out_bridges : f.dscan);
   if (bev) cudaEventRecord(bev[5], L.stream);

@@ -385,13 +385,21 @@ void snapshot_bitmap(const Launch& L, const CertPlan& p, const CertBufs& b) {
 template <int MODE, bool VEC>
 void launch_leaf(const Launch& L, const CertPlan& p, const LeafArgs& a, size_t smem) {
   auto k = leaf_kernel<MODE, VEC>;
-  if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   // the warm-up launch is contention-bound on the union-finds: it may use fewer threads
   k<<<(unsigned)((int64_t)p.M * p.G), a.mode == 0 ? p.warm_block : p.block, smem, L.stream>>>(a);
   *L.launches += 1;
 }
 
 }  // namespace
+
+bool certify_prepare(size_t smem_optin) {
+  const int most = (int)(smem_optin - 1024);
+  for (const void* k : {(const void*)leaf_kernel<1, true>, (const void*)leaf_kernel<1, false>,
+                        (const void*)leaf_kernel<2, true>, (const void*)leaf_kernel<2, false>,
+                        (const void*)merge_kernel<true>})
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most) != cudaSuccess) return false;
+  return true;
+}
 
 CertPlan make_plan(int64_t E, int32_t V, int32_t M, int32_t fan_in, int32_t block, int32_t ctas_per_sm, int64_t warm,
                    int num_sms, size_t smem_optin, int32_t warm_block) {
@@ -589,7 +597,6 @@ void cert_merge(const Launch& L, const CertPlan& p, const CertBufs& b) {
     if (cache) {
       snapshot(L, p, b, step, njobs);
       auto k = merge_kernel<true>;
-      if (smem > 48 * 1024) cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       k<<<(unsigned)(njobs * G), block, smem, L.stream>>>(a);
     } else {
       merge_kernel<false><<<(unsigned)(njobs * G), block, 0, L.stream>>>(a);

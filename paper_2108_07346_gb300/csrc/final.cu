@@ -1390,8 +1390,7 @@ FinalBufs carve_final(void* base, int32_t V, int32_t* status) {
   c += 256;
   f.nkeys = reinterpret_cast<int32_t*>(c);
   c += 256;
-  f.bar_count = reinterpret_cast<unsigned*>(c);
-  c += 256;
+  c += 256;  // (spare)
   f.nroots = reinterpret_cast<int32_t*>(c);
   c += 256;
   int32_t** va[13] = {&f.P,  &f.root, &f.head,  &f.rslot, &f.rlist, &f.pre, &f.sz,
@@ -1455,21 +1454,21 @@ FinArgs final_args(const Launch& L, const FinalBufs& f, int32_t V, int32_t* out,
 // grid barrier slower than they make the phases faster); small forests take fewer, one thread per
 // element of the tour (2V), which makes every grid barrier cheaper and leaves SMs free for work on
 // other streams (the server).
-void launch_final(const Launch& L, const FinalBufs& f, const void* kernel, int32_t V, size_t smem, size_t smem_max,
-                  void** args) {
-  // function attributes are per device: set on every call (a host-side call, no launch)
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_max);
-  int occ = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, kThreads, smem);
+void launch_final(const Launch& L, const void* kernel, int32_t V, size_t smem, void** args) {
   const int64_t want = ceil_div(2 * (int64_t)std::max(V, 1), kThreads);
-  const int blocks = (int)std::min<int64_t>({(int64_t)kMaxBlocks, (int64_t)std::max(occ, 1) * L.num_sms, want,
-                                             (int64_t)L.num_sms});
-  cudaMemsetAsync(f.bar_count, 0, sizeof(unsigned), L.stream);
+  const int blocks = (int)std::min<int64_t>({(int64_t)kMaxBlocks, want, (int64_t)L.num_sms});
   cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(kThreads), args, smem, L.stream);
   *L.launches += 1;
 }
 
 }  // namespace
+
+bool final_prepare() {
+  const size_t most = std::max(kSmemTables, kSmemSort);
+  return cudaFuncSetAttribute(final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) == cudaSuccess &&
+         cudaFuncSetAttribute(reduced_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)std::max(most, (size_t)CoreLayout::kBytes)) == cudaSuccess;
+}
 
 void final_stage(const Launch& L, const FinalBufs& f, int32_t V, const int32_t* tu, const int32_t* tv,
                  const int32_t* d_nt, int64_t cap_tree, const int32_t* xu, const int32_t* xv, const int32_t* d_nx,
@@ -1487,7 +1486,7 @@ void final_stage(const Launch& L, const FinalBufs& f, int32_t V, const int32_t* 
   A.P_tree = P_tree;
   A.ordered = ordered ? 1 : 0;
   void* args[] = {&A};
-  launch_final(L, f, (const void*)final_kernel, V, smem, std::max(kSmemTables, kSmemSort), args);
+  launch_final(L, (const void*)final_kernel, V, smem, args);
 }
 
 void reduced_stage(const Launch& L, const FinalBufs& f, const CertBufs& c, int32_t V, int32_t* out) {
@@ -1505,8 +1504,7 @@ void reduced_stage(const Launch& L, const FinalBufs& f, const CertBufs& c, int32
   R.tmp = c.tmp;
   smem = std::max(smem, (size_t)CoreLayout::kBytes);
   void* args[] = {&R};
-  launch_final(L, f, (const void*)reduced_kernel, V, smem,
-               std::max({kSmemTables, kSmemSort, (size_t)CoreLayout::kBytes}), args);
+  launch_final(L, (const void*)reduced_kernel, V, smem, args);
 }
 
 }  // namespace bridges

@@ -79,8 +79,8 @@ struct CertBufs {
 // Device buffers of the final stage (Euler tour, ranges, test, sort), one cooperative kernel.
 struct FinalBufs {
   int32_t* status;
-  int64_t* count;  // [1] bridges found (device)
-  unsigned* bar_count;  // grid barrier: arrivals (grows within a launch)
+  int64_t* count;  // [1] receives the bridges found (written only; device or mapped host memory)
+  unsigned* bar_count;  // grid barrier: arrivals (grows within a launch; cleared by the caller before it)
   int32_t* nroots;  // [1] trees of the forest (one-vertex trees included)
   int32_t* P;      // [V] union-find over the tree (built by the stage when it owns it)
   int32_t* root;   // [V] root (minimum vertex) of each vertex's tree
@@ -146,6 +146,12 @@ struct FusedBufs {
   int64_t nwords;  // E / 32 + 1
   int64_t ntop;    // nwords / 32 + 1
 };
+
+// Every kernel's shared-memory attribute on the current device, once per context (function attributes
+// stay with the device's context; setting them on each call cost host time before every launch).
+bool certify_prepare(size_t smem_optin);
+bool final_prepare();
+bool blocks_prepare(size_t smem_optin);
 
 // ---- certify.cu ----
 void cert_init(const Launch& L, const CertPlan& p, const CertBufs& b);

@@ -11,6 +11,7 @@
 #include <mutex>
 
 #include "../../include/bridges.h"
+#include "batched.h"
 #include "internal.h"
 
 namespace {
@@ -57,6 +58,10 @@ int64_t setup_device(int dev, DeviceSetup** out) {
       return BRIDGES_ECUDA;
     }
     s.smem_optin = (size_t)optin;
+    if (!certify_prepare(s.smem_optin) || !final_prepare() || !batched_prepare()) {
+      cudaGetLastError();
+      return BRIDGES_ECUDA;
+    }
     s.scratch = ptr;
     s.ready = true;
   }
@@ -90,6 +95,7 @@ extern "C" int64_t bridges_find_noalloc(struct CUstream_st* stream, const int32_
   FinalBufs fb = carve_final(base + kMiscBytes + cert, p.V, status);
   cb.hook = reinterpret_cast<unsigned long long*>(fb.sr);
   cb.roots = fb.sr2;
+  fb.bar_count = reinterpret_cast<unsigned*>(base + 128);  // in the cleared page, beside the status word
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   Launch L{s, &S->launches, S->num_sms, S->smem_optin};
   // a graph of at most one vertex has no pairs to write; its output pointer may be null, so the

@@ -57,6 +57,65 @@ __device__ __forceinline__ bool checked(int32_t a, int32_t b, int32_t V, int32_t
   return a != b;
 }
 
+// A warp's winners on their way to the lists, in shared memory: kStage places for F, then for F', and how
+// many of each are taken.  A warp sends a list's winners on when it has 32 of them, with one add to the
+// list's counter; without that every warp with a winner adds for itself, and the adds to one address queue
+// (16.8 M R-MAT edges, about a million winners: 175 + 397 us for prefix and stream, 161 + 174 so).
+constexpr int kStage = 64;
+
+struct WinBuf {
+  int2* place;  // this warp's 2 * kStage; null: winners go straight to the lists
+  int32_t* n;   // this warp's [2]
+};
+
+// Sends the c winners in w's list `which` to the certificate's list from place `at` on.
+__device__ __forceinline__ void send(const Job& J, const WinBuf& w, int which, int32_t c, int32_t at, int32_t cap,
+                                     int32_t* status) {
+  int32_t* ou = which ? J.f2u : J.f1u;
+  int32_t* ov = which ? J.f2v : J.f1v;
+  for (int32_t i = threadIdx.x & 31; i < c; i += 32) {
+    const int2 e = w.place[which * kStage + i];
+    if (at + i < cap) {
+      ou[at + i] = e.x;
+      ov[at + i] = e.y;
+    } else {
+      set_status(status, BRIDGES_EINTERNAL_CODE);
+    }
+  }
+}
+
+// Every lane of the warp calls it (pred may be false).
+__device__ __forceinline__ void stage_append(const Job& J, const WinBuf& w, int which, bool pred, int32_t a, int32_t b,
+                                             int32_t cap, int32_t* status) {
+  const unsigned m = __ballot_sync(kFull, pred);
+  if (!m) return;
+  int32_t c = w.n[which];
+  if (pred) w.place[which * kStage + c + __popc(m & lanemask_lt())] = make_int2(a, b);
+  c += __popc(m);
+  __syncwarp();
+  if (c >= 32) {
+    int32_t at = 0;
+    if ((threadIdx.x & 31) == 0) at = atomicAdd(J.cnt + which, c);
+    send(J, w, which, c, __shfl_sync(kFull, at, 0), cap, status);
+    c = 0;
+  }
+  if ((threadIdx.x & 31) == 0) w.n[which] = c;
+  __syncwarp();
+}
+
+// settle with the winners staged.
+__device__ __forceinline__ void settle(const Job& J, const WinBuf& w, bool need, int32_t a, int32_t b, int32_t cap,
+                                       int32_t* status) {
+  if (!w.place) {
+    settle(J, need, a, b, cap, status);
+    return;
+  }
+  if (!__any_sync(kFull, need)) return;
+  const int r = need ? offer(J, a, b) : 0;
+  stage_append(J, w, 0, r == 1, a, b, cap, status);
+  stage_append(J, w, 1, r == 2, a, b, cap, status);
+}
+
 // Scalar slot for the merge and offer kernels: every lane of the warp calls it (valid may be
 // false).
 __device__ __forceinline__ void scalar_slot(const Job& J, bool valid, int32_t a, int32_t b, int32_t V,
@@ -67,7 +126,7 @@ __device__ __forceinline__ void scalar_slot(const Job& J, bool valid, int32_t a,
 // The edges of this thread's current tile whose bit is set in `m` go through the union-finds.
 // Kept out of line so the streaming loop stays small; the edges are re-read (they are still in
 // L1/L2).
-__device__ __noinline__ void offer_misses(const Job& J, uint32_t m, const int32_t* __restrict__ u,
+__device__ __noinline__ void offer_misses(const Job& J, const WinBuf& w, uint32_t m, const int32_t* __restrict__ u,
                                           const int32_t* __restrict__ v, int64_t unit, int64_t step, int32_t V,
                                           int32_t* status, int64_t first, uint32_t stride) {
   while (__any_sync(kFull, m != 0)) {
@@ -81,28 +140,28 @@ __device__ __noinline__ void offer_misses(const Job& J, uint32_t m, const int32_
       b = v[e];
       go = checked(a, b, V, status) && !excluded(first + e, stride);
     }
-    const int r = go ? offer(J, a, b) : 0;
-    warp_append(r == 1, a, b, J.cnt + 0, J.f1u, J.f1v, V, status);
-    warp_append(r == 2, a, b, J.cnt + 1, J.f2u, J.f2v, V, status);
+    settle(J, w, go, a, b, V, status);
   }
 }
 
 // The forest pass's slow path (see stream_range): Alg. 2's two union-finds.
 struct ForestSink {
   const Job& J;
+  const WinBuf& w;
   int32_t V;
   int32_t* status;
   const int32_t* u;  // the list's start, and the stride of the sample already certified
   uint32_t stride;
   __device__ __forceinline__ void slot(bool need, int32_t a, int32_t b, int64_t i) const {
-    settle(J, need && checked(a, b, V, status) && !excluded(i, stride), a, b, V, status);
+    settle(J, w, need && checked(a, b, V, status) && !excluded(i, stride), a, b, V, status);
   }
   __device__ __forceinline__ void misses(uint32_t m, const int32_t* ub, const int32_t* vb, int64_t unit,
                                          int64_t step) const {
-    offer_misses(J, m, ub, vb, unit, step, V, status, ub - u, stride);
+    offer_misses(J, w, m, ub, vb, unit, step, V, status, ub - u, stride);
   }
 };
 
+constexpr size_t kStageBytes = 32 * 2 * kStage * sizeof(int2);  // of a block of 1,024 threads
 constexpr int kUnroll = 4;  // int4 units of u (and of v) in flight per thread: 16 edges
 
 struct LeafArgs {
@@ -117,6 +176,7 @@ struct LeafArgs {
   int32_t Vb;    // bitmap snapshot: vertices it covers
   int64_t r0, r1;  // mode 1: only edges [r0, r1) of the rest (r1 <= r0: all of it)
   uint32_t stride;  // > 1: every stride-th group was certified before (a sample of the whole chunk)
+  int32_t stage_at;  // the warps' winners' place behind the snapshot in shared memory (bytes; < 0: none)
   unsigned* queue;  // mode 1, one launch over one partition: the stream's claims (stream_range); else null
   CertBufs b;
 };
@@ -144,7 +204,14 @@ __global__ void __launch_bounds__(1024, 1) leaf_kernel(LeafArgs A) {
   if (MODE == 1) load_labels(slab, A.b.lab + j * A.b.Vpad, A.b.Vpad);
   if (MODE == 2) load_words(slab, A.b.lab + j * A.b.Vpad, (A.Vb / 32 + 4) / 4);
   const Job J = job_of(A.b, A.V, j);
-  const ForestSink S{J, A.V, A.b.status, A.u, A.mode == 1 ? A.stride : 0};
+  __shared__ int32_t staged[32][2], sent[2];
+  if (threadIdx.x < 64) staged[threadIdx.x >> 1][threadIdx.x & 1] = 0;
+  __syncthreads();
+  const int warp = threadIdx.x >> 5;
+  const WinBuf win{A.stage_at < 0 ? nullptr
+                                  : reinterpret_cast<int2*>(reinterpret_cast<char*>(slab) + A.stage_at) + warp * 2 * kStage,
+                 staged[warp]};
+  const ForestSink S{J, win, A.V, A.b.status, A.u, A.mode == 1 ? A.stride : 0};
   const uint32_t clampv = MODE == 2 ? (uint32_t)A.Vb : (uint32_t)A.V;
   if (A.mode == 1 && use_tiles(a, z, A.G, blockDim.x, kUnroll)) {
     stream_range<MODE, VEC, kUnroll>(S, A.u, A.v, a, z, clampv, slab, m, A.G, A.queue);
@@ -152,6 +219,20 @@ __global__ void __launch_bounds__(1024, 1) leaf_kernel(LeafArgs A) {
     const int64_t n = z - a;
     const int64_t s = a + n * m / A.G, t = a + n * (m + 1) / A.G;
     stream_range<MODE, VEC, kUnroll>(S, A.u, A.v, s, t, clampv, slab);
+  }
+  if (A.stage_at < 0) return;
+  // the winners still staged, with one add per list and block
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    int32_t sum = 0;
+    for (int k = 0; k < (int)(blockDim.x >> 5); k++) sum += staged[k][threadIdx.x];
+    sent[threadIdx.x] = sum ? atomicAdd(J.cnt + threadIdx.x, sum) : 0;
+  }
+  __syncthreads();
+  for (int which = 0; which < 2; which++) {
+    int32_t at = sent[which];
+    for (int k = 0; k < warp; k++) at += staged[k][which];
+    send(J, win, which, staged[warp][which], at, A.V, A.b.status);
   }
 }
 
@@ -276,50 +357,38 @@ __global__ void snap_roots_kernel(CertBufs b, int32_t V, int64_t step, int64_t n
   }
 }
 
-// ---- bitmap snapshot (large V): the largest F' component of each job as one bit per vertex ----
-// 1) sizes of the F' components (tmp counts members; the flatten set tmp to 0), lanes with the
-//    same root adding once per warp
-__global__ void bm_count_kernel(CertBufs b, int32_t V, int64_t njobs) {
-  const int64_t total = njobs * V;
-  const int lane = threadIdx.x & 31;
-  for (int64_t base = blockIdx.x * (int64_t)blockDim.x; base < total; base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    const bool in = i < total;
-    const int64_t j = in ? i / V : 0;
-    const int32_t x = in ? (int32_t)(i % V) : 0;
-    const long long key = in ? j * (long long)V + b.P2[j * V + x] : -1LL - lane;
-    const unsigned peers = __match_any_sync(kFull, (unsigned long long)key);
-    if (in && lane == __ffs(peers) - 1) atomicAdd(b.tmp + key, __popc(peers));
-  }
+// ---- bitmap snapshot (large V): one large F' component of each job as one bit per vertex ----
+// 1) the component: the most frequent root among 256 vertices spread over [0, V) (any component would be
+//    exact; counting every vertex took 46 us on 2^20 vertices, the giant's counter taking an atomic from
+//    every warp)
+constexpr int kProbes = 256;
+
+__global__ void __launch_bounds__(kProbes) bm_probe_kernel(CertBufs b, int32_t V, int64_t njobs) {
+  __shared__ int32_t probe[kProbes];
+  __shared__ unsigned best;
+  const int64_t j = blockIdx.x;
+  const int32_t mine = b.P2[j * V + (int64_t)threadIdx.x * V / kProbes];
+  probe[threadIdx.x] = mine;
+  if (threadIdx.x == 0) best = 0;
+  __syncthreads();
+  unsigned same = 0;
+  for (int k = 0; k < kProbes; k++) same += probe[k] == mine;
+  atomicMax(&best, same << 8 | (unsigned)(kProbes - 1 - threadIdx.x));
+  __syncthreads();
+  if (threadIdx.x == 0) b.giant[j] = (unsigned long long)(uint32_t)probe[kProbes - 1 - (best & (kProbes - 1))];
 }
 
-// 2) the largest component of each job: (size << 32 | ~root), ties to the smaller root
-__global__ void bm_best_kernel(CertBufs b, int32_t V, int64_t njobs) {
-  const int64_t total = njobs * V;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t j = i / V;
-    const int32_t x = (int32_t)(i % V);
-    if (b.P2[i] != x) continue;
-    const int32_t c = b.tmp[i];
-    if (c >= 2) atomicMax(b.giant + j, ((unsigned long long)c << 32) | (0xffffffffu - (uint32_t)x));
-  }
-}
-
-// 3) the bitmap words (in the job's label area): bit x set iff x < min(V, Vb) lies in the largest
-//    component; the word past Vb / 32 stays clear (the clamp target of out-of-range ids)
+// 2) the bitmap words (in the job's label area): bit x set iff x < min(V, Vb) lies in that component; the
+//    words from Vb / 32 on stay clear (the clamp target of out-of-range ids).  A warp writes a word.
 __global__ void bm_write_kernel(CertBufs b, int32_t V, int32_t Vb, int64_t njobs) {
   const int64_t nw = Vb / 32 + 4;  // a multiple of 4 words: the leaf kernel copies 16-byte units
-  const int64_t total = njobs * nw;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t j = i / nw, w = i % nw;
-    const unsigned long long g = b.giant[j];
-    const int32_t root = g ? (int32_t)(0xffffffffu - (uint32_t)(g & 0xffffffffu)) : -1;
-    uint32_t bits = 0;
-    for (int k = 0; k < 32; k++) {
-      const int64_t x = w * 32 + k;
-      if (root >= 0 && x < V && x < Vb && b.P2[j * V + x] == root) bits |= 1u << k;
-    }
-    reinterpret_cast<uint32_t*>(b.lab + j * b.Vpad)[w] = bits;
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; i < njobs * nw; i += warps) {
+    const int64_t j = i / nw, w = i % nw, x = w * 32 + lane;
+    const int32_t root = (int32_t)b.giant[j];
+    const unsigned bits = __ballot_sync(kFull, x < V && x < Vb && b.P2[j * V + x] == root);
+    if (lane == 0) reinterpret_cast<uint32_t*>(b.lab + j * b.Vpad)[w] = bits;
   }
 }
 
@@ -376,10 +445,9 @@ void snapshot_bitmap(const Launch& L, const CertPlan& p, const CertBufs& b) {
   const int bs = 256;
   const int g = grid_for(L, (int64_t)p.M * p.V, bs);
   snap_flatten_kernel<<<g, bs, 0, L.stream>>>(b, p.V, 1, p.M, 0);
-  bm_count_kernel<<<g, bs, 0, L.stream>>>(b, p.V, p.M);
-  bm_best_kernel<<<g, bs, 0, L.stream>>>(b, p.V, p.M);
-  bm_write_kernel<<<grid_for(L, (int64_t)p.M * (p.Vb / 32 + 4), bs), bs, 0, L.stream>>>(b, p.V, p.Vb, p.M);
-  *L.launches += 4;
+  bm_probe_kernel<<<(unsigned)p.M, kProbes, 0, L.stream>>>(b, p.V, p.M);
+  bm_write_kernel<<<grid_for(L, (int64_t)p.M * (p.Vb + 128), bs), bs, 0, L.stream>>>(b, p.V, p.Vb, p.M);
+  *L.launches += 3;
 }
 
 template <int MODE, bool VEC>
@@ -532,11 +600,11 @@ void cert_warm(const Launch& L, const CertPlan& p, const CertBufs& b, const int3
     return;
   }
   if (p.E == 0) return;
-  const LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 0, p.Vb, 0, 0, 0, nullptr, b};
+  const LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 0, p.Vb, 0, 0, 0, 0, nullptr, b};
   if (((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v)) & 15) == 0)
-    launch_leaf<0, true>(L, p, a, 0);
+    launch_leaf<0, true>(L, p, a, kStageBytes);
   else
-    launch_leaf<0, false>(L, p, a, 0);
+    launch_leaf<0, false>(L, p, a, kStageBytes);
 }
 
 void cert_snapshot(const Launch& L, const CertPlan& p, const CertBufs& b) {
@@ -550,17 +618,22 @@ void cert_snapshot(const Launch& L, const CertPlan& p, const CertBufs& b) {
 void cert_stream(const Launch& L, const CertPlan& p, const CertBufs& b, const int32_t* u, const int32_t* v, int64_t r0,
                  int64_t r1) {
   if (p.E == 0 || !p.cache) return;
-  const LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 1, p.Vb, r0, r1, p.sampled ? (uint32_t)p.stride : 0u,
-                   p.M == 1 && r1 <= r0 ? b.ctl + kCtlQueue : nullptr, b};
+  LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 1, p.Vb, r0, r1, p.sampled ? (uint32_t)p.stride : 0u,
+             -1, p.M == 1 && r1 <= r0 ? b.ctl + kCtlQueue : nullptr, b};
   const bool vec = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v)) & 15) == 0;
+  // the snapshot, and behind it the warps' winners where the block's shared memory has room
+  size_t smem = align_up(p.mode == 1 ? (size_t)b.Vpad * 2 : (size_t)(p.Vb / 32 + 4) * 4, 16);
+  const size_t stage = kStageBytes * (size_t)p.block / 1024;
+  if (smem + stage + 1024 <= L.smem_optin) {
+    a.stage_at = (int32_t)smem;
+    smem += stage;
+  }
   if (p.mode == 1) {
-    const size_t smem = (size_t)b.Vpad * 2;
     if (vec)
       launch_leaf<1, true>(L, p, a, smem);
     else
       launch_leaf<1, false>(L, p, a, smem);
   } else {
-    const size_t smem = (size_t)(p.Vb / 32 + 4) * 4;
     if (vec)
       launch_leaf<2, true>(L, p, a, smem);
     else

@@ -51,7 +51,7 @@ struct CertPlan {
                    // 1: the whole list)
   bool cache;      // a snapshot is taken after the warm-up
   int32_t mode;    // its form: 1 = 16-bit F' labels (2V bytes fit in shared memory), 2 = bitmap
-                   // of the largest F' component (for larger V)
+                   // of one large F' component (for larger V)
   int32_t Vb;      // mode 2: vertices [0, Vb) covered by the bitmap (a multiple of 128)
 };
 
@@ -64,7 +64,7 @@ struct CertBufs {
   int2* roots;               // [V] its roots in both forests (scratch of the final stage, idle until then)
   int32_t* cnt;     // [2*M] forest sizes |F|, |F'| per job
   int32_t* nlab;    // [M] labels handed out per job
-  unsigned long long* giant;  // [M] bitmap snapshot: (size << 32 | ~root) of the largest F' component
+  unsigned long long* giant;  // [M] bitmap snapshot: root of the F' component it marks
   int32_t* P1;
   int32_t* P2;
   int32_t* f1u;

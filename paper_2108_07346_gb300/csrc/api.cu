@@ -1397,7 +1397,8 @@ static int64_t articulation_fused_run(bridges_ctx* c, cudaStream_t s, const Laun
   }
   cudaMemsetAsync(k.status, 0, kClearBytes, s);
   cert_init(L, p, k.cert);
-  articulation_fused(L, p, k.cert, k.fin, b0, b1, fb, u, v, out_points, out_bridges, b1.count, bev, aev, chunks);
+  articulation_fused(L, p, k.cert, k.fin, b0, b1, fb, u, v, out_points, out_bridges, out_counts_device != nullptr,
+                     out_counts_device ? b1.count : c->h_pinned, bev, aev, chunks);
   if (bev) c->calls++;
   if (aev) c->ap_calls++;
   if (cudaGetLastError() != cudaSuccess) return BRIDGES_ECUDA;
@@ -1408,9 +1409,7 @@ static int64_t articulation_fused_run(bridges_ctx* c, cudaStream_t s, const Laun
       return cuda_fail(cudaGetLastError());
     return BRIDGES_OK;
   }
-  if (cudaMemcpyAsync(c->h_pinned, b1.count, sizeof(int64_t), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-      cudaStreamSynchronize(s) != cudaSuccess)
-    return cuda_fail(cudaGetLastError());
+  if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_fail(cudaGetLastError());
   return c->h_pinned[0];
 }
 

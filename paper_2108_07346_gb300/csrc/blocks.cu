@@ -353,26 +353,78 @@ __global__ void ap_mark_kernel(ApBufs b, int32_t V, const int32_t* status) {
 }
 
 constexpr int kCompactThreads = 1024;
-constexpr int kCompactItems = 4;  // flags per thread and tile
+constexpr int kCompactItems = 4;   // flags per thread and tile
+constexpr int kCompactTiles = 64;  // tiles that every block counts for itself (one launch)
 
-// Ordered compaction of the flagged vertices: per-tile counts, one-block scan, scatter.
+// Ordered compaction of the flagged vertices.  Up to kCompactTiles tiles one launch does it: every block
+// takes a tile and counts the flags before it by itself (a tile's 4,096 flags are 16 KB from L2), bound by
+// what one SM reads for the last tile.  Counting, scanning and scattering in launches of their own took
+// 15.6 us and two gaps on 37,147 vertices, this 9.2 us; it takes 20 us at 2^18 vertices and 44 at 2^20,
+// where the three launches take 22 and the gaps: so the line.
+__device__ __forceinline__ int32_t block_flags(const int32_t* flag, int64_t lo, int64_t hi, int32_t* red) {
+  // (flag and lo are multiples of 16 bytes: tiles of a 256-byte aligned array)
+  int32_t c = 0;
+  const int4* f4 = reinterpret_cast<const int4*>(flag + lo);
+  const int64_t n4 = (hi - lo) >> 2;
+#pragma unroll 8
+  for (int64_t i = threadIdx.x; i < n4; i += kCompactThreads) {
+    const int4 f = f4[i];
+    c += f.x + f.y + f.z + f.w;
+  }
+  for (int64_t x = lo + 4 * n4 + threadIdx.x; x < hi; x += kCompactThreads) c += flag[x];
+  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(kFull, c, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = c;
+  __syncthreads();
+  int32_t t = 0;
+  for (int w = 0; w < kCompactThreads / 32; w++) t += red[w];
+  return t;
+}
+
+// Writes the flagged vertices of one tile from out[at] on.
+__device__ __forceinline__ int32_t write_tile(const int32_t* flag, int64_t tile, int32_t V, int32_t at, int32_t* wsum,
+                                              int32_t* out) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int k = 0; k < kCompactItems; k++) {
+    const int64_t x = (tile * kCompactItems + k) * kCompactThreads + threadIdx.x;
+    const bool f = x < V && flag[x];
+    const unsigned m = __ballot_sync(kFull, f);
+    if (lane == 0) wsum[w] = __popc(m);
+    __syncthreads();
+    int32_t before = 0, total = 0;
+    for (int q = 0; q < kCompactThreads / 32; q++) {
+      if (q < w) before += wsum[q];
+      total += wsum[q];
+    }
+    if (f) out[at + before + __popc(m & lanemask_lt())] = (int32_t)x;
+    at += total;
+    __syncthreads();
+  }
+  return at;
+}
+
+// One block per tile; the last tile's block writes the number of points (or the status) to *count.
+__global__ void __launch_bounds__(kCompactThreads) ap_compact_kernel(ApBufs b, int32_t V, const int32_t* status,
+                                                                     int32_t* out, int64_t* count) {
+  __shared__ int32_t red[kCompactThreads / 32];
+  const int32_t st = *status;  // (no kernel sets it any more)
+  const int64_t tile = blockIdx.x, tile_sz = (int64_t)kCompactThreads * kCompactItems;
+  int32_t at = 0;
+  if (st == 0) {
+    at = block_flags(b.flag, 0, tile * tile_sz, red);
+    __syncthreads();
+    at = write_tile(b.flag, tile, V, at, red, out);
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *count = st ? (int64_t)st : (int64_t)at;
+}
+
+// The same for more tiles in three launches: per-tile counts, one-block scan, scatter.
 __global__ void ap_tile_count_kernel(ApBufs b, int32_t V, int64_t ntiles) {
   __shared__ int32_t red[kCompactThreads / 32];
   const int64_t tile_sz = (int64_t)kCompactThreads * kCompactItems;
   for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    int32_t c = 0;
-    for (int k = 0; k < kCompactItems; k++) {
-      const int64_t x = tile * tile_sz + k * kCompactThreads + threadIdx.x;
-      c += x < V ? b.flag[x] : 0;
-    }
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_down_sync(kFull, c, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int32_t t = 0;
-      for (int w = 0; w < kCompactThreads / 32; w++) t += red[w];
-      b.tiles[tile] = t;
-    }
+    const int32_t t = block_flags(b.flag, tile * tile_sz, min((int64_t)V, (tile + 1) * tile_sz), red);
+    if (threadIdx.x == 0) b.tiles[tile] = t;
     __syncthreads();
   }
 }
@@ -407,26 +459,8 @@ __global__ void ap_tile_scan_kernel(ApBufs b, int64_t ntiles, const int32_t* sta
 __global__ void ap_scatter_kernel(ApBufs b, int32_t V, int64_t ntiles, const int32_t* status, int32_t* out) {
   __shared__ int32_t wsum[kCompactThreads / 32];
   if (*status) return;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t tile_sz = (int64_t)kCompactThreads * kCompactItems;
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    int32_t at = b.tiles[tile];
-    for (int k = 0; k < kCompactItems; k++) {
-      const int64_t x = tile * tile_sz + k * kCompactThreads + threadIdx.x;
-      const bool f = x < V && b.flag[x];
-      const unsigned m = __ballot_sync(kFull, f);
-      if (lane == 0) wsum[w] = __popc(m);
-      __syncthreads();
-      int32_t before = 0, total = 0;
-      for (int q = 0; q < kCompactThreads / 32; q++) {
-        if (q < w) before += wsum[q];
-        total += wsum[q];
-      }
-      if (f) out[at + before + __popc(m & lanemask_lt())] = (int32_t)x;
-      at += total;
-      __syncthreads();
-    }
-  }
+  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x)
+    write_tile(b.flag, tile, V, b.tiles[tile], wsum, out);
 }
 
 // ---- the fused path: the certificate's stream and the block pass in one read of the list ----
@@ -692,6 +726,11 @@ void ap_finish(const Launch& L, const FinalBufs& f, const ApBufs& b, int32_t V, 
   const int bs = 256;
   const int64_t ntiles = ceil_div(std::max(V, 1), (int64_t)kCompactThreads * kCompactItems);
   ap_mark_kernel<<<grid_of(L, V, bs), bs, 0, L.stream>>>(b, V, f.status);
+  if (ntiles <= kCompactTiles) {
+    ap_compact_kernel<<<(unsigned)ntiles, kCompactThreads, 0, L.stream>>>(b, V, f.status, out, count_dev);
+    *L.launches += 2;
+    return;
+  }
   ap_tile_count_kernel<<<grid_of(L, ntiles * kCompactThreads, kCompactThreads), kCompactThreads, 0, L.stream>>>(
       b, V, ntiles);
   ap_tile_scan_kernel<<<1, kCompactThreads, 0, L.stream>>>(b, ntiles, f.status, count_dev);
@@ -850,7 +889,7 @@ FusedBufs carve_fused(void* base, int64_t E) {
 
 void articulation_fused(const Launch& L, const CertPlan& p, const CertBufs& cb, const FinalBufs& f, const ApBufs& b0,
                         const ApBufs& b1, const FusedBufs& fb, const int32_t* u, const int32_t* v, int32_t* out_points,
-                        int32_t* out_bridges, int64_t* count_dev, cudaEvent_t* bev, cudaEvent_t* aev,
+                        int32_t* out_bridges, bool count_bridges, int64_t* count_dev, cudaEvent_t* bev, cudaEvent_t* aev,
                         const ChunkSchedule& chunks) {
   const int32_t V = p.V;
   int32_t* cnt = cb.cnt;
@@ -860,9 +899,9 @@ void articulation_fused(const Launch& L, const CertPlan& p, const CertBufs& cb, 
   cudaMemsetAsync(fb.top, 0, sizeof(uint32_t) * (size_t)fb.ntop, L.stream);
   cert_warm(L, p, cb, u, v);
   if (bev) cudaEventRecord(bev[1], L.stream);
-  // T_0: F after the warm-up, rooted and numbered (the bridges of this partial certificate are
-  // not needed and go to dscan), then the classes of T_0 u F'
-  final_stage(L, f, V, cb.f1u, cb.f1v, cnt + 0, V, cb.f2u, cb.f2v, cnt + 1, V, cb.P1, f.dscan);
+  // T_0: F after the warm-up, rooted, numbered and tested (the bridges of this partial certificate are
+  // not needed, the subtree extrema are), then the classes of T_0 u F'
+  final_stage(L, f, V, cb.f1u, cb.f1v, cnt + 0, V, cb.f2u, cb.f2v, cnt + 1, V, cb.P1, nullptr, false, Upto::tested);
   ap_seed(L, f, b0, V, cb.f2u, cb.f2v, cnt + 1);
   if (aev) cudaEventRecord(aev[1], L.stream);
   cert_snapshot(L, p, cb);
@@ -902,8 +941,9 @@ void articulation_fused(const Launch& L, const CertPlan& p, const CertBufs& cb, 
   if (aev) cudaEventRecord(aev[3], L.stream);
   // the final certificate: its bridges and the final T (the barrier's count starts over)
   cudaMemsetAsync(f.bar_count, 0, sizeof(unsigned), L.stream);
-  final_stage(L, f, V, cb.f1u, cb.f1v, cnt + 0, V, cb.f2u, cb.f2v, cnt + 1, V, cb.P1,
-              out_bridges ? out_bridges : f.dscan);
+  // (its count and its sort only for a caller that wants them: the classes need the rooted forest alone)
+  final_stage(L, f, V, cb.f1u, cb.f1v, cnt + 0, V, cb.f2u, cb.f2v, cnt + 1, V, cb.P1, out_bridges, false,
+              out_bridges ? Upto::bridges : (count_bridges ? Upto::tested : Upto::rooted));
   if (bev) cudaEventRecord(bev[5], L.stream);
   const int bs = 256;
   const int g = grid_of(L, V, bs);

@@ -78,6 +78,7 @@ struct FinArgs {
   int kbits;
   int32_t sup_log;  // chunks per superchunk = kSuperChunks << sup_log
   int32_t ordered;  // trees in increasing order of their roots
+  int32_t upto;     // Upto: where final_kernel may stop
   unsigned bar_polls;  // polls a barrier waits before it gives up
   int32_t hold_polls;  // > 0: the last block sleeps this many ~100 ns polls before its first barrier
 };
@@ -543,6 +544,7 @@ __device__ bool forest_bridges(const FinArgs& A, int32_t* sm, int32_t* red, unsi
       return p;
     };
     for (int64_t x = gspread(); x < V; x += gstride()) f.pre[x] = preorder((int32_t)x);
+    if (!RED && A.upto == (int32_t)Upto::rooted) return true;
     for (int64_t e = gspread(); e < nx; e += gstride()) {
       const int32_t a = A.xu[e], b = A.xv[e];
       if ((uint32_t)a >= (uint32_t)V || (uint32_t)b >= (uint32_t)V) {
@@ -925,8 +927,9 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
   if (!may_start(A)) return;
   if (gtid() == 0) *A.f.nkeys = 0;
   if (!forest_bridges<false>(A, sm, red, &bar_epoch)) return;
+  if (A.upto == (int32_t)Upto::rooted) return;
   if (!grid_barrier(A.f, A.bar_polls, &bar_epoch)) return;
-  if (!sort_keys(A, nullptr, -1, sm, red, &bar_epoch)) return;
+  if (A.upto == (int32_t)Upto::bridges && !sort_keys(A, nullptr, -1, sm, red, &bar_epoch)) return;
   write_count(A);
 }
 
@@ -1472,7 +1475,7 @@ bool final_prepare() {
 
 void final_stage(const Launch& L, const FinalBufs& f, int32_t V, const int32_t* tu, const int32_t* tv,
                  const int32_t* d_nt, int64_t cap_tree, const int32_t* xu, const int32_t* xv, const int32_t* d_nx,
-                 int64_t cap_extra, const int32_t* P_tree, int32_t* out, bool ordered) {
+                 int64_t cap_extra, const int32_t* P_tree, int32_t* out, bool ordered, Upto upto) {
   size_t smem = 0;
   FinArgs A = final_args(L, f, V, out, &smem);
   A.tu = tu;
@@ -1485,6 +1488,7 @@ void final_stage(const Launch& L, const FinalBufs& f, int32_t V, const int32_t* 
   A.cx = (int32_t)std::min<int64_t>(cap_extra, INT32_MAX);
   A.P_tree = P_tree;
   A.ordered = ordered ? 1 : 0;
+  A.upto = (int32_t)upto;
   void* args[] = {&A};
   launch_final(L, (const void*)final_kernel, V, smem, args);
 }

@@ -195,6 +195,9 @@ void two_edge_components(const Launch& L, const FinalBufs& fb, const CertBufs& c
 // Offers n extra edges to partition 0's union-finds (its certificate grows to a certificate of
 // the union).  Ids are range-checked first; on ERANGE nothing is changed.
 void cert_offer(const Launch& L, const CertPlan& p, const CertBufs& b, const int32_t* u, const int32_t* v, int64_t n);
+// What a caller of final_stage reads: the rooted forest alone (pre, par, sz, root; no count), that and the
+// subtree extrema and bridge flags and their count, or all of it and the sorted pairs.
+enum class Upto { rooted, tested, bridges };
 // Bridges of T u X (T a spanning forest of every tree it touches, X edges inside trees).
 // Counts on device.  P_tree: union-find of T (roots = minimum vertex), or null to build it.
 // ordered: trees take consecutive preorder ranges in increasing order of their roots (otherwise
@@ -202,7 +205,7 @@ void cert_offer(const Launch& L, const CertPlan& p, const CertBufs& b, const int
 void final_stage(const Launch& L, const FinalBufs& fb, int32_t V, const int32_t* tu, const int32_t* tv,
                  const int32_t* d_ntree, int64_t cap_tree, const int32_t* xu, const int32_t* xv,
                  const int32_t* d_nextra, int64_t cap_extra, const int32_t* P_tree, int32_t* out,
-                 bool ordered = false);
+                 bool ordered = false, Upto upto = Upto::bridges);
 
 // The bridges of job 0's certificate alone, sorted to out, their number to fb.count: the final stage of
 // calls that need no rooted forest.  Flattens P2; fb.bflag[e] tells whether F edge e is a bridge.
@@ -232,7 +235,7 @@ size_t fused_bytes(int64_t E);
 FusedBufs carve_fused(void* base, int64_t E);
 void articulation_fused(const Launch& L, const CertPlan& p, const CertBufs& cb, const FinalBufs& f, const ApBufs& b0,
                         const ApBufs& b1, const FusedBufs& fb, const int32_t* u, const int32_t* v, int32_t* out_points,
-                        int32_t* out_bridges, int64_t* count_dev, cudaEvent_t* bev, cudaEvent_t* aev,
+                        int32_t* out_bridges, bool count_bridges, int64_t* count_dev, cudaEvent_t* bev, cudaEvent_t* aev,
                         const ChunkSchedule& chunks);
 
 inline int64_t ceil_div(int64_t a, int64_t b) { return (a + b - 1) / b; }

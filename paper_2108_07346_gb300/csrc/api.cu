@@ -50,7 +50,7 @@ struct Carved {
 // The launch context of a call on c: its stream, its launch counter and the final stage's test
 // knobs from the options (zero in normal use).
 Launch launch_for(bridges_ctx* c, cudaStream_t s) {
-  Launch L{s, &c->launches, c->num_sms, c->smem_optin};
+  Launch L{s, &c->launches, c->num_sms, c->smem_optin, c->share};
   L.bar_polls = c->opts.test_barrier_polls > 0 ? (unsigned)c->opts.test_barrier_polls : 0u;
   L.hold_polls = c->opts.test_hold_polls > 0 ? c->opts.test_hold_polls : 0;
   return L;
@@ -171,6 +171,7 @@ int init_ctx(bridges_ctx* c, int device, const bridges_opts* opts) {
   if (!opts) c->opts.warm_edges = -1;
   if (cudaSetDevice(device) != cudaSuccess) return -1;
   cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device);
+  c->share = c->num_sms;
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
   c->smem_optin = (size_t)optin;

@@ -22,6 +22,9 @@ struct bridges_ctx {
   int64_t* h_pinned = nullptr;  // pinned host scratch (counts)
   bridges_opts opts{};
   int num_sms = 0;
+  // blocks of the next call's cooperative kernels at most: one per SM, or a server's share while other
+  // requests are in flight (set by its scheduler, the context's one user)
+  int share = 0;
   size_t smem_optin = 0;
   int64_t launches = 0;
   int64_t allocs = 0;  // device allocations of the context's own buffers since its options were set

@@ -1459,7 +1459,8 @@ FinArgs final_args(const Launch& L, const FinalBufs& f, int32_t V, int32_t* out,
 // other streams (the server).
 void launch_final(const Launch& L, const void* kernel, int32_t V, size_t smem, void** args) {
   const int64_t want = ceil_div(2 * (int64_t)std::max(V, 1), kThreads);
-  const int blocks = (int)std::min<int64_t>({(int64_t)kMaxBlocks, want, (int64_t)L.num_sms});
+  const int64_t most = std::max<int64_t>(L.coop_blocks, want / 8);  // a share, or eight elements a thread
+  const int blocks = (int)std::min<int64_t>({(int64_t)kMaxBlocks, want, most, (int64_t)L.num_sms});
   cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(kThreads), args, smem, L.stream);
   *L.launches += 1;
 }

@@ -29,6 +29,7 @@ struct Launch {
   int64_t* launches;
   int num_sms;
   size_t smem_optin;  // max dynamic shared memory per block
+  int coop_blocks;    // blocks of a cooperative kernel at most: one per SM, or a share of them
   // test knobs of the final stage (bridges_opts.test_barrier_polls / test_hold_polls); zero in
   // normal use
   unsigned bar_polls = 0;  // polls a grid barrier waits before it gives up (0: the default cap)

@@ -97,7 +97,7 @@ extern "C" int64_t bridges_find_noalloc(struct CUstream_st* stream, const int32_
   cb.roots = fb.sr2;
   fb.bar_count = reinterpret_cast<unsigned*>(base + 128);  // in the cleared page, beside the status word
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  Launch L{s, &S->launches, S->num_sms, S->smem_optin};
+  Launch L{s, &S->launches, S->num_sms, S->smem_optin, S->num_sms};
   // a graph of at most one vertex has no pairs to write; its output pointer may be null, so the
   // stage gets a slot of the scratch array instead (a device address, never a host one)
   int32_t* spare_out = reinterpret_cast<int32_t*>(base + kSpareOut);

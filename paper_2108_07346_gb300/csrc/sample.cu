@@ -378,9 +378,11 @@ void cert_sample(const Launch& L, const CertPlan& p, const CertBufs& b, const in
     return;
   }
   // one thread per sampled edge and per vertex, at most one block per SM (fewer blocks make the
-  // barriers cheaper), at most 8 edges a thread (the plan keeps the sample below that)
+  // barriers cheaper) or per SM of the call's share, at most 8 edges a thread (the plan keeps the
+  // sample below that for all SMs; a share takes more blocks if it must)
   const int64_t work = std::max<int64_t>({a.groups * kGroup, (int64_t)p.V, 1});
-  const int blocks = (int)std::min<int64_t>(ceil_div(work, kThreads), L.num_sms);
+  const int64_t most = std::max<int64_t>(L.coop_blocks, ceil_div(a.groups, kThreads));
+  const int blocks = (int)std::min<int64_t>({ceil_div(work, kThreads), most, (int64_t)L.num_sms});
   const int64_t per = ceil_div(a.groups * kGroup, (int64_t)blocks * kThreads);
   a.first = (int32_t)std::min<int64_t>(8, ceil_div(2 * (int64_t)std::max(p.V, 1), (int64_t)blocks * kThreads));
   if (per <= 1)

@@ -829,6 +829,9 @@ __device__ bool sort_keys(const FinArgs& A, const int32_t* ko, int32_t listed, i
     uint32_t(*const wcnt)[256] = reinterpret_cast<uint32_t(*)[256]>(sm);  // [kWarps][256]
     uint32_t* const run = reinterpret_cast<uint32_t*>(sm) + kWarps * 256;   // [256]
     const int passes = (2 * A.kbits + 7) / 8;
+    // Every block sums the blocks' histograms to its own digits' places (155 KB from L2), so that a pass has
+    // two barriers.  With the places from a grid-wide scan it has four: 140 k keys of 40 bits, five passes,
+    // took 66 us, 47 so.
     const int64_t lo = min((int64_t)n, per * (int64_t)blockIdx.x), hi = min((int64_t)n, lo + per);
     uint64_t* src = f.keys;
     uint64_t* dst = f.keys2;
@@ -839,13 +842,32 @@ __device__ bool sort_keys(const FinArgs& A, const int32_t* ko, int32_t listed, i
       __syncthreads();
       for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) atomicAdd(&run[(src[i] >> shift) & 255], 1u);
       __syncthreads();
-      if (threadIdx.x < 256) f.hist[(int64_t)threadIdx.x * gridDim.x + blockIdx.x] = (int32_t)run[threadIdx.x];
+      if (threadIdx.x < 256) f.hist[(int64_t)blockIdx.x * 256 + threadIdx.x] = (int32_t)run[threadIdx.x];
       BARRIER();
-      if (!grid_scan(f, A.bar_polls, bar_epoch, f.hist, f.hist, nullptr, nullptr, (int64_t)256 * gridDim.x, red)) return false;
-      BARRIER();
-      if (threadIdx.x < 256) {
-        run[threadIdx.x] = (uint32_t)f.hist[(int64_t)threadIdx.x * gridDim.x + blockIdx.x];
-        for (int w = 0; w < kWarps; w++) wcnt[w][threadIdx.x] = 0;
+      {
+        const int d = threadIdx.x & 255, q = threadIdx.x >> 8;
+        uint32_t total = 0, before = 0;
+#pragma unroll 8
+        for (int b = q; b < (int)gridDim.x; b += kThreads / 256) {
+          const uint32_t c = (uint32_t)__ldcg(f.hist + (int64_t)b * 256 + d);
+          total += c;
+          if (b < (int)blockIdx.x) before += c;
+        }
+        wcnt[2 * q][d] = total;
+        wcnt[2 * q + 1][d] = before;
+        __syncthreads();
+        total = before = 0;
+        if (q == 0)
+          for (int k = 0; k < kThreads / 256; k++) {
+            total += wcnt[2 * k][d];
+            before += wcnt[2 * k + 1][d];
+          }
+        int32_t all;
+        const int32_t smaller = block_excl((int32_t)total, red, &all);  // (its barriers: wcnt has been read)
+        if (q == 0) {
+          run[d] = (uint32_t)smaller + before;
+          for (int w = 0; w < kWarps; w++) wcnt[w][d] = 0;
+        }
       }
       __syncthreads();
       for (int64_t t0 = lo; t0 < hi; t0 += blockDim.x) {  // stable: chunk, warp, lane = index order
@@ -952,7 +974,7 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
 //      most kCoreMax vertices, else by every block: a spanning forest of it, then the phases above.
 //   5  The keys are sorted, as above.
 // 2.5 M edges on 37,147 vertices: 79 us with the phases above on the whole forest, 27 us so; 16.8 M
-// R-MAT edges on 2^20 vertices (141 k kept edges, 140.1 k of them bridges): 417 and 177 us.
+// R-MAT edges on 2^20 vertices (141 k kept edges, 140.1 k of them bridges): 417 and 156 us.
 
 struct ReducedArgs {
   FinArgs a;          // a.V: the graph's vertices; tu, tv, d_nt: F; kbits, sup_log, bar_polls, hold_polls

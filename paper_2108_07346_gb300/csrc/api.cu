@@ -26,7 +26,7 @@ constexpr size_t kMiscBytes = 1024;  // status word, device counts of bridges_fr
 constexpr int64_t kSmallCallEdges = 22528;  // a whole call on one block up to this many edges
 constexpr size_t kClearBytes = kMiscBytes + 256;  // cleared at a call's start: the misc area and the
                                                   // certificate's control words, which follow it
-constexpr size_t kBarAt = 128;       // the final stage's barrier count
+constexpr size_t kBarAt = 128;       // the final stage's barrier count; the reduced stage's counters at 768
 constexpr size_t kSpareAt = 512;     // the spare output slot: where a call that has no pairs or points
                                      // to write (V <= 1, null output) points the stages
 

@@ -961,11 +961,12 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
 // one 2-edge-connected component: contracting the F' components changes no bridge, and the edges that are
 // left all come from F (s_contract, smem.cuh, does the same for small graphs).  Dense graphs keep only
 // their sparse fringe: 4,443 vertices of 37,147, 8.3 k of 73,719.
-//   1  P2 flattened: every vertex's F' root.
-//   2  F edges between two roots are kept; the roots are numbered as they are met, and the trees of F that
-//      kept edges lie in counted.  If the kept edges number the roots less the trees, the reduced graph is
-//      a forest and all of them are bridges.  If they are many more than the roots (a sparse graph with
-//      cycles throughout), the reduction gained little and the phases above run on F and F' as they are.
+//   1  P2 flattened: every vertex's F' root.  F edges between two roots are kept.
+//   2  F' has V - |F'| components and F has V - |F|, each of them some whole ones of F': the reduced graph's
+//      spanning forests have |F| - |F'| edges.  If the kept edges are that many, it is a forest and all of
+//      them are bridges.  If they are many more (a sparse graph with cycles throughout), the reduction
+//      gained little and the phases above run on F and F' as they are.  Else the roots with kept edges are
+//      numbered.
 //   3  Else leaves are stripped.  The one edge of a vertex of degree 1 is a bridge; without it its other
 //      end may be the next leaf, and the thread goes on there (at most kStripSteps times, so that a long
 //      path does not run in one thread; vertices of kHub edges and more keep their degree, so that their
@@ -973,8 +974,9 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
 //   4  What is left, the cycles and what joins them, is solved by block 0 in shared memory when it has at
 //      most kCoreMax vertices, else by every block: a spanning forest of it, then the phases above.
 //   5  The keys are sorted, as above.
-// 2.5 M edges on 37,147 vertices: 79 us with the phases above on the whole forest, 27 us so; 16.8 M
-// R-MAT edges on 2^20 vertices (141 k kept edges, 140.1 k of them bridges): 417 and 156 us.
+// 2.5 M edges on 37,147 vertices: 79 us with the phases above on the whole forest, 18 us so (25 with the
+// roots numbered before it was known that all kept edges are bridges); 16.8 M R-MAT edges on 2^20 vertices
+// (141 k kept edges, 140.1 k of them bridges): 417 and 156 us.
 
 struct ReducedArgs {
   FinArgs a;          // a.V: the graph's vertices; tu, tv, d_nt: F; kbits, sup_log, bar_polls, hold_polls
@@ -986,10 +988,11 @@ struct ReducedArgs {
   int32_t* tmp;       // [V] scratch
 };
 
-// counters behind f.nroots (one page)
+// counters behind the barrier's, cleared with it before the launch, in a line of their own (appends beside
+// the word that waiting blocks poll: 4 us more for 141 k kept edges)
+constexpr int kCntAt = 160;
 constexpr int kCntVerts = 1;  // reduced vertices
 constexpr int kCntKept = 2;   // kept edges
-constexpr int kCntTrees = 3;  // trees of F with kept edges
 constexpr int kCoreVerts = 4;
 constexpr int kCoreEdges = 5;
 constexpr int kCntTree = 6;
@@ -1132,7 +1135,6 @@ __global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
   const int lane = threadIdx.x & 31;
   if (!may_start(A)) return;
   int32_t* const id = f.pre;    // a root's number
-  int32_t* const tree = f.head; // a tree's (its root's in F)
   int32_t* const deg = f.sz;    // by number
   int32_t* const inc = f.slo;
   int32_t* const id2 = f.hi;    // a core vertex's number
@@ -1143,11 +1145,13 @@ __global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
   int32_t* const cu = reinterpret_cast<int32_t*>(f.sr2);
   int32_t* const cv = cu + V;
   int32_t* const cs = cv + V;
-  // 1: flat F' roots
+  int32_t* const cnt = reinterpret_cast<int32_t*>(f.bar_count) + kCntAt;
+  // 1: flat F' roots; kept edges.  Up to a vertex or so per thread the edges' ends look their roots up
+  // themselves, while other threads flatten: a barrier between the two took 2 us more (37,147 vertices).
+  // With many more the lookups are bound by their L2 sectors, and flat roots need one each.
   for (int64_t x = gspread(); x < V; x += gstride()) {
     R.P2[x] = uf_root_static(R.P2, (int32_t)x);
     id[x] = -1;
-    tree[x] = -1;
     id2[x] = -1;
     deg[x] = 0;
     inc[x] = 0;
@@ -1155,51 +1159,33 @@ __global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
     f.P[x] = (int32_t)x;
     f.bflag[x] = 0;
   }
-  if (gtid() < 8) f.nroots[gtid()] = 0;
-  if (gtid() == 8) *f.nkeys = 0;
-  if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
-  // 2: kept edges.  With more F edges than two per thread they are listed first and numbered after a
-  // barrier, one per thread: the numbering is a chain of accesses, and a thread's edges would queue.
-  const int32_t nt = min(*A.d_nt, A.ct);
-  const bool list_first = nt > 2 * gstride();
-  auto number = [&](bool has, int32_t ra, int32_t rb, int32_t t) {
-    number_once<3>(has, {ra, rb, t}, {id, id, tree}, {f.nroots + kCntVerts, f.nroots + kCntVerts, f.nroots + kCntTrees});
-  };
+  if (gtid() == 0) *f.nkeys = 0;
+  const int32_t nt = min(*A.d_nt, A.ct), nx = min(*R.d_nx, V);
+  if (V > 2 * gstride() && !grid_barrier(f, A.bar_polls, &bar_epoch)) return;
   for (int64_t base = gspread() & ~31LL; base < nt; base += gstride()) {
     const int64_t e = base + lane;
-    int32_t ra = -1, rb = -1, t = -1;
+    int32_t ra = -1, rb = -1;
     if (e < nt) {
       const int32_t a = A.tu[e], b = A.tv[e];
       if ((uint32_t)a >= (uint32_t)V || (uint32_t)b >= (uint32_t)V) {
         set_status(f.status, BRIDGES_EINTERNAL_CODE);
       } else {
-        ra = R.P2[a];
-        rb = R.P2[b];
-        if (ra != rb && !list_first) t = uf_root_static(R.P1, a);
+        ra = uf_root_static(R.P2, a);
+        rb = uf_root_static(R.P2, b);
       }
     }
     const bool keep = ra != rb;
-    if (!__any_sync(kFull, keep)) continue;
-    const int32_t at = warp_place(keep, f.nroots + kCntKept);
+    const int32_t at = warp_place(keep, cnt + kCntKept);
     if (keep) {
       ku[at] = ra;
       kv[at] = rb;
       ko[at] = (int32_t)e;
     }
-    if (!list_first) number(keep, ra, rb, t);
-  }
-  if (list_first) {
-    if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
-    const int32_t m = f.nroots[kCntKept];
-    for (int64_t base = gspread() & ~31LL; base < m; base += gstride()) {
-      const int64_t i = base + lane;
-      const bool in = i < m;
-      number(in, in ? ku[i] : 0, in ? kv[i] : 0, in ? uf_root_static(R.P1, A.tu[ko[i]]) : 0);
-    }
   }
   if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
-  const int32_t kept = f.nroots[kCntKept], verts = f.nroots[kCntVerts];
-  if (kept == verts - f.nroots[kCntTrees]) {
+  // 2
+  const int32_t kept = cnt[kCntKept], span = nt - nx;
+  if (kept == span) {
     // a forest: every kept edge is a bridge, listed by its place
     if (kept <= kRankMax) {
       if (!sort_keys(A, ko, kept, sm, red, &bar_epoch)) return;
@@ -1212,7 +1198,7 @@ __global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
     write_count(A);
     return;
   }
-  if (kept > kCyclicMin && kept > verts + verts / 4) {
+  if (kept > kCyclicMin && kept > span + span / 4) {
     FinArgs B = A;
     B.orig = nullptr;
     B.ou = A.tu;
@@ -1228,6 +1214,13 @@ __global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
     write_count(A);
     return;
   }
+  for (int64_t base = gspread() & ~31LL; base < kept; base += gstride()) {
+    const int64_t i = base + lane;
+    const bool in = i < kept;
+    number_once<2>(in, {in ? ku[i] : 0, in ? kv[i] : 0}, {id, id}, {cnt + kCntVerts, cnt + kCntVerts});
+  }
+  if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
+  const int32_t verts = cnt[kCntVerts];
   // 3: degrees, then the strip
   for (int64_t base = gspread() & ~31LL; base < kept; base += gstride()) {
     const int64_t i = base + lane;
@@ -1266,14 +1259,14 @@ __global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
     const int32_t at = warp_place(bridge, f.nkeys);
     if (bridge) f.keys[at] = kSlotTag | (uint64_t)i;
     if (!__any_sync(kFull, core)) continue;
-    const int32_t ct = warp_place(core, f.nroots + kCoreEdges);
+    const int32_t ct = warp_place(core, cnt + kCoreEdges);
     if (core) cs[ct] = (int32_t)i;
     number_once<2>(core, {core ? cu[i] : 0, core ? cv[i] : 0}, {id2, id2},
-                   {f.nroots + kCoreVerts, f.nroots + kCoreVerts});
+                   {cnt + kCoreVerts, cnt + kCoreVerts});
   }
   if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
   // 4
-  const int32_t VC = f.nroots[kCoreVerts], mc = f.nroots[kCoreEdges];
+  const int32_t VC = cnt[kCoreVerts], mc = cnt[kCoreEdges];
   if (mc > 0 && VC <= kCoreMax) {
     if (blockIdx.x == 0) solve_core(R, reinterpret_cast<char*>(sm), gs, id2, cu, cv, cs, VC, mc);
     if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
@@ -1298,8 +1291,8 @@ __global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
         b = id2[cv[slot]];
       }
       const bool joins = live && uf_link(f.P, a, b);
-      const int32_t at = warp_place(joins, f.nroots + kCntTree);
-      const int32_t xt = warp_place(live && !joins, f.nroots + kCntRest);
+      const int32_t at = warp_place(joins, cnt + kCntTree);
+      const int32_t xt = warp_place(live && !joins, cnt + kCntRest);
       if (joins) {
         tu[at] = a;
         tv[at] = b;
@@ -1311,17 +1304,17 @@ __global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
     }
     if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
     FinArgs B = A;
-    const int32_t nx = f.nroots[kCntRest];
+    const int32_t nx = cnt[kCntRest];
     B.V = VC;
     B.orig = R.tmp;
     B.ou = A.tu;
     B.ov = A.tv;
     B.tu = tu;
     B.tv = tv;
-    B.d_nt = f.nroots + kCntTree;
+    B.d_nt = cnt + kCntTree;
     B.xu = tu + (V - nx);
     B.xv = tv + (V - nx);
-    B.d_nx = f.nroots + kCntRest;
+    B.d_nx = cnt + kCntRest;
     B.cx = V;
     B.P_tree = f.P;
     if (!forest_bridges<true>(B, sm, red, &bar_epoch)) return;

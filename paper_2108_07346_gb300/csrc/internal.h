@@ -81,7 +81,8 @@ struct CertBufs {
 struct FinalBufs {
   int32_t* status;
   int64_t* count;  // [1] receives the bridges found (written only; device or mapped host memory)
-  unsigned* bar_count;  // grid barrier: arrivals (grows within a launch; cleared by the caller before it)
+  unsigned* bar_count;  // grid barrier: arrivals (grows within a launch; cleared by the caller before it;
+                        // reduced_stage: with the 191 words behind it, where it counts)
   int32_t* nroots;  // [1] trees of the forest (one-vertex trees included)
   int32_t* P;      // [V] union-find over the tree (built by the stage when it owns it)
   int32_t* root;   // [V] root (minimum vertex) of each vertex's tree

@@ -19,6 +19,8 @@
 #include <unordered_map>
 #include <vector>
 
+#include <sys/prctl.h>
+
 #include "../../include/bridges.h"
 #include "batched.h"
 #include "ctx.h"
@@ -81,8 +83,11 @@ namespace {
 // request alone takes all.
 constexpr int kShare = 4;
 
-// Launches queued work on free slots.  Caller holds mu.
-void admit(bridges_server* S) {
+// Launches queued work on free slots.  Caller holds mu (lk); it is released while a request's work is
+// enqueued, about 9 us of calls, so that submissions do not wait behind it: what admit uses meanwhile, the
+// slots and the tickets it has taken off the queue (no longer cancelable, not collected before they are
+// done), nobody else touches.
+void admit(bridges_server* S, std::unique_lock<std::mutex>& lk) {
   int busy = 0;
   for (const SrvSlot& sl : S->slots) busy += sl.busy;
   for (SrvSlot& sl : S->slots) {
@@ -102,8 +107,9 @@ void admit(bridges_server* S) {
       q.t_start = now_s();
       sl.tickets.push_back(t);
       sl.reserved = q.ws;
-      rc = run_single(sl.ctx, sl.stream, q.r.edges_u, q.r.edges_v, q.r.E, q.r.V, q.r.M, q.r.out_bridges, sl.d_counts);
-      S->stats[2]++;
+      const bridges_request r = q.r;
+      lk.unlock();
+      rc = run_single(sl.ctx, sl.stream, r.edges_u, r.edges_v, r.E, r.V, r.M, r.out_bridges, sl.d_counts);
     } else {
       // gather the oldest small requests; large ones keep their place in the queue
       std::vector<BatchTask> graphs, tasks;
@@ -132,15 +138,17 @@ void admit(bridges_server* S) {
       }
       if (graphs.empty()) return;  // only large requests wait, and the head does not fit yet
       sl.reserved = 0;
+      lk.unlock();
       const int64_t slot_words = plan_batch_tasks(sl.ctx, graphs, total_e, tasks);
       rc = launch_batch_tasks(sl.ctx, sl.stream, tasks, (int32_t)graphs.size(), slot_words);
-      S->stats[1]++;
     }
     if (rc == BRIDGES_OK &&
         cudaMemcpyAsync(sl.h_counts, sl.d_counts, sizeof(int64_t) * sl.tickets.size(), cudaMemcpyDeviceToHost,
                         sl.stream) != cudaSuccess)
       rc = BRIDGES_ECUDA;
     if (rc == BRIDGES_OK && cudaEventRecord(sl.ev, sl.stream) != cudaSuccess) rc = BRIDGES_ECUDA;
+    lk.lock();
+    S->stats[take_large ? 2 : 1]++;
     if (rc != BRIDGES_OK) {
       // the requests fail; the slot stays free
       cudaGetLastError();
@@ -191,11 +199,12 @@ bool retire(bridges_server* S) {
 
 void scheduler(bridges_server* S) {
   cudaSetDevice(S->device);
+  prctl(PR_SET_TIMERSLACK, 1000);  // this thread's short waits end on time (by default 50 us late or more)
   std::unique_lock<std::mutex> lk(S->mu);
   while (true) {
     const bool finished = retire(S);
     if (finished) S->cv_done.notify_all();
-    admit(S);
+    admit(S, lk);
     bool busy = false;
     for (const SrvSlot& sl : S->slots) busy = busy || sl.busy;
     if (S->stop && !busy && S->queue.empty()) break;

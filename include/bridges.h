@@ -62,8 +62,12 @@ typedef struct bridges_opts {
   int32_t fan_in;      /* certificates merged per merge job; <= 1: auto (Sec. 3 uses 2) */
   int32_t block;       /* threads per block of the forest pass; 0: auto */
   int32_t ctas_per_sm; /* resident blocks per SM for the forest pass; 0: auto */
-  int64_t warm_edges;  /* edges per partition certified before the label snapshot;
-                          < 0: auto, 0: never snapshot (every edge takes the union-find path) */
+  int64_t warm_edges;  /* edges per partition certified before the label snapshot: with one partition
+                          and labels a sample of the whole list (at most 8,192 per SM), else a prefix
+                          of each partition; < 0: auto, 0: never snapshot (every edge takes the
+                          union-find path).  A call for the bridges of at most 22,528 edges on
+                          2 to 4,096 vertices in one partition, warm_edges not 0, runs on one block
+                          with no snapshot */
   int32_t profile;     /* 1: record per-stage CUDA events on the launch stream */
   int32_t host_read;   /* bridges_find_host: 1 = when the host buffers are pinned and mapped,
                           kernels read them in place over the host link instead of copying
@@ -73,7 +77,8 @@ typedef struct bridges_opts {
                             none with the bitmap that larger V takes), > 0: that many, < 0: none
                             (snapshot right after the certificate's own edges) */
   int32_t warm_block;    /* threads per block of the forest pass's warm-up launch (the prefix certified
-                            through the union-finds before the snapshot); 0: auto */
+                            through the union-finds before the snapshot; no effect on a sample);
+                            0: auto */
   int32_t ap_fused;      /* bridges_articulation_points: 0 = auto (one read of the list for the
                             certificate and the block pass when the plan is one partition with a
                             16-bit label snapshot and the larger workspace of that form fits the
@@ -228,7 +233,8 @@ int32_t bridges_batch_autotune(bridges_ctx* ctx, struct CUstream_st* stream, con
  * A request is a graph whose edge arrays are already resident on the device; the caller keeps
  * edges_u / edges_v / out_bridges valid until the request completes.  A scheduler thread keeps
  * up to max_slots units of work in flight, each on its own stream and workspace, so requests
- * overlap on the device.  Queued small graphs (V <= 4096) are gathered into one batched launch
+ * overlap on the device (while others wait or run, a request's cooperative kernels take a share
+ * of the SMs).  Queued small graphs (V <= 4096) are gathered into one batched launch
  * (as bridges_find_batched); a large graph runs the single-graph path once its workspace fits
  * in what mem_budget_bytes has left.  The budget counts the workspaces of the single-graph
  * requests running at the time; a slot keeps the workspace it grew to, and batched buffers are

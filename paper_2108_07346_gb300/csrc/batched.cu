@@ -1,4 +1,5 @@
-// batched.cu -- many small graphs in two persistent launches.
+// batched.cu -- many small graphs in two persistent launches, and the one-block kernels of single
+// small graphs.
 //
 // Certification (certify_kernel): four 256-thread groups per block take tasks from a queue with
 // two ends (most edges first; one group per block starts with the fewest).  A task is a whole
@@ -11,13 +12,13 @@
 // stage's shared-memory layout and its bridge stage runs right there, beside the other groups'
 // streams.
 //
-// Bridges (bridge_kernel), for the larger graphs: per graph, a group copies its certificate from
-// its slot (one task) or offers the F then F' edges of every one of the graph's slots to fresh
-// union-finds in shared memory (several: the Sec. 3 merge with fan-in = the number of partitions)
-// and runs the bridge stage.  The stage is the same Euler-tour / preorder-range test as final.cu,
-// on 16-bit arrays with barriers between phases (list ranking by a ruling set, subtree ranges
-// from shuffle windows and chunk extrema), then a rank sort of the packed (a << 12 | b) keys
-// (bitonic above the group's thread count).  A graph's fixed cost is its barriers, so graphs of
+// Bridges (bridge_kernel), for the larger graphs: per graph, a group copies F and the roots of F' from
+// the first task's slot, offers the other tasks' edges (several: the Sec. 3 merge with fan-in = the
+// number of partitions) and runs the bridge stage.  The stage contracts the F' components first
+// (s_contract: what is left of a dense graph is a small fringe); if cycles are left it is the same
+// Euler-tour / preorder-range test as final.cu, on 16-bit arrays with barriers between phases (list
+// ranking by a ruling set, subtree ranges from shuffle windows and chunk extrema); then a rank sort
+// of the packed (a << 12 | b) keys (bitonic above the group's thread count).  A graph's fixed cost is its barriers, so graphs of
 // up to 3,008 vertices run two per block: the block splits into 512-thread groups with their own
 // half of shared memory and their own named barrier, so that one graph's barrier waits overlap
 // with the other's work.  Nothing waits on another block, so there is no spin anywhere.

@@ -14,7 +14,9 @@
 //
 // Dense partitions become one giant component after about V ln V edges, after which nearly all
 // edges are rejected by both forests.  To reject those from shared memory, each job first
-// certifies a warm-up prefix of its chunk through the union-finds, then takes a snapshot: a
+// certifies some of its chunk -- one partition a sample of the whole list, in rounds (sample.cu);
+// several, or more vertices than labels, a prefix of the chunk through the union-finds -- and
+// takes a snapshot: a
 // 16-bit label per vertex naming its F' component (components with >= 2 vertices, up to 65,535
 // of them).  F' components nest inside F components (every F' edge joins two ends F already
 // joined), so two vertices with equal labels are joined in both forests and their edge can be

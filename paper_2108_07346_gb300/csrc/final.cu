@@ -9,10 +9,13 @@
 // the range -- the same test as Alg. 1's low[v] > disc[u], evaluated for all tree edges at once
 // (Tarjan 1974; Tarjan & Vishkin 1985).
 //
-// The whole stage is ONE cooperative kernel (every block resident) whose phases are separated
-// by a software grid barrier; the work per phase is small (O(V)), so launch overhead, not
-// bandwidth, would dominate a kernel-per-phase design, and the barriers (about 1.9 us each)
-// dominate the kernel: the phases are arranged to need few of them.
+// A call that wants the rooted forest runs all of this as one cooperative kernel (final_kernel, every
+// block resident); one that wants only the bridges first contracts the components of F'
+// (reduced_kernel, below), after which a dense graph is a forest, or a small rest solved by one
+// block, and only a sparse graph with cycles throughout comes back to these phases.  They are
+// separated by a software grid barrier; the work per phase is small (O(V)), so launch overhead, not
+// bandwidth, would dominate a kernel-per-phase design, and the barriers (1.3 to 3 us with the
+// stores before them) dominate the kernel: the phases are arranged to need few of them.
 //   * Arc lists: tree edge e gives arcs 2e (tu -> tv) and 2e+1 (tv -> tu), twins by i ^ 1; each
 //     arc is pushed on its tail's list with one atomic exchange (no degree count, scan or
 //     placement pass).

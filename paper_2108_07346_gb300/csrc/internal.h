@@ -77,7 +77,7 @@ struct CertBufs {
   int64_t Vpad;  // stride of lab
 };
 
-// Device buffers of the final stage (Euler tour, ranges, test, sort), one cooperative kernel.
+// Device buffers of the final stage (reduced graph, Euler tour, ranges, test, sort), one cooperative kernel.
 struct FinalBufs {
   int32_t* status;
   int64_t* count;  // [1] receives the bridges found (written only; device or mapped host memory)

@@ -1052,16 +1052,14 @@ __device__ __forceinline__ void number_once(bool has, const int32_t (&r)[N], int
   }
 }
 
-// Adds edge `slot` to its end x's degree and to the xor of x's edges (lanes with one end together).
-__device__ __forceinline__ void add_edge_end(bool has, int32_t x, int32_t slot, int32_t* deg, int32_t* inc) {
+// Adds edge `slot` to its end x's word: the degree in the low half, the sum of the edges' slots (mod 2^32)
+// in the high one (lanes with one end together).
+__device__ __forceinline__ void add_edge_end(bool has, int32_t x, uint32_t slot, unsigned long long* inc) {
   const int lane = threadIdx.x & 31;
   const unsigned peers = __match_any_sync(kFull, has ? x : -1 - lane);
   if (!has) return;
-  const uint32_t all = __reduce_xor_sync(peers, (uint32_t)slot);
-  if (lane == __ffs(peers) - 1) {
-    atomicAdd(deg + x, __popc(peers));
-    atomicXor(reinterpret_cast<uint32_t*>(inc + x), all);
-  }
+  const uint32_t all = __reduce_add_sync(peers, slot);
+  if (lane == __ffs(peers) - 1) atomicAdd(inc + x, (unsigned long long)all << 32 | (unsigned)__popc(peers));
 }
 
 // Step 4 by block 0: the core's edges i < mc, between id2[cu[cs[i]]] and id2[cv[cs[i]]], VC <= kCoreMax
@@ -1138,8 +1136,7 @@ __global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
   const int lane = threadIdx.x & 31;
   if (!may_start(A)) return;
   int32_t* const id = f.pre;    // a root's number
-  int32_t* const deg = f.sz;    // by number
-  int32_t* const inc = f.slo;
+  unsigned long long* const inc = reinterpret_cast<unsigned long long*>(f.next);  // by number (add_edge_end)
   int32_t* const id2 = f.hi;    // a core vertex's number
   int32_t* const gone = f.shi;  // by kept edge: stripped
   int32_t* const ku = reinterpret_cast<int32_t*>(f.sr);
@@ -1156,7 +1153,6 @@ __global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
     R.P2[x] = uf_root_static(R.P2, (int32_t)x);
     id[x] = -1;
     id2[x] = -1;
-    deg[x] = 0;
     inc[x] = 0;
     gone[x] = 0;
     f.P[x] = (int32_t)x;
@@ -1233,25 +1229,26 @@ __global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
       cu[i] = a;
       cv[i] = b;
     }
-    add_edge_end(in, a, (int32_t)i, deg, inc);
-    add_edge_end(in, b, (int32_t)i, deg, inc);
+    add_edge_end(in, a, (uint32_t)i, inc);
+    add_edge_end(in, b, (uint32_t)i, inc);
   }
   if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
+  // (a vertex's word names its one live edge as soon as it is its last, so that a step is three accesses deep;
+  // with the degree and the edges in words of their own, and a fence between them, it was seven: 24 us for
+  // the strip of 4,317 edges with paths of up to 8, 12 so)
   for (int64_t x0 = gspread(); x0 < verts; x0 += gstride()) {
     int32_t x = (int32_t)x0;
-    for (int step = 0; step < kStripSteps && ld_relaxed(deg + x) == 1; step++) {
-      // x's one live edge; if its other end's thread is taking it, the word read here may be any edge:
-      // one that does not touch x, or one that is gone
-      const int32_t i = ld_relaxed(inc + x);
-      if ((uint32_t)i >= (uint32_t)kept) break;
+    const unsigned long long w = inc[x];
+    uint32_t i = (uint32_t)(w >> 32);
+    if ((uint32_t)w != 1) continue;
+    for (int step = 0; step < kStripSteps && i < (uint32_t)kept; step++) {
       const int32_t a = cu[i], b = cv[i];
-      if ((a != x && b != x) || atomicExch(gone + i, 1) != 0) break;
+      if (atomicExch(gone + i, 1) != 0) break;  // its other end's thread has it
       const int32_t y = a ^ b ^ x;
-      st_relaxed(deg + x, 0);
-      if (ld_relaxed(deg + y) >= kHub) break;
-      atomicXor(reinterpret_cast<uint32_t*>(inc + y), (uint32_t)i);
-      __threadfence();  // whoever sees y's new degree sees its edges without this one
-      if (atomicSub(deg + y, 1) != 2) break;
+      if (ld_relaxed(reinterpret_cast<const int32_t*>(inc + y)) >= kHub) break;  // (the low half)
+      const unsigned long long old = atomicAdd(inc + y, 0ull - ((unsigned long long)i << 32 | 1ull));
+      if ((uint32_t)old != 2) break;
+      i = (uint32_t)(old >> 32) - i;
       x = y;
     }
   }

@@ -24,6 +24,9 @@ namespace {
 
 constexpr size_t kMiscBytes = 1024;  // status word, device counts of bridges_from_forest, spare output
 constexpr int64_t kSmallCallEdges = 22528;  // a whole call on one block up to this many edges
+// A batch of this many graphs is planned on the device (256 graphs of 64 to 256 vertices: 107 us a call with
+// the host's plan, 100 so; of 64 to 4,096: 420 and 417; 1,024 graphs 179 and 126, 614 and 545).
+constexpr int32_t kPlanGraphs = 256;
 constexpr size_t kClearBytes = kMiscBytes + 256;  // cleared at a call's start: the misc area and the
                                                   // certificate's control words, which follow it
 constexpr size_t kBarAt = 128;       // the final stage's barrier count; the reduced stage's counters at 768
@@ -468,6 +471,7 @@ void bridges_ctx_destroy(bridges_ctx* c) {
   if (c->h_pinned) cudaFreeHost(c->h_pinned);
   for (int k = 0; k < 2; k++) {
     if (c->b_exec[k]) cudaGraphExecDestroy(c->b_exec[k]);
+    if (c->b_exec_plan[k]) cudaGraphExecDestroy(c->b_exec_plan[k]);
     if (c->bstage[k]) cudaFreeHost(c->bstage[k]);
     if (c->b_done_ev[k]) cudaEventDestroy(c->b_done_ev[k]);
   }
@@ -730,6 +734,40 @@ int64_t next_pow2(int64_t x) {
   return p;
 }
 
+// Captures a batch whose descriptors are staged in copy k: reset counters, upload them (planned: the graphs,
+// from which plan_kernel makes the tasks; they lie where the tasks do in the staging copy and at the
+// certificate slots on the device), run the kernels.
+cudaGraphExec_t capture_batch(bridges_ctx* c, int k, bool planned) {
+  const BLayout L = blayout(c->b_task_cap, c->b_graph_cap, c->b_slot_cap);
+  char* d = static_cast<char*>(c->bws);
+  char* h = static_cast<char*>(c->bstage[k]);
+  BatchArgs* args = reinterpret_cast<BatchArgs*>(d + L.args);
+  cudaStream_t cs;
+  cudaGraph_t graph = nullptr;
+  cudaGraphExec_t exec = nullptr;
+  if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+  ok = ok && cudaMemsetAsync(d + L.queue, 0, 256, cs) == cudaSuccess;
+  ok = ok && cudaMemsetAsync(d + L.gerr, 0, L.slots - L.gerr, cs) == cudaSuccess;
+  if (planned) {
+    ok = ok && cudaMemcpyAsync(d + L.slots, h + L.s_tasks, (size_t)batch_plan_bytes(c->b_graph_cap),
+                               cudaMemcpyHostToDevice, cs) == cudaSuccess;
+    ok = ok && batched_plan_launch(cs, d + L.slots, args);
+  } else {
+    ok = ok && cudaMemcpyAsync(d, h, L.s_total, cudaMemcpyHostToDevice, cs) == cudaSuccess;
+  }
+  ok = ok && batched_launch(cs, args, c->num_sms);
+  ok = (cudaStreamEndCapture(cs, &graph) == cudaSuccess) && ok;
+  if (ok && cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess) exec = nullptr;
+  if (graph) cudaGraphDestroy(graph);
+  cudaStreamDestroy(cs);
+  if (!exec) cudaGetLastError();
+  return exec;
+}
+
 // (Re)creates the batched buffers and the two captured CUDA graphs for these capacities.
 int64_t ensure_batched(bridges_ctx* c, cudaStream_t s, int64_t ntasks, int64_t G, int64_t slots) {
   if (ntasks <= c->b_task_cap && G <= c->b_graph_cap && slots <= c->b_slot_cap && c->b_exec[0] && c->b_exec[1])
@@ -744,8 +782,10 @@ int64_t ensure_batched(bridges_ctx* c, cudaStream_t s, int64_t ntasks, int64_t G
   cudaStreamSynchronize(s);
   for (int k = 0; k < 2; k++) {
     if (c->b_exec[k]) cudaGraphExecDestroy(c->b_exec[k]);
+    if (c->b_exec_plan[k]) cudaGraphExecDestroy(c->b_exec_plan[k]);
     if (c->bstage[k]) cudaFreeHost(c->bstage[k]);
     c->b_exec[k] = nullptr;
+    c->b_exec_plan[k] = nullptr;
     c->bstage[k] = nullptr;
   }
   if (c->bws) cudaFree(c->bws);
@@ -764,32 +804,8 @@ int64_t ensure_batched(bridges_ctx* c, cudaStream_t s, int64_t ntasks, int64_t G
   c->bws_bytes = L.total;
   c->bstage_bytes = L.s_total;
   c->b_next = 0;
-  // capture, once per staging copy: reset counters, upload descriptors from that copy, run the
-  // kernel
-  char* d = static_cast<char*>(c->bws);
-  cudaStream_t cs;
-  if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) != cudaSuccess) return cuda_fail(cudaGetLastError());
-  bool ok = true;
-  for (int k = 0; k < 2 && ok; k++) {
-    cudaGraph_t graph;
-    ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
-    ok = ok && cudaMemsetAsync(d + L.queue, 0, 256, cs) == cudaSuccess;
-    ok = ok && cudaMemsetAsync(d + L.gerr, 0, L.slots - L.gerr, cs) == cudaSuccess;
-    ok = ok && cudaMemcpyAsync(d, c->bstage[k], L.s_total, cudaMemcpyHostToDevice, cs) == cudaSuccess;
-    ok = ok && batched_launch(cs, reinterpret_cast<const BatchArgs*>(d + L.args), c->num_sms);
-    ok = (cudaStreamEndCapture(cs, &graph) == cudaSuccess) && ok;
-    if (ok) ok = cudaGraphInstantiate(&c->b_exec[k], graph, 0) == cudaSuccess;
-    cudaGraphDestroy(graph);
-  }
-  cudaStreamDestroy(cs);
-  if (!ok) {
-    cudaGetLastError();
-    for (int k = 0; k < 2; k++) {
-      if (c->b_exec[k]) cudaGraphExecDestroy(c->b_exec[k]);
-      c->b_exec[k] = nullptr;
-    }
-    return BRIDGES_ECUDA;
-  }
+  for (int k = 0; k < 2; k++) c->b_exec[k] = capture_batch(c, k, false);
+  if (!c->b_exec[0] || !c->b_exec[1]) return BRIDGES_ECUDA;  // (tried again by the next batch)
   return BRIDGES_OK;
 }
 
@@ -816,11 +832,11 @@ int64_t plan_batch_tasks(const bridges_ctx* c, std::vector<BatchTask>& graphs, i
     const int b = batch_bucket(P, g.V);
     const int64_t split = b >= 0 && P.split[b] > 0 ? P.split[b] : auto_split;
     const int64_t E = g.hi - g.lo;
-    const int32_t np = (int32_t)std::min<int64_t>(64, std::max<int64_t>(1, (E + split - 1) / split));
+    const int32_t np = batch_parts(E, split);
     // the plan's group, raised to the smallest one the task fits (class 0 is the largest group)
     int cls = batch_min_class(g.V, np);
     if (b >= 0 && P.group[b] > 0) cls = std::min(cls, P.group[b] >= 1024 ? 0 : (P.group[b] >= 512 ? 1 : 2));
-    int64_t warm = 4LL * g.V + 2048;  // measured on the batched workload against 2V + 1024, 8V + 2048, 16V + 2048
+    int64_t warm = batch_warm(g.V);
     if (b >= 0 && (P.warm_per_v[b] > 0 || P.warm_add[b] > 0)) warm = (int64_t)P.warm_per_v[b] * g.V + P.warm_add[b];
     for (int32_t p = 0; p < np; p++) {
       BatchTask t = g;
@@ -907,6 +923,51 @@ int64_t launch_batch_tasks(bridges_ctx* c, cudaStream_t s, const std::vector<Bat
   return BRIDGES_OK;
 }
 
+// The same for a batch of G graphs planned on the device: `ntasks` tasks in all, split as given.  False in
+// *done: the descriptors do not fit where they would lie, or the graph cannot be captured; the host plans.
+int64_t launch_batch_planned(bridges_ctx* c, cudaStream_t s, const int32_t* u, const int32_t* v, const int64_t* edge_off,
+                             const int32_t* Vs, int32_t G, int32_t* out, int64_t* counts, int64_t split, int64_t ntasks,
+                             int64_t slot_words, bool* done) {
+  *done = false;
+  Range range("bridges: batched launch");
+  int64_t rc = ensure_batched(c, s, ntasks, G, slot_words);
+  if (rc) return rc;
+  const BLayout L = blayout(c->b_task_cap, c->b_graph_cap, c->b_slot_cap);
+  if (batch_plan_bytes(c->b_graph_cap) > (int64_t)std::min(L.total - L.slots, L.s_corder - L.s_tasks)) return BRIDGES_OK;
+  const int k = c->b_next;
+  if (!c->b_exec_plan[k]) c->b_exec_plan[k] = capture_batch(c, k, true);
+  if (!c->b_exec_plan[k]) return BRIDGES_OK;
+  *done = true;
+  c->b_next ^= 1;
+  cudaEventSynchronize(c->b_done_ev[k]);  // (see launch_batch_tasks)
+  char* d = static_cast<char*>(c->bws);
+  char* h = static_cast<char*>(c->bstage[k]) + L.s_tasks;
+  BatchPlanArgs P{};
+  P.u = u;
+  P.v = v;
+  P.out = out;
+  P.counts = counts;
+  P.split = split;
+  P.back_edges = c->b_back_edges;
+  P.G = G;
+  P.args.tasks = reinterpret_cast<const BatchTask*>(d + L.tasks);
+  P.args.corder = reinterpret_cast<const int32_t*>(d + L.corder);
+  P.args.d_ntasks = reinterpret_cast<const int32_t*>(d + L.ntasks);
+  P.args.queue = reinterpret_cast<int32_t*>(d + L.queue);
+  P.args.gerr = reinterpret_cast<int32_t*>(d + L.gerr);
+  P.args.slots = reinterpret_cast<uint32_t*>(d + L.slots);
+  P.args.G = G;
+  P.args.slot_words = c->b_slot_cap;
+  std::memcpy(h, &P, sizeof(P));
+  std::memcpy(h + kPlanHeader, edge_off, sizeof(int64_t) * (size_t)(G + 1));
+  std::memcpy(h + kPlanHeader + 8 * (size_t)(G + 1), Vs, sizeof(int32_t) * (size_t)G);
+  if (cudaStreamWaitEvent(s, c->b_done_ev[k ^ 1], 0) != cudaSuccess) return cuda_fail(cudaGetLastError());
+  if (cudaGraphLaunch(c->b_exec_plan[k], s) != cudaSuccess) return cuda_fail(cudaGetLastError());
+  if (cudaEventRecord(c->b_done_ev[k], s) != cudaSuccess) return cuda_fail(cudaGetLastError());
+  c->launches += 3;
+  return BRIDGES_OK;
+}
+
 // The automatic split: the batch's edges over three certification groups per SM (there are
 // four), no task above 2^20 edges and none below 2^17 (every task pays its own warm-up prefix).
 // A small batch then cuts its large graphs finer, so that the launch does not wait on its one
@@ -943,6 +1004,22 @@ extern "C" int64_t bridges_find_batched(bridges_ctx* c, struct CUstream_st* stre
   if (total_out > 0 && !out) return BRIDGES_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (cudaSetDevice(c->device) != cudaSuccess) return cuda_fail(cudaGetLastError());
+  // many graphs, automatic plan: planned on the device
+  bool planned = false;
+  if (c->bplan.n <= 0 && G >= kPlanGraphs) {
+    const int64_t split = default_split(c, total_e);
+    int64_t ntasks = 0, words = 0;
+    for (int32_t g = 0; g < G; g++) {
+      if (Vs[g] > kBatchVmax) continue;
+      const int64_t np = batch_parts(edge_off[g + 1] - edge_off[g], split);
+      ntasks += np;
+      words += np * batch_slot_words(Vs[g]);
+    }
+    if (ntasks > 0) {
+      const int64_t rc = launch_batch_planned(c, s, u, v, edge_off, Vs, G, out, out_counts, split, ntasks, words, &planned);
+      if (rc) return rc;
+    }
+  }
   // small graphs become batch tasks; graphs above the shared-memory size take the single-graph
   // path afterwards on the same stream
   std::vector<BatchTask> graphs, tasks;
@@ -956,6 +1033,7 @@ extern "C" int64_t bridges_find_batched(bridges_ctx* c, struct CUstream_st* stre
       large.push_back(g);
       continue;
     }
+    if (planned) continue;
     BatchTask t{};
     t.u = u;
     t.v = v;
@@ -967,8 +1045,11 @@ extern "C" int64_t bridges_find_batched(bridges_ctx* c, struct CUstream_st* stre
     t.V = Vs[g];
     graphs.push_back(t);
   }
-  const int64_t slots = plan_batch_tasks(c, graphs, total_e, tasks);
-  int64_t rc = launch_batch_tasks(c, s, tasks, (int32_t)graphs.size(), slots);
+  int64_t rc = BRIDGES_OK;
+  if (!planned) {
+    const int64_t slots = plan_batch_tasks(c, graphs, total_e, tasks);
+    rc = launch_batch_tasks(c, s, tasks, (int32_t)graphs.size(), slots);
+  }
   if (rc) return rc;
   for (int32_t g : large) {
     rc = run_single(c, s, u + edge_off[g], v + edge_off[g], edge_off[g + 1] - edge_off[g], Vs[g], 0, out + out_off[g],

@@ -53,7 +53,7 @@ struct BatchArgs {
 // The smallest group a task fits: 0 a whole block (more than kBatchHalfVmax vertices, or a
 // partition of a graph: partitions merge from the slots), 1 a half block, 2 the certification
 // group (a quarter block).
-inline int batch_min_class(int32_t V, int32_t nparts) {
+__host__ __device__ inline int batch_min_class(int32_t V, int32_t nparts) {
   if (V > kBatchHalfVmax || nparts > 1) return 0;
   return V > kBatchQuarterVmax ? 1 : 2;
 }
@@ -62,11 +62,38 @@ inline int batch_min_class(int32_t V, int32_t nparts) {
 // smallest it fits; never a smaller one).
 inline int batch_task_class(const BatchTask& t) { return t.cls; }
 
+// Partitions of a graph of E edges when lists of more than `split` are cut.
+__host__ __device__ inline int32_t batch_parts(int64_t E, int64_t split) {
+  const int64_t np = E <= split ? 1 : (E + split - 1) / split;
+  return (int32_t)(np < 64 ? np : 64);
+}
+
+// Edges certified one by one before a task's union-finds are flattened, with the automatic plan (measured on
+// the batched workload against 2V + 1024, 8V + 2048, 16V + 2048).
+__host__ __device__ inline int64_t batch_warm(int32_t V) { return 4LL * V + 2048; }
+
 // Words of a task's certificate slot: [nF, nF', F (V words), F' (V words), the root of each vertex's
 // F' tree (V u16, padded to a word), the root of each vertex's F tree (likewise)]; the roots are
 // written by a graph's first task (the F roots only when more tasks follow).  A graph's slots are
 // consecutive.
 __host__ __device__ inline int64_t batch_slot_words(int32_t V) { return 2 + 2 * (int64_t)V + 2 * (((int64_t)V + 1) / 2); }
+
+// A batch whose tasks are planned on the device (plan_kernel): this header, then edge_off (G + 1 int64), then
+// the vertex counts (G int32), in the memory of the certificate slots, which nothing else uses before
+// certification.
+struct BatchPlanArgs {
+  const int32_t* u;
+  const int32_t* v;
+  int32_t* out;
+  int64_t* counts;
+  int64_t split;  // edges above which a graph is cut
+  int64_t back_edges;  // tasks below this many edges may be claimed from the back (see BatchArgs.nback)
+  BatchArgs args;  // all but nbig, nmid and nback
+  int32_t G;
+};
+constexpr int64_t kPlanHeader = 256;
+static_assert(sizeof(BatchPlanArgs) <= kPlanHeader, "the plan's header");
+inline int64_t batch_plan_bytes(int64_t G) { return kPlanHeader + 8 * (G + 1) + 4 * G; }
 
 // One graph's final stage on one block (small_final_launch): the final certificate as the forest
 // pass and the merge tree leave it in global memory, for a graph of 2..kBatchVmax vertices.
@@ -120,5 +147,7 @@ bool small_final_launch(cudaStream_t s, const SmallFinalArgs& a);
 // Launches the two persistent kernels (one block per SM each: certification, then the bridge
 // stages) reading their arguments from *dev_args.
 bool batched_launch(cudaStream_t s, const BatchArgs* dev_args, int num_sms);
+// Launches plan_kernel on one block: the tasks of the batch at `plan` to *dev_args and the lists it names.
+bool batched_plan_launch(cudaStream_t s, const void* plan, BatchArgs* dev_args);
 
 }  // namespace bridges

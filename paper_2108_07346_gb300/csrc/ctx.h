@@ -51,6 +51,7 @@ struct bridges_ctx {
   int64_t b_task_cap = 0, b_graph_cap = 0, b_slot_cap = 0;
   std::vector<int32_t> b_order;  // the last batch's certification order (host scratch)
   cudaGraphExec_t b_exec[2]{};
+  cudaGraphExec_t b_exec_plan[2]{};  // the same for a batch planned on the device (captured at first use)
   cudaEvent_t b_done_ev[2]{};
   int b_next = 0;                // the staging copy the next batch fills
   int64_t b_split_edges = 0;     // partition graphs with more edges than this (0: automatic)

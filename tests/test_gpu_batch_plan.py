@@ -1,0 +1,48 @@
+"""Batches planned on the device (256 graphs and more) against the same graphs in batches that the host plans."""
+
+import numpy as np
+import pytest
+import torch
+
+import graphgen
+import paper_2108_07346_gb300 as pb
+
+pytestmark = pytest.mark.gpu
+
+SIZES = [0, 1, 2, 3, 64, 700, 1024, 1025, 2000, 3008, 3009, 4096, 4097, 6000]
+
+
+def results(ctx, u, v, off, Vs):
+    out, counts, at = ctx.find_batched(u, v, off, Vs)
+    out, counts = out.cpu().numpy(), counts.cpu().numpy()
+    return [(int(c), out[a:a + 2 * max(int(c), 0)].tolist()) for c, a in zip(counts, at)]
+
+
+@pytest.mark.parametrize("G", [256, 257, 1024, 1500])
+@pytest.mark.parametrize("split", [0, 300])
+def test_planned_on_device_equals_host(G, split):
+    """Every class, empty graphs and lists, graphs above the shared-memory size among the others, lists cut in up
+    to 64 parts, more graphs than the block has threads; one vertex id out of range."""
+    rng = np.random.default_rng(G + split)
+    Vs = np.array([SIZES[i % len(SIZES)] for i in range(G)], dtype=np.int32)
+    us, vs = [], []
+    for g, V in enumerate(Vs.tolist()):
+        E = 0 if V < 2 or g % 17 == 5 else int(rng.integers(1, 5 * V))
+        u, v = graphgen.random_multigraph(1000 * G + g, V, E) if E else (np.empty(0), np.empty(0))
+        us.append(np.asarray(u, dtype=np.int32))
+        vs.append(np.asarray(v, dtype=np.int32))
+    us[4] = us[4].copy()
+    us[4][-1] = 64  # SIZES[4] vertices
+    off = np.concatenate([[0], np.cumsum([len(u) for u in us])]).astype(np.int64)
+    u = torch.from_numpy(np.concatenate(us)).cuda()
+    v = torch.from_numpy(np.concatenate(vs)).cuda()
+    ctx = pb.Context()
+    ctx.set_batch_split(split)
+    got = results(ctx, u, v, off, Vs)
+    assert results(ctx, u, v, off, Vs) == got  # the other staging copy
+    want = []
+    for a in range(0, G, 255):
+        b = min(G, a + 255)
+        want += results(ctx, u, v, off[a:b + 1], Vs[a:b])
+    assert got == want
+    assert got[4][0] < 0 and sum(c for c, _ in got) > 100

@@ -24,8 +24,9 @@ namespace {
 
 constexpr size_t kMiscBytes = 1024;  // status word, device counts of bridges_from_forest, spare output
 constexpr int64_t kSmallCallEdges = 22528;  // a whole call on one block up to this many edges
-// A batch of this many graphs is planned on the device (256 graphs of 64 to 256 vertices: 107 us a call with
+// A batch of this many graphs is planned on the device when the context's previous batch is done (256 graphs of 64 to 256 vertices: 107 us a call with
 // the host's plan, 100 so; of 64 to 4,096: 420 and 417; 1,024 graphs 179 and 126, 614 and 545).
+// While the previous one runs, the host's plan costs nothing and plan_kernel its 22 us.
 constexpr int32_t kPlanGraphs = 256;
 constexpr size_t kClearBytes = kMiscBytes + 256;  // cleared at a call's start: the misc area and the
                                                   // certificate's control words, which follow it
@@ -923,6 +924,19 @@ int64_t launch_batch_tasks(bridges_ctx* c, cudaStream_t s, const std::vector<Bat
   return BRIDGES_OK;
 }
 
+// Whether every choice of plan P is the automatic one.
+static bool automatic_plan(const bridges_batch_plan& P) {
+  for (int b = 0; b < P.n; b++)
+    if (P.group[b] > 0 || P.split[b] > 0 || P.warm_per_v[b] > 0 || P.warm_add[b] > 0) return false;
+  return true;
+}
+
+// Whether the context's last batch has finished (or there was none).
+static bool batch_idle(const bridges_ctx* c) {
+  cudaEvent_t last = c->b_done_ev[c->b_next ^ 1];
+  return !last || cudaEventQuery(last) == cudaSuccess;
+}
+
 // The same for a batch of G graphs planned on the device: `ntasks` tasks in all, split as given.  False in
 // *done: the descriptors do not fit where they would lie, or the graph cannot be captured; the host plans.
 int64_t launch_batch_planned(bridges_ctx* c, cudaStream_t s, const int32_t* u, const int32_t* v, const int64_t* edge_off,
@@ -1004,9 +1018,9 @@ extern "C" int64_t bridges_find_batched(bridges_ctx* c, struct CUstream_st* stre
   if (total_out > 0 && !out) return BRIDGES_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (cudaSetDevice(c->device) != cudaSuccess) return cuda_fail(cudaGetLastError());
-  // many graphs, automatic plan: planned on the device
+  // many graphs, automatic plan, no batch to hide the host's planning behind: planned on the device
   bool planned = false;
-  if (c->bplan.n <= 0 && G >= kPlanGraphs) {
+  if (G >= kPlanGraphs && automatic_plan(c->bplan) && batch_idle(c)) {
     const int64_t split = default_split(c, total_e);
     int64_t ntasks = 0, words = 0;
     for (int32_t g = 0; g < G; g++) {

@@ -52,7 +52,7 @@ namespace {
 constexpr int kThreads = 1024;
 constexpr int kMaxRounds = 24;  // rounds before the remaining edges take the union-finds one by one
 // Live edges that take the union-finds one by one, and at most V / 2 (what a round more or less costs: 2.5 M
-// edges on 37,147 vertices 70.7 us with 8,192 and V / 4, 66.8 so; 110 k on 90,000: 66.8 and 57.5; 9 k on 8,000:
+// edges on 37,147 vertices 70.7 us with 8,192 and V / 4, 66.8 with these; 110 k on 90,000: 66.8 and 57.5; 9 k on 8,000:
 // 45.6 and 39.7; with V, 30 k on 20,000 take 108 us instead of 59: the sets have not met yet).
 constexpr unsigned kFewLive = 32768;
 constexpr int kGroup = 8;       // edges per group of the sample (kSampleShift)
@@ -81,19 +81,26 @@ __device__ __forceinline__ unsigned long long hook_of(uint32_t slot, int32_t lo)
   return (unsigned long long)(slot * 0x9e3779b1u) << 32 | (uint32_t)lo;
 }
 
-// Vertex x's new root in the forest `which` (0: F, 1: F'), its last one r having hook h.  A long chain
-// (a path in list order) shortens as all its vertices walk it: past a few hooks the walk goes on from
-// what R holds for the vertex reached and leaves its own progress in R[x], so jumps double.
-__device__ __forceinline__ int32_t climb(int2* R, int which, const unsigned long long* H, int64_t x, int32_t r,
-                                         unsigned long long h) {
-  int32_t* roots = reinterpret_cast<int32_t*>(R) + which;
-  for (int k = 0; h != kNoHook; k++) {
-    r = (int32_t)(uint32_t)h;
+// Vertex x's new roots in F and F', its last ones r having hooks h1 and h2; the two walks run side by side (one
+// after the other: 67.3 us for the sample of 2.5 M edges on 37,147 vertices, 65.0 so; sorted 61.3 and 58.5).
+// A long chain (a path in list order) shortens as all its vertices walk it: past a few hooks the walk goes
+// on from what R holds for the vertex reached and leaves its own progress in R[x], so jumps double.
+__device__ __forceinline__ int2 climb(int2* R, const unsigned long long* H1, const unsigned long long* H2, int64_t x,
+                                      int2 r, unsigned long long h1, unsigned long long h2) {
+  int32_t* roots = reinterpret_cast<int32_t*>(R);
+  for (int k = 0; h1 != kNoHook || h2 != kNoHook; k++) {
+    const bool a = h1 != kNoHook, b = h2 != kNoHook;
+    if (a) r.x = (int32_t)(uint32_t)h1;
+    if (b) r.y = (int32_t)(uint32_t)h2;
     if (k >= 6) {
-      r = ld_relaxed(roots + 2 * (int64_t)r);
-      st_relaxed(roots + 2 * x, r);
+      const int32_t ra = a ? ld_relaxed(roots + 2 * (int64_t)r.x) : 0;
+      const int32_t rb = b ? ld_relaxed(roots + 2 * (int64_t)r.y + 1) : 0;
+      if (a) st_relaxed(roots + 2 * x, r.x = ra);
+      if (b) st_relaxed(roots + 2 * x + 1, r.y = rb);
     }
-    h = H[r];
+    const unsigned long long n1 = a ? H1[r.x] : kNoHook, n2 = b ? H2[r.y] : kNoHook;
+    h1 = n1;
+    h2 = n2;
   }
   return r;
 }
@@ -255,8 +262,7 @@ __global__ void __launch_bounds__(kThreads, 1) sample_kernel(SampleArgs A) {
     for (int64_t x = gspread(); x < V; x += gstride()) {
       int2 r = R[x];
       const unsigned long long h1 = H1[r.x], h2 = H2[r.y];
-      if (h1 != kNoHook) r.x = climb(R, 0, H1, x, r.x, h1);
-      if (h2 != kNoHook) r.y = climb(R, 1, H2, x, r.y, h2);
+      r = climb(R, H1, H2, x, r, h1, h2);
       R[x] = r;
       if (last || t == kMaxRounds) {
         J.P1[x] = r.x;

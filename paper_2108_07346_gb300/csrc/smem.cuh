@@ -545,21 +545,18 @@ __device__ void s_certify_rounds(const Grp<NT>& G, uint32_t* ed, int32_t slots, 
       if (w2) put(2, b2, ed[((h2 >> kLoBits) * kKeyInv) & kKeyMask]);
       if (h1 == kFree && h2 == kFree) continue;
       // a long chain shortens as all its vertices walk it (climb, sample.cu)
-      for (int k = 0; h1 != kFree; k++) {
-        r1 = h1 & ((1u << kLoBits) - 1);
+      for (int k = 0; h1 != kFree || h2 != kFree; k++) {
+        const bool a = h1 != kFree, b = h2 != kFree;
+        if (a) r1 = h1 & ((1u << kLoBits) - 1);
+        if (b) r2 = h2 & ((1u << kLoBits) - 1);
         if (k >= 6) {
-          r1 = Rv[r1] & 0xffff;
-          Rv[x] = r1 | (r & 0xffff0000u);
-        }
-        h1 = H1[r1];
-      }
-      for (int k = 0; h2 != kFree; k++) {
-        r2 = h2 & ((1u << kLoBits) - 1);
-        if (k >= 6) {
-          r2 = Rv[r2] >> 16;
+          if (a) r1 = Rv[r1] & 0xffff;
+          if (b) r2 = Rv[r2] >> 16;
           Rv[x] = r1 | r2 << 16;
         }
-        h2 = H2[r2];
+        const uint32_t n1 = a ? H1[r1] : kFree, n2 = b ? H2[r2] : kFree;
+        h1 = n1;
+        h2 = n2;
       }
       Rv[x] = r1 | r2 << 16;
     }

@@ -82,7 +82,7 @@ __device__ __forceinline__ unsigned long long hook_of(uint32_t slot, int32_t lo)
 }
 
 // Vertex x's new roots in F and F', its last ones r having hooks h1 and h2; the two walks run side by side (one
-// after the other: 67.3 us for the sample of 2.5 M edges on 37,147 vertices, 65.0 so; sorted 61.3 and 58.5).
+// after the other: 67.3 us for the sample of 2.5 M edges on 37,147 vertices, 65.0 so).
 // A long chain (a path in list order) shortens as all its vertices walk it: past a few hooks the walk goes
 // on from what R holds for the vertex reached and leaves its own progress in R[x], so jumps double.
 __device__ __forceinline__ int2 climb(int2* R, const unsigned long long* H1, const unsigned long long* H2, int64_t x,

@@ -524,6 +524,9 @@ CertPlan make_plan(int64_t E, int32_t V, int32_t M, int32_t fan_in, int32_t bloc
     warm = std::min(warm, cap);
     const int64_t groups = ceil_div(E, 1 << kSampleShift);
     p.stride = E <= warm ? 1 : ceil_div(groups, std::max<int64_t>(warm >> kSampleShift, 1));
+    // (a sample is one group at least: a list of one group is certified whole whatever `warm` is, and
+    // nothing of it may be offered again)
+    if (p.stride <= 1) warm = std::max(warm, E);
     p.cache = E > warm;
     p.warm = warm;
     p.warm_block = p.block;

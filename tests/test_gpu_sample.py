@@ -96,3 +96,30 @@ def test_ids_out_of_range(cuda_lib, E, at):
     with pytest.raises(cuda_lib.BridgesError) as err:
         ctx.find(torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda(), V)
     assert err.value.code == -2
+
+
+@pytest.mark.parametrize("V", [9, 5000])
+@pytest.mark.parametrize("warm", [1, 3, 7, 8, 9])
+@pytest.mark.parametrize("E", [1, 2, 4, 7, 8, 9, 10, 16, 17])
+def test_samples_below_one_group(cuda_lib, V, warm, E):
+    """warm_edges below a sample's group of 8, lists around one and two groups: every edge is certified once, in
+    each call that starts from a sample."""
+    import torch
+
+    rng = np.random.default_rng(100 * warm + E)
+    x = np.arange(E, dtype=np.int32)
+    paths = (x % (V - 1), x % (V - 1) + 1)  # (V 9, E 9 and more: a path with doubled edges)
+    few = rng.integers(0, min(V, E + 1), (2, E)).astype(np.int32)
+    for u, v in [tuple(a.astype(np.int32) for a in paths), (few[0].copy(), few[1].copy())]:
+        _check(cuda_lib, u, v, V, warm_edges=warm)
+        du, dv = torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda()
+        ref = oracle.dfs_bridges(u, v, V).tolist()
+        count, labels = oracle.two_edge_components(u, v, V)
+        ctx = cuda_lib.Context(device="cuda:0", warm_edges=warm)
+        got, lab = ctx.two_edge_components(du, dv, V)
+        assert got == count and np.array_equal(lab.cpu().numpy(), labels)
+        points, bridges = ctx.articulation_points(du, dv, V, with_bridges=True)
+        assert bridges.cpu().numpy().tolist() == ref
+        assert points.cpu().numpy().tolist() == oracle.articulation_points(u, v, V).tolist()
+        inc = cuda_lib.Incremental(device="cuda:0", warm_edges=warm)
+        assert inc.reset(du, dv, V).cpu().numpy().tolist() == ref

@@ -503,6 +503,8 @@ CertPlan make_plan(int64_t E, int32_t V, int32_t M, int32_t fan_in, int32_t bloc
     cps = fits ? (int)std::max<size_t>(1, std::min<size_t>(2, (228 * 1024) / (snap_bytes + 2048))) : 2;
   }
   p.block = block > 0 ? block : (cps < 2 || !fits ? 1024 : 512);
+  // whole warps: the winners' staging counts, places and sends by warps
+  if (p.block < 1024) p.block = (p.block + 31) / 32 * 32;
   p.G = (int32_t)std::max<int64_t>(1, ((int64_t)num_sms * cps) / p.M);
   // a short list takes fewer blocks, one 16-byte unit of each array per thread (130 k edges: 18 us with
   // 608 blocks, 12 with 64)

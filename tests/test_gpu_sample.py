@@ -123,3 +123,13 @@ def test_samples_below_one_group(cuda_lib, V, warm, E):
         assert points.cpu().numpy().tolist() == oracle.articulation_points(u, v, V).tolist()
         inc = cuda_lib.Incremental(device="cuda:0", warm_edges=warm)
         assert inc.reset(du, dv, V).cpu().numpy().tolist() == ref
+
+
+@pytest.mark.parametrize("block", [1, 33, 100, 500, 1000])
+@pytest.mark.parametrize("V,E", [(5000, 200_000), (70_000, 2_000_000), (130_000, 400_000)])
+def test_blocks_of_odd_sizes(cuda_lib, block, V, E):
+    """A block size that is no whole number of warps: labels, bitmap and (the second call) no snapshot."""
+    rng = np.random.default_rng(block)
+    u, v = _er(rng, V, E)
+    _check(cuda_lib, u, v, V, block=block)
+    _check(cuda_lib, u, v, V, block=block, warm_edges=0)

@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(1024, 1) leaf_kernel(LeafArgs A) {
                  staged[warp]};
   const ForestSink S{J, win, A.V, A.b.status, A.u, A.mode == 1 ? A.stride : 0};
   const uint32_t clampv = MODE == 2 ? (uint32_t)A.Vb : (uint32_t)A.V;
-  if (A.mode == 1 && use_tiles(a, z, A.G, blockDim.x, kUnroll)) {
+  if (A.mode == 1 && use_tiles<VEC>(a, z, A.G, blockDim.x, kUnroll)) {
     stream_range<MODE, VEC, kUnroll>(S, A.u, A.v, a, z, clampv, slab, m, A.G, A.queue);
   } else {
     const int64_t n = z - a;

@@ -182,9 +182,12 @@ __device__ __forceinline__ bool excluded(int64_t i, uint32_t stride) {
 // Whether `members` blocks of nt threads share [s, t) in interleaved tiles (true) or take one
 // slice each (false): tiles only when every block gets at least 16 of them -- a tile is 4U edges
 // per thread, so on a short list tiles would leave blocks idle (a 1 M-edge list has 61 tiles of
-// 16,384 edges for 152 blocks).
+// 16,384 edges for 152 blocks).  Only the vector body of a range is tiled: without it (arrays off
+// their 16-byte boundaries) member 0 would read the whole range by itself (45 M edges: 53 ms in
+// tiles, 0.37 in slices).
+template <bool VEC>
 __device__ __forceinline__ bool use_tiles(int64_t s, int64_t t, int64_t members, int nt, int U) {
-  return members > 1 && t - s >= 16 * members * (int64_t)nt * 4 * U;
+  return VEC && members > 1 && t - s >= 16 * members * (int64_t)nt * 4 * U;
 }
 
 // Edge index of bit `bit` of a miss mask (see stream_range).

@@ -133,3 +133,35 @@ def test_blocks_of_odd_sizes(cuda_lib, block, V, E):
     u, v = _er(rng, V, E)
     _check(cuda_lib, u, v, V, block=block)
     _check(cuda_lib, u, v, V, block=block, warm_edges=0)
+
+
+@pytest.mark.parametrize("V", [20_000, 60_000, 130_000])
+def test_long_unaligned_slices(cuda_lib, V):
+    """A list long enough for interleaved tiles whose arrays start off a 16-byte boundary: the aligned copy's
+    result, in a time of the same order (one block alone would take 200 times as long)."""
+    import time
+
+    import torch
+
+    E = 60_000_000
+    gen = torch.Generator(device="cuda").manual_seed(V)
+    u = torch.randint(0, V, (E + 1,), dtype=torch.int32, device="cuda", generator=gen)
+    v = torch.randint(0, V, (E + 1,), dtype=torch.int32, device="cuda", generator=gen)
+    tail = torch.arange(V, V + 40, dtype=torch.int32, device="cuda")  # a pendant path
+    u[E - 40:E], v[E - 40:E] = tail, tail - 1
+    u, v = u[:E], v[:E]
+    ctx = cuda_lib.Context(device="cuda:0", ap_fused=0 if V != 60_000 else -1)
+
+    def timed(call):
+        call()
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        got = call()
+        torch.cuda.synchronize()
+        return got.cpu().numpy().tolist(), time.perf_counter() - t
+
+    for call in (ctx.find, ctx.articulation_points):
+        want, aligned = timed(lambda: call(u[4:], v[4:], V + 40))
+        got, unaligned = timed(lambda: call(u[1:], v[1:], V + 40))
+        assert got == want and len(got) >= 39
+        assert unaligned < 8 * aligned

@@ -471,7 +471,8 @@ int32_t bridges_wait_value(bridges_ctx* ctx, struct CUstream_st* stream, const i
  * bridges_ctx_last_config: the M, fan-in, CTAs per partition, block size and warm-up edges
  * of the last call (5 values), then the last bridges_articulation_points call's block-pass
  * prefix edges (-1: no snapshot) and blocks (values 6 and 7) and its form (value 8: 1 = one
- * fused read of the list, 0 = two passes); returns min(n, 8).
+ * fused read of the list, 0 = two passes), then how many blocks of the last call's forest pass one
+ * SM holds at once (value 9; 0: the plan had no snapshot to stream against); returns min(n, 9).
  * bridges_status_string: a static description of a status code.
  */
 int32_t bridges_ctx_stage_ms(const bridges_ctx* ctx, float* ms, int32_t n);

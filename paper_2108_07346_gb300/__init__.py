@@ -469,9 +469,10 @@ class Context:
         return int(self._lib.bridges_ctx_launches(self._h))
 
     def last_config(self):
-        buf = (ctypes.c_int64 * 8)()
-        k = self._lib.bridges_ctx_last_config(self._h, buf, 8)
-        names = ["M", "fan_in", "blocks_per_partition", "block", "warm_edges", "ap_warm_edges", "ap_blocks", "ap_fused"]
+        buf = (ctypes.c_int64 * 9)()
+        k = self._lib.bridges_ctx_last_config(self._h, buf, 9)
+        names = ["M", "fan_in", "blocks_per_partition", "block", "warm_edges", "ap_warm_edges", "ap_blocks", "ap_fused",
+                 "stream_resident"]
         return {names[i]: int(buf[i]) for i in range(k)}
 
 

@@ -235,6 +235,7 @@ int64_t run_path(bridges_ctx* c, cudaStream_t s, const int32_t* u, const int32_t
   Carved k = carve(c, p);
   if (count) k.fin.count = count;
   Launch L = launch_for(c, s);
+  c->last_plan = p;
   c->last_cfg[0] = p.M;
   c->last_cfg[1] = p.f;
   c->last_cfg[2] = p.G;
@@ -395,6 +396,7 @@ int64_t run_path_host(bridges_ctx* c, cudaStream_t s, const int32_t* hu, const i
   Carved k = carve(c, p);
   if (count) k.fin.count = count;
   Launch L = launch_for(c, s);
+  c->last_plan = p;
   c->last_cfg[0] = p.M;
   c->last_cfg[1] = p.f;
   c->last_cfg[2] = p.G;
@@ -674,8 +676,9 @@ int64_t bridges_ctx_launches(const bridges_ctx* c) { return c ? c->launches : 0;
 
 int32_t bridges_ctx_last_config(const bridges_ctx* c, int64_t* vals, int32_t n) {
   if (!c || !vals) return 0;
-  int32_t k = std::min<int32_t>(n, 8);
-  for (int i = 0; i < k; i++) vals[i] = c->last_cfg[i];
+  int32_t k = std::min<int32_t>(n, 9);
+  for (int i = 0; i < std::min(k, 8); i++) vals[i] = c->last_cfg[i];
+  if (k == 9) vals[8] = cudaSetDevice(c->device) == cudaSuccess ? cert_stream_resident(c->last_plan) : 0;
   return k;
 }
 
@@ -1459,6 +1462,7 @@ static int64_t articulation_fused_run(bridges_ctx* c, cudaStream_t s, const Laun
   const ApBufs b0 = carve_ap(ws + ap_at, V);
   const ApBufs b1 = carve_ap(ws + ap_at + apb, V);
   const FusedBufs fb = carve_fused(ws + ap_at + 2 * apb, E);
+  c->last_plan = p;
   c->last_cfg[0] = p.M;
   c->last_cfg[1] = p.f;
   c->last_cfg[2] = p.G;

@@ -163,7 +163,11 @@ struct ForestSink {
   }
 };
 
-constexpr size_t kStageBytes = 32 * 2 * kStage * sizeof(int2);  // of a block of 1,024 threads
+// Shared memory of the staging of a block of so many threads.
+constexpr size_t stage_bytes(int threads) { return (size_t)((threads + 31) / 32) * 2 * kStage * sizeof(int2); }
+// Shared memory that a block of the stream takes besides its snapshot and staging: the 1 KB that every block
+// is charged, and its static arrays (under 512 bytes).
+constexpr size_t kBlockShared = 1024 + 512;
 constexpr int kUnroll = 4;  // int4 units of u (and of v) in flight per thread: 16 edges
 
 struct LeafArgs {
@@ -452,6 +456,12 @@ void snapshot_bitmap(const Launch& L, const CertPlan& p, const CertBufs& b) {
   *L.launches += 3;
 }
 
+// Dynamic shared memory of a block of the plan's stream.
+size_t stream_smem(const CertPlan& p) {
+  const size_t snap = p.mode == 1 ? align_up((size_t)p.V + 1, 8) * 2 : (size_t)(p.Vb / 32 + 4) * 4;
+  return align_up(snap, 16) + (p.stage ? stage_bytes(p.block) : 0);
+}
+
 template <int MODE, bool VEC>
 void launch_leaf(const Launch& L, const CertPlan& p, const LeafArgs& a, size_t smem) {
   auto k = leaf_kernel<MODE, VEC>;
@@ -494,17 +504,31 @@ CertPlan make_plan(int64_t E, int32_t V, int32_t M, int32_t fan_in, int32_t bloc
   p.mode = labels_fit ? 1 : 2;
   p.Vb = (int32_t)std::min<int64_t>(align_up((size_t)std::max(V, 1), 128), std::max<int64_t>(bm_cap, 128));
   const bool fits = labels_fit || bm_cap >= 128;
-  // Blocks per SM: 1,024 threads of the stream fit (64 registers each), as one block of 1,024 or two of
-  // 512; a second wave would wait for the first (2.5 M edges, 16-bit labels of 74 KB: 26 us with three
-  // blocks of 512 per SM, 24 with two).
+  // Blocks per SM, all of them in one wave (a second wave would wait for the first): 1,024 threads of the
+  // stream fit (64 registers each), as two blocks of 512 while two snapshots do, each with the staging of
+  // its warps' winners, else as one block of 1,024.  The line is where the second block would no longer be
+  // resident (49,528 vertices, or 792 k with the bitmap): past it two blocks of 512 run in two waves of half
+  // the threads (300 M edges on 53,000 vertices 606 us a call, 515 as one block; 57,000: 599 and 503; 20 M
+  // R-MAT edges on 850,000: 567 and 521).  Before it the two shapes are close (37,000: 499 and 494; R-MAT
+  // 400,000: 410 and 426), but for the longest lists near the line (300 M edges on 49,000: 565 and 510; 20 M:
+  // 200 and 197).
+  const size_t snap = align_up(labels_fit ? lab_bytes : (size_t)(p.Vb / 32 + 4) * 4, 16);
+  auto resident = [&](int threads) {
+    const size_t bytes = snap + stage_bytes(threads) + kBlockShared;
+    return (int)std::min<size_t>(1024 / std::max(threads, 1), (smem_optin + 1024) / bytes);
+  };
   int cps = ctas_per_sm;
-  if (cps <= 0) {
-    const size_t snap_bytes = labels_fit ? lab_bytes : (size_t)(p.Vb / 32 + 4) * 4;
-    cps = fits ? (int)std::max<size_t>(1, std::min<size_t>(2, (228 * 1024) / (snap_bytes + 2048))) : 2;
-  }
-  p.block = block > 0 ? block : (cps < 2 || !fits ? 1024 : 512);
+  p.block = block;
+  if (cps <= 0 && block <= 0)
+    cps = fits ? (resident(512) >= 2 ? 2 : 1) : 2;
+  else if (cps <= 0)
+    cps = fits ? std::max(1, std::min(2, resident(block))) : 2;
+  if (block <= 0) p.block = cps < 2 || !fits ? 1024 : 512;
   // whole warps: the winners' staging counts, places and sends by warps
   if (p.block < 1024) p.block = (p.block + 31) / 32 * 32;
+  // (also where blocks per SM set by the caller then run in two waves: 20 M R-MAT edges on 850,000 vertices,
+  // two blocks of 512 per SM, 561 us a call, 687 in one wave without the staging)
+  p.stage = snap + stage_bytes(p.block) + 1024 <= smem_optin;
   p.G = (int32_t)std::max<int64_t>(1, ((int64_t)num_sms * cps) / p.M);
   // a short list takes fewer blocks, one 16-byte unit of each array per thread (130 k edges: 18 us with
   // 608 blocks, 12 with 64)
@@ -559,6 +583,17 @@ CertPlan make_plan(int64_t E, int32_t V, int32_t M, int32_t fan_in, int32_t bloc
   return p;
 }
 
+int cert_stream_resident(const CertPlan& p) {
+  if (!p.cache) return 0;
+  int n = 0;
+  const void* k = p.mode == 1 ? (const void*)leaf_kernel<1, true> : (const void*)leaf_kernel<2, true>;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, p.block, stream_smem(p)) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
 size_t cert_bytes(const CertPlan& p) {
   const size_t MV = (size_t)p.M * (size_t)std::max(p.V, 1);
   const size_t Vpad = align_up((size_t)p.V + 1, 8);
@@ -609,9 +644,9 @@ void cert_warm(const Launch& L, const CertPlan& p, const CertBufs& b, const int3
   if (p.E == 0) return;
   const LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 0, p.Vb, 0, 0, 0, 0, nullptr, b};
   if (((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v)) & 15) == 0)
-    launch_leaf<0, true>(L, p, a, kStageBytes);
+    launch_leaf<0, true>(L, p, a, stage_bytes(p.warm_block));
   else
-    launch_leaf<0, false>(L, p, a, kStageBytes);
+    launch_leaf<0, false>(L, p, a, stage_bytes(p.warm_block));
 }
 
 void cert_snapshot(const Launch& L, const CertPlan& p, const CertBufs& b) {
@@ -628,13 +663,9 @@ void cert_stream(const Launch& L, const CertPlan& p, const CertBufs& b, const in
   LeafArgs a{u, v, p.E, p.V, p.M, p.G, p.warm, 1, p.Vb, r0, r1, p.sampled ? (uint32_t)p.stride : 0u,
              -1, p.M == 1 && r1 <= r0 ? b.ctl + kCtlQueue : nullptr, b};
   const bool vec = ((reinterpret_cast<uintptr_t>(u) | reinterpret_cast<uintptr_t>(v)) & 15) == 0;
-  // the snapshot, and behind it the warps' winners where the block's shared memory has room
-  size_t smem = align_up(p.mode == 1 ? (size_t)b.Vpad * 2 : (size_t)(p.Vb / 32 + 4) * 4, 16);
-  const size_t stage = kStageBytes * (size_t)p.block / 1024;
-  if (smem + stage + 1024 <= L.smem_optin) {
-    a.stage_at = (int32_t)smem;
-    smem += stage;
-  }
+  // the snapshot, and behind it the warps' winners
+  const size_t smem = stream_smem(p);
+  if (p.stage) a.stage_at = (int32_t)(smem - stage_bytes(p.block));
   if (p.mode == 1) {
     if (vec)
       launch_leaf<1, true>(L, p, a, smem);

@@ -51,6 +51,7 @@ struct CertPlan {
   int64_t stride;  // ... and are every stride-th group of the list (0: its first `warm` edges;
                    // 1: the whole list)
   bool cache;      // a snapshot is taken after the warm-up
+  bool stage;      // the stream's blocks have room to stage their warps' winners
   int32_t mode;    // its form: 1 = 16-bit F' labels (2V bytes fit in shared memory), 2 = bitmap
                    // of one large F' component (for larger V)
   int32_t Vb;      // mode 2: vertices [0, Vb) covered by the bitmap (a multiple of 128)
@@ -181,6 +182,8 @@ void cert_merge(const Launch& L, const CertPlan& p, const CertBufs& b);
 // Plan for (E, V, M) on this device.
 CertPlan make_plan(int64_t E, int32_t V, int32_t M, int32_t fan_in, int32_t block, int32_t ctas_per_sm,
                    int64_t warm, int num_sms, size_t smem_optin, int32_t warm_block = 0);
+// Blocks of the plan's stream that one SM holds at once (0: the plan has no stream).
+int cert_stream_resident(const CertPlan& p);
 // Workspace bytes of the certificate stage.
 size_t cert_bytes(const CertPlan& p);
 CertBufs carve_cert(void* base, const CertPlan& p);

@@ -165,3 +165,28 @@ def test_long_unaligned_slices(cuda_lib, V):
         got, unaligned = timed(lambda: call(u[1:], v[1:], V + 40))
         assert got == want and len(got) >= 39
         assert unaligned < 8 * aligned
+
+
+@pytest.mark.parametrize("V", [4097, 20_000, 37_147, 46_000, 49_527, 49_528, 53_000, 57_343, 57_344, 60_000, 99_000,
+                               113_000, 130_000, 792_000, 793_000, 850_000, 917_400, 917_600, 1_500_000])
+@pytest.mark.parametrize("opts", [{}, {"block": 1024}, {"block": 768}, {"block": 256}, {"M": 3}])
+def test_stream_in_one_wave(cuda_lib, V, opts):
+    """Every block of the automatic stream is resident at once, around the sizes at which the snapshot, with and
+    without the winners' staging, fits an SM twice; and the result there."""
+    import torch
+
+    gen = torch.Generator(device="cuda").manual_seed(V)
+    E = max(20 * V, 6_000_000)  # every partition has a snapshot, and every block edges
+    u = torch.randint(0, V, (E,), dtype=torch.int32, device="cuda", generator=gen)
+    v = torch.randint(0, V, (E,), dtype=torch.int32, device="cuda", generator=gen)
+    tail = torch.arange(V, V + 40, dtype=torch.int32, device="cuda")  # a pendant path, its last edge doubled
+    u[-41:], v[-41:] = torch.cat([tail, tail[-1:]]), torch.cat([tail - 1, tail[-1:] - 1])
+    ctx = cuda_lib.Context(device="cuda:0", **opts)
+    got = ctx.find(u, v, V + 40).cpu().numpy()
+    cfg = ctx.last_config()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert 1 <= cfg["M"] * cfg["blocks_per_partition"] <= sms * cfg["stream_resident"]
+    if V <= 850_000:  # (a sparse random graph has bridges of its own)
+        want = [[V - 1 + i, V + i] for i in range(39)]
+        inner = got[got[:, 1] < V]
+        assert got[got[:, 1] >= V].tolist() == want and (V > 113_000 or len(inner) == 0)

@@ -84,10 +84,11 @@ typedef struct bridges_opts {
                             16-bit label snapshot and the larger workspace of that form fits the
                             context's budget or workspace), < 0 = always the two-pass form */
   int32_t test_barrier_polls; /* for tests of the failure path; 0 in normal use.  > 0: a grid
-                                 barrier of the final stage gives up after this many polls
-                                 (~100 ns apart; default 2^22) with BRIDGES_ETIMEDOUT */
-  int32_t test_hold_polls;    /* for tests of the failure path; 0 in normal use.  > 0: the final
-                                 stage's last block sleeps this many ~100 ns polls before its first
+                                 barrier of the sampled certificate or the final stage gives up
+                                 after this many polls (~100 ns apart; default 2^22) with
+                                 BRIDGES_ETIMEDOUT */
+  int32_t test_hold_polls;    /* for tests of the failure path; 0 in normal use.  > 0: the last
+                                 block of either sleeps this many ~100 ns polls before its first
                                  barrier, so that a short barrier wait above gives up */
   int32_t test_fail_alloc;    /* for tests of the failure path; 0 in normal use.  n > 0: the n-th
                                  device allocation of the context's own buffers (workspace,

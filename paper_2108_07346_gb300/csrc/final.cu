@@ -937,10 +937,7 @@ __device__ __forceinline__ bool may_start(const FinArgs& A) {
     if (gtid() == 0) *A.f.count = (int64_t)st;
     return false;
   }
-  // a test knob: hold the last block back (a bounded sleep) so that the others' first barrier
-  // gives up; never set in normal use
-  if (A.hold_polls > 0 && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0)
-    for (int32_t i = 0; i < A.hold_polls; i++) __nanosleep(100);
+  hold_last_block(A.hold_polls);
   return true;
 }
 

@@ -48,6 +48,13 @@ static __device__ __noinline__ bool grid_barrier(unsigned* bar_count, int32_t* s
   return ok != 0;
 }
 
+// A test knob: the last block sleeps (a bounded time) before its first barrier, so that the others' wait
+// there gives up.  Never set in normal use.
+__device__ __forceinline__ void hold_last_block(int32_t hold_polls) {
+  if (hold_polls > 0 && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0)
+    for (int32_t i = 0; i < hold_polls; i++) __nanosleep(100);
+}
+
 __device__ __forceinline__ int64_t gtid() { return (int64_t)blockIdx.x * blockDim.x + threadIdx.x; }
 __device__ __forceinline__ int64_t gstride() { return (int64_t)gridDim.x * blockDim.x; }
 // This thread's index among all threads with the warps dealt round-robin over the blocks (warp w

@@ -67,6 +67,8 @@ struct SampleArgs {
   int32_t V;
   int32_t snap;  // whether the labels are wanted
   int32_t first;  // a thread's edges let in from the start
+  unsigned bar_polls;  // polls a barrier waits before it gives up
+  int32_t hold_polls;  // > 0: the last block sleeps this many ~100 ns polls before its first barrier
   int2* R;
   unsigned long long* H1;
   unsigned long long* H2;
@@ -110,8 +112,8 @@ __device__ __forceinline__ int2 climb(int2* R, const unsigned long long* H1, con
 // the numbers so far; `seen` is what they were before.  A barrier without numbers (n null) leaves
 // `seen` alone, and one stands between any two with numbers: a fast block may add its number for the
 // next barrier while a slow one still polls this one, but not for the one after.
-static __device__ __noinline__ bool sum_barrier(unsigned long long* word, int32_t* status, const unsigned* n,
-                                                unsigned* epoch, unsigned* seen, unsigned* sum) {
+static __device__ __noinline__ bool sum_barrier(unsigned long long* word, int32_t* status, unsigned polls,
+                                                const unsigned* n, unsigned* epoch, unsigned* seen, unsigned* sum) {
   __shared__ int ok;
   __shared__ unsigned got;
   __syncthreads();
@@ -125,7 +127,7 @@ static __device__ __noinline__ bool sum_barrier(unsigned long long* word, int32_
           asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(word) : "memory");
           return (int)((unsigned)w - target) >= 0;
         },
-        kSpinCap);
+        polls);
     if (!ok) set_status(status, BRIDGES_ETIMEDOUT_CODE);
     if (n) {
       got = (unsigned)(w >> 32) - *seen;
@@ -143,6 +145,7 @@ __global__ void __launch_bounds__(kThreads, 1) sample_kernel(SampleArgs A) {
   __shared__ unsigned epoch, seen, nlive;
   __shared__ unsigned won[2];
   if (threadIdx.x == 0) epoch = seen = nlive = won[0] = won[1] = 0;
+  hold_last_block(A.hold_polls);
   const Job J = job_of(A.b, A.V, 0);
   const int32_t V = A.V;
   int2* const R = A.R;
@@ -153,7 +156,7 @@ __global__ void __launch_bounds__(kThreads, 1) sample_kernel(SampleArgs A) {
   const uint32_t slot0 = (uint32_t)gspread(), nslots = (uint32_t)gstride();
   unsigned left = 0;  // live edges of the grid
   auto barrier = [&](const unsigned* n) {
-    return sum_barrier(reinterpret_cast<unsigned long long*>(ctl), A.b.status, n, &epoch, &seen, &left);
+    return sum_barrier(reinterpret_cast<unsigned long long*>(ctl), A.b.status, A.bar_polls, n, &epoch, &seen, &left);
   };
 
   for (int64_t x = gspread(); x < V; x += gstride()) {
@@ -375,6 +378,8 @@ void cert_sample(const Launch& L, const CertPlan& p, const CertBufs& b, const in
   a.groups = ceil_div(ceil_div(a.n, kGroup), a.stride);
   a.V = p.V;
   a.snap = p.cache;
+  a.bar_polls = L.bar_polls > 0 ? L.bar_polls : kSpinCap;
+  a.hold_polls = L.hold_polls;
   a.H1 = b.hook;
   a.H2 = b.hook + std::max(p.V, 1);
   a.R = b.roots;

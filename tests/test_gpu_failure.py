@@ -65,6 +65,36 @@ def test_final_stage_barrier_timeout_leaves_a_usable_context(cuda_lib):
     assert ctx.find(u, v, g.V, 4).cpu().numpy().tolist() == ref
 
 
+def test_sample_barrier_timeout_leaves_a_usable_context(cuda_lib):
+    """The same for the sampled certificate's barriers, which run before the final stage's: 20,000 vertices take
+    them on several blocks, with and without a stream behind the sample.  The certificate alone has no other
+    wait; every other call returns the status too, and the context is exact afterwards."""
+    V = 20_000
+    rng = np.random.default_rng(1)
+    for E in (60_000, 900_000):
+        hu, hv = (rng.integers(0, V, E).astype(np.int32) for _ in range(2))
+        u, v = torch.from_numpy(hu).cuda(), torch.from_numpy(hv).cuda()
+        ref = oracle.dfs_bridges(hu, hv, V).tolist()
+        cuts = oracle.articulation_points(hu, hv, V).tolist()
+        ctx = cuda_lib.Context(device="cuda:0")
+        assert ctx.find(u, v, V).cpu().numpy().tolist() == ref
+        ctx.set_opts(test_barrier_polls=1000, test_hold_polls=200_000)
+        for call in (ctx.certificate, ctx.find, ctx.two_edge_components, ctx.articulation_points, ctx.certificate):
+            with pytest.raises(cuda_lib.BridgesError) as ei:
+                call(u, v, V)
+            assert ei.value.code == -5
+        cnt = torch.zeros(2, dtype=torch.int64, device="cuda:0")
+        ctx.find(u, v, V, count_device=cnt[:1])
+        torch.cuda.synchronize()
+        assert int(cnt[0]) == -5
+        ctx.articulation_points(u, v, V, with_bridges=True, counts_device=cnt)
+        torch.cuda.synchronize()
+        assert cnt.tolist() == [-5, -5]
+        ctx.set_opts()
+        assert ctx.find(u, v, V).cpu().numpy().tolist() == ref
+        assert ctx.articulation_points(u, v, V).cpu().numpy().tolist() == cuts
+
+
 def test_injected_allocation_failure_leaves_the_context_usable(cuda_lib):
     """A device allocation that fails (injected with opts.test_fail_alloc: the n-th allocation of
     the context's own buffers fails as on a full device) makes that call return ENOMEM; the next

@@ -436,11 +436,14 @@ int32_t bridges_ctx_ap_stage_ms_history(const bridges_ctx* ctx, float* ms, int32
 
 /* ---------------------------------------------------------------------------------------
  * Autotuning.
- * bridges_autotune: times candidate plans on the given device-resident input (M in
+ * bridges_autotune: times the automatic plan and candidates on the given device-resident input (M in
  * {1,2,4,8,16,32}, fan-in 2 or M, warm-up 0.3/0.45/0.6/0.8/1.2/2.0 x V ln V edges, block 1024,
- * 768 or 512; `reps` timed calls each, CUDA events on `stream`), then the warm-up launch's block
- * size (128 to 1024) for the winner, and keeps the fastest in the context's options (read them
- * back whole with bridges_ctx_get_opts).  best[0..4] receives M, fan-in, warm-up edges, block
+ * 768 or 512; `reps` timed calls each, CUDA events on `stream`; none that runs the automatic plan's
+ * very kernels), then, for a winner with a warm-up prefix, that launch's block size (128 to 1024).
+ * A change is kept only when it is at least 0.5% faster, and the plan found is then timed against the
+ * automatic one, in turn, five more times: the automatic plan (warm-up edges -1, block 0) stays
+ * unless beaten by the same margin.  The plan kept goes to the context's options (read them
+ * back whole with bridges_ctx_get_opts); best[0..4] receives M, fan-in, warm-up edges, block
  * size and microseconds per call.  Uses a little scratch memory of its own (the output buffers).
  * Returns BRIDGES_OK or an error (the options are then unchanged).
  * bridges_ctx_set_opts: replaces the context's tuning options (e.g. from a cache of tuning

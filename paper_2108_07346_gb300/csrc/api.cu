@@ -1247,9 +1247,42 @@ extern "C" int32_t bridges_autotune(bridges_ctx* c, struct CUstream_st* stream, 
   cudaEventCreate(&e1);
   const bridges_opts saved = c->opts;
   const double lnv = std::log((double)V + 1.0);
-  float best_ms = 1e30f;
-  bridges_opts best_o = saved;
   int32_t rc = BRIDGES_OK;
+  // time of one call under options o (ms), or a negative value on error
+  auto time_opts = [&](const bridges_opts& o) -> float {
+    c->opts = o;
+    Carved k{};
+    int64_t r = run_path(c, s, u, v, E, V, 0, out, nullptr, &k, nullptr, Want::bridges);  // untimed: first use
+    cudaEventRecord(e0, s);
+    for (int i = 0; i < reps && !r; i++) r = run_path(c, s, u, v, E, V, 0, out, nullptr, &k, nullptr, Want::bridges);
+    cudaEventRecord(e1, s);
+    if (r || cudaEventSynchronize(e1) != cudaSuccess) {
+      rc = r ? (int32_t)r : (int32_t)BRIDGES_ECUDA;
+      return -1.0f;
+    }
+    float ms = 0;
+    cudaEventElapsedTime(&ms, e0, e1);
+    return ms / reps;
+  };
+  // the automatic plan comes first, and stays unless another is faster by more than the noise of a few calls
+  // (as in the batched tuner)
+  bridges_opts automatic = saved;
+  automatic.M = 1;
+  automatic.fan_in = 2;
+  automatic.block = 0;
+  automatic.warm_edges = -1;
+  automatic.warm_block = 0;
+  automatic.profile = 0;
+  bridges_opts best_o = automatic;
+  float best_ms = time_opts(automatic);
+  constexpr float kMargin = 0.995f;
+  auto consider = [&](const bridges_opts& o) {
+    const float ms = time_opts(o);
+    if (ms >= 0 && ms < best_ms * kMargin) {
+      best_ms = ms;
+      best_o = o;
+    }
+  };
   const int32_t Ms[] = {1, 2, 4, 8, 16, 32};
   const double warms[] = {0.3, 0.45, 0.6, 0.8, 1.2, 2.0};
   const int32_t blocks[] = {1024, 768, 512};
@@ -1260,64 +1293,46 @@ extern "C" int32_t bridges_autotune(bridges_ctx* c, struct CUstream_st* stream, 
       if (M > 1 && f == 2 && M == 2) continue;  // same as f = M
       for (double w : warms) {
         for (int32_t blk : blocks) {
-          bridges_opts o = saved;
+          if (rc) break;
+          bridges_opts o = automatic;
           o.M = M;
           o.fan_in = f;
           o.block = blk;
           o.warm_edges = (int64_t)std::ceil(w * V * lnv) + 4096;
-          o.profile = 0;
           c->opts = o;
-          // one untimed run (workspace growth, first-touch), then reps timed runs
-          int64_t r = BRIDGES_OK;
-          Carved k{};
-          r = run_path(c, s, u, v, E, V, 0, out, nullptr, &k, nullptr, Want::bridges);
-          if (r) {
-            rc = (int32_t)r;
-            break;
-          }
-          cudaEventRecord(e0, s);
-          for (int i = 0; i < reps && !r; i++) r = run_path(c, s, u, v, E, V, 0, out, nullptr, &k, nullptr, Want::bridges);
-          cudaEventRecord(e1, s);
-          if (r || cudaEventSynchronize(e1) != cudaSuccess) {
-            rc = r ? (int32_t)r : (int32_t)BRIDGES_ECUDA;
-            break;
-          }
-          float ms = 0;
-          cudaEventElapsedTime(&ms, e0, e1);
-          ms /= reps;
-          if (ms < best_ms) {
-            best_ms = ms;
-            best_o = o;
-          }
+          const CertPlan p = plan_for(c, E, V, 0);
+          // one kernel whatever the choices, or one certified whole by a sample, whose launch has its own shape
+          if (small_call(c, p) || (p.sampled && !p.cache)) continue;
+          consider(o);
         }
-        if (rc) break;
       }
-      if (rc) break;
     }
-    if (rc) break;
   }
-  // refinement: the warm-up launch's block size for the chosen plan
-  for (int32_t wb : {128, 256, 512, 1024}) {
-    if (rc) break;
-    bridges_opts o = best_o;
-    o.warm_block = wb;
-    o.profile = 0;
-    c->opts = o;
-    Carved k{};
-    int64_t r = run_path(c, s, u, v, E, V, 0, out, nullptr, &k, nullptr, Want::bridges);
-    cudaEventRecord(e0, s);
-    for (int i = 0; i < reps && !r; i++) r = run_path(c, s, u, v, E, V, 0, out, nullptr, &k, nullptr, Want::bridges);
-    cudaEventRecord(e1, s);
-    if (r || cudaEventSynchronize(e1) != cudaSuccess) {
-      rc = r ? (int32_t)r : (int32_t)BRIDGES_ECUDA;
-      break;
+  // refinement: the warm-up launch's block size for the chosen plan, where it has such a launch
+  c->opts = best_o;
+  if (!plan_for(c, E, V, 0).sampled) {
+    for (int32_t wb : {128, 256, 512, 1024}) {
+      if (rc) break;
+      bridges_opts o = best_o;
+      o.warm_block = wb;
+      consider(o);
     }
-    float ms = 0;
-    cudaEventElapsedTime(&ms, e0, e1);
-    ms /= reps;
-    if (ms < best_ms) {
-      best_ms = ms;
-      best_o = o;
+  }
+  // the search's plan against the automatic one, timed in turn over more calls
+  auto same = [](const bridges_opts& x, const bridges_opts& y) {
+    return x.M == y.M && x.block == y.block && x.warm_edges == y.warm_edges && x.warm_block == y.warm_block;
+  };
+  if (!rc && !same(best_o, automatic)) {
+    float t_best = 0, t_auto = 0;
+    for (int k = 0; k < 5 && !rc; k++) {
+      t_auto += time_opts(automatic);
+      t_best += time_opts(best_o);
+    }
+    if (t_best < t_auto * kMargin) {
+      best_ms = t_best / 5;
+    } else {
+      best_o = automatic;
+      best_ms = t_auto / 5;
     }
   }
   cudaEventDestroy(e0);

@@ -221,8 +221,9 @@ int32_t bridges_ctx_get_batch_plan(const bridges_ctx* ctx, bridges_batch_plan* p
  * partition splits of 2^18 to 2^22 edges or automatic, and warm-up prefixes of 2V + 1024, 4V + 2048
  * and 8V + 2048 edges, each timed over `reps` batched calls (CUDA events on `stream`).  A change
  * is kept only when it is at least 0.5% faster (the timing noise of a few calls), and the plan
- * found is then timed against the automatic plan, in turn, three more times: the automatic plan
- * stays unless beaten by the same margin.  The plan kept goes to the context and to *best (may be
+ * found is then timed against the automatic plan, in turn, three more times, in calls enqueued behind
+ * one another and in calls waited for one by one: the automatic plan stays unless beaten by the same
+ * margin in the first and equalled in the second.  The plan kept goes to the context and to *best (may be
  * NULL); *best_us (may be NULL) gets its microseconds per batch.  Graphs above 4,096 vertices are not batched and not tuned.  Uses
  * the context's batched buffers; returns BRIDGES_OK or an error (the plan is then unchanged). */
 int32_t bridges_batch_autotune(bridges_ctx* ctx, struct CUstream_st* stream, const int32_t* edges_u,

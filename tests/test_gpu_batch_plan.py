@@ -1,4 +1,6 @@
-"""Batches planned on the device (256 graphs and more) against the same graphs in batches that the host plans."""
+"""Batches planned on the device (256 graphs and more) against the same graphs in batches that the host plans; a tuned plan in calls that are waited for."""
+
+import time
 
 import numpy as np
 import pytest
@@ -46,3 +48,31 @@ def test_planned_on_device_equals_host(G, split):
         want += results(ctx, u, v, off[a:b + 1], Vs[a:b])
     assert got == want
     assert got[4][0] < 0 and sum(c for c, _ in got) > 100
+
+
+def test_a_tuned_plan_is_no_slower_when_waited_for():
+    """2,048 graphs of 300 to 500 vertices: a shorter prefix gains a few microseconds in batches enqueued behind one
+    another, and costs the device's planning (120 us) where each batch is waited for."""
+    G = 2048
+    rng = np.random.default_rng(3)
+    Vs = rng.integers(300, 500, G).astype(np.int32)
+    Es = Vs.astype(np.int64) * (Vs - 1) // 4
+    off = np.concatenate([[0], np.cumsum(Es)]).astype(np.int64)
+    size = torch.from_numpy(np.repeat(Vs, Es)).cuda()
+    u, v = (torch.randint(0, 1 << 30, size.shape, dtype=torch.int32, device="cuda").remainder_(size) for _ in range(2))
+    ctx = pb.Context()
+
+    def waited():
+        out, counts, _ = ctx.find_batched(u, v, off, Vs)
+        times = []
+        for _ in range(21):
+            t = time.perf_counter()
+            ctx.find_batched(u, v, off, Vs, out=out, counts=counts)
+            times.append(time.perf_counter() - t)
+        return sorted(times)[10], counts.cpu().numpy()
+
+    fresh, want = waited()
+    ctx.batch_autotune(u, v, off, Vs)
+    tuned, got = waited()
+    assert np.array_equal(got, want)
+    assert tuned < 1.15 * fresh

@@ -208,11 +208,12 @@ void scheduler(bridges_server* S) {
     bool busy = false;
     for (const SrvSlot& sl : S->slots) busy = busy || sl.busy;
     if (S->stop && !busy && S->queue.empty()) break;
-    // short waits while work is in flight (completion is polled), long ones when idle
+    // short waits while work is in flight (completion is polled), long ones when idle.  A request that came
+    // while admit had the lock released has notified nobody: the idle wait looks at the queue first
     if (busy)
       S->cv_work.wait_for(lk, std::chrono::microseconds(20));
     else
-      S->cv_work.wait_for(lk, std::chrono::milliseconds(50));
+      S->cv_work.wait_for(lk, std::chrono::milliseconds(50), [&] { return S->stop || !S->queue.empty(); });
   }
 }
 

@@ -165,3 +165,30 @@ def test_cancel_withdraws_queued_requests(cuda_lib):
     with pytest.raises(cuda_lib.BridgesError):
         srv.cancel(t)  # released
     srv.close()
+
+
+def test_a_request_behind_a_failing_one_is_not_left_waiting(cuda_lib):
+    """A request that arrives while the scheduler enqueues another (its lock released then) is launched right after
+    it, also when that one fails and leaves nothing in flight.  The second device allocation of the server's one
+    slot fails, in a batch that outgrows its buffers (freeing them first takes the scheduler a while); the next
+    request is submitted a varying time later."""
+    import time
+
+    pair = dev([0, 1]), dev([1, 2])
+    late = []
+    for k in range(24):
+        srv = cuda_lib.Server(device="cuda:0", max_slots=1, test_fail_alloc=2)
+        assert len(srv.wait(srv.submit(*pair, 64))[0]) == 2
+        a = srv.submit(*pair, 4096)
+        end = time.perf_counter() + 5e-5 * k
+        while time.perf_counter() < end:
+            pass
+        b = srv.submit(*pair, 64)
+        got, latency = srv.wait(b)
+        assert got.cpu().numpy().tolist() == [[0, 1], [1, 2]]
+        with pytest.raises(cuda_lib.BridgesError) as ei:
+            srv.wait(a)
+        assert ei.value.code == -3
+        late.append(latency)
+        srv.close()
+    assert max(late) < 30  # (an idle scheduler looks again after 50 ms)

@@ -51,10 +51,13 @@ namespace {
 
 constexpr int kThreads = 1024;
 constexpr int kMaxRounds = 24;  // rounds before the remaining edges take the union-finds one by one
-// Live edges that take the union-finds one by one, and at most V / 2 (what a round more or less costs: 2.5 M
-// edges on 37,147 vertices 70.7 us with 8,192 and V / 4, 66.8 with these; 110 k on 90,000: 66.8 and 57.5; 9 k on 8,000:
-// 45.6 and 39.7; with V, 30 k on 20,000 take 108 us instead of 59: the sets have not met yet).
-constexpr unsigned kFewLive = 32768;
+// Live edges that take the union-finds one by one, and at most V / 4.  They gain a round or two where they are
+// the last ones, but where their sets have yet to meet (sparse random lists around the densities at which F or
+// F' forms its large set), every link chases the others' roots.  Over random lists of 0.55 V to 10 V edges on 5,000
+// to 113,000 vertices and lists of clusters and R-MAT graphs, mean and worst against the best of eleven limits:
+// 32,768 and V / 2 84.6 us and 4.0 times (60,000 vertices, 123,000 edges: 299 us instead of 74), 8,192 and V / 4
+// 70.6 and 2.2 times, 4,096 and V / 4 70.3 and 1.27, 1,024 and V / 16 72.2 and 1.36.
+constexpr unsigned kFewLive = 4096;
 constexpr int kGroup = 8;       // edges per group of the sample (kSampleShift)
 static_assert(kGroup == 1 << kSampleShift, "the stream's test of a sampled edge");
 
@@ -261,7 +264,7 @@ __global__ void __launch_bounds__(kThreads, 1) sample_kernel(SampleArgs A) {
     if (threadIdx.x == 0) nlive = 0;
 
     // C: new roots, at the end also for the union-finds
-    const bool last = all_in && left <= min(kFewLive, (unsigned)V / 2);
+    const bool last = all_in && left <= min(kFewLive, (unsigned)V / 4);
     for (int64_t x = gspread(); x < V; x += gstride()) {
       int2 r = R[x];
       const unsigned long long h1 = H1[r.x], h2 = H2[r.y];

@@ -190,3 +190,21 @@ def test_stream_in_one_wave(cuda_lib, V, opts):
         want = [[V - 1 + i, V + i] for i in range(39)]
         inner = got[got[:, 1] < V]
         assert got[got[:, 1] >= V].tolist() == want and (V > 113_000 or len(inner) == 0)
+
+
+@pytest.mark.parametrize("V", [60_000, 100_000])
+def test_sparse_lists_take_one_another_s_time(cuda_lib, V):
+    """Sparse random lists around the densities at which F and F' form their large sets: the sample's time changes
+    little from one to the next (three to four times the others' when its last edges link before their sets meet)."""
+    import torch
+
+    gen = torch.Generator(device="cuda").manual_seed(V)
+    times = {}
+    for d in (0.85, 0.95, 1.05, 1.15, 1.5, 1.85, 1.95, 2.05, 2.15, 2.5):
+        u, v = (torch.randint(0, V, (int(d * V),), dtype=torch.int32, device="cuda", generator=gen) for _ in range(2))
+        ctx = cuda_lib.Context(device="cuda:0", profile=True)
+        for _ in range(9):
+            got = ctx.find(u, v, V)
+        times[d] = sorted(t["warmup"] for t in ctx.stage_ms_history(8))[4]
+        assert got.cpu().numpy().tolist() == oracle.dfs_bridges(u.cpu().numpy(), v.cpu().numpy(), V).tolist()
+    assert max(times.values()) < 2 * sorted(times.values())[len(times) // 2], times

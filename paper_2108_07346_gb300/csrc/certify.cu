@@ -519,7 +519,12 @@ CertPlan make_plan(int64_t E, int32_t V, int32_t M, int32_t fan_in, int32_t bloc
   };
   int cps = ctas_per_sm;
   p.block = block;
-  if (cps <= 0 && block <= 0)
+  if (cps <= 0 && warm == 0)
+    // no snapshot, every edge to the union-finds: the blocks of the later waves start when sets have formed
+    // (calls with one wave of 304 blocks and with 608: 500 vertices, 200 k edges 503 and 284 us; 3,000, 300 k: 520
+    // and 279; 60,000, 720 k: 707 and 263; 20,000, 80 k: 164 and 159)
+    cps = 4;
+  else if (cps <= 0 && block <= 0)
     cps = fits ? (resident(512) >= 2 ? 2 : 1) : 2;
   else if (cps <= 0)
     cps = fits ? std::max(1, std::min(2, resident(block))) : 2;
@@ -530,9 +535,6 @@ CertPlan make_plan(int64_t E, int32_t V, int32_t M, int32_t fan_in, int32_t bloc
   // two blocks of 512 per SM, 561 us a call, 687 in one wave without the staging)
   p.stage = snap + stage_bytes(p.block) + 1024 <= smem_optin;
   p.G = (int32_t)std::max<int64_t>(1, ((int64_t)num_sms * cps) / p.M);
-  // a short list takes fewer blocks, one 16-byte unit of each array per thread (130 k edges: 18 us with
-  // 608 blocks, 12 with 64)
-  if (p.M == 1) p.G = (int32_t)std::max<int64_t>(1, std::min<int64_t>(p.G, ceil_div(E, 4 * (int64_t)p.block)));
   p.warm_block = p.block;
   const int64_t chunk = ceil_div(std::max<int64_t>(E, 1), p.M);
   p.sampled = p.M == 1 && labels_fit && warm != 0;
@@ -555,6 +557,9 @@ CertPlan make_plan(int64_t E, int32_t V, int32_t M, int32_t fan_in, int32_t bloc
     if (p.stride <= 1) warm = std::max(warm, E);
     p.cache = E > warm;
     p.warm = warm;
+    // behind a sample few edges link, and a short list takes fewer blocks, one 16-byte unit of each array per
+    // thread (130 k edges: 18 us with 608 blocks, 12 with 64)
+    p.G = (int32_t)std::max<int64_t>(1, std::min<int64_t>(p.G, ceil_div(E, 4 * (int64_t)p.block)));
     p.warm_block = p.block;
     return p;
   }

@@ -208,3 +208,23 @@ def test_sparse_lists_take_one_another_s_time(cuda_lib, V):
         times[d] = sorted(t["warmup"] for t in ctx.stage_ms_history(8))[4]
         assert got.cpu().numpy().tolist() == oracle.dfs_bridges(u.cpu().numpy(), v.cpu().numpy(), V).tolist()
     assert max(times.values()) < 2 * sorted(times.values())[len(times) // 2], times
+
+
+@pytest.mark.parametrize("V,opts", [(3000, {"warm_edges": 0}), (60_000, {"warm_edges": 0}), (130_000, {}),
+                                    (500_000, {})])
+def test_grid_of_a_list_that_links_edge_by_edge(cuda_lib, V, opts):
+    """Without a sample every edge, or most of them, take the union-finds: a short list has as many blocks as a long
+    one, and without a snapshot as many as four per SM."""
+    import torch
+
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    grids = set()
+    for E in (20_000, 200_000, 3_000_000):
+        rng = np.random.default_rng(E)
+        u, v = _er(rng, V, E)
+        du, dv = torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda()
+        ctx = cuda_lib.Context(device="cuda:0", **opts)
+        assert ctx.find(du, dv, V).cpu().numpy().tolist() == oracle.dfs_bridges(u, v, V).tolist()
+        grids.add(ctx.last_config()["blocks_per_partition"])
+    assert len(grids) == 1
+    assert not opts or grids == {4 * sms}

@@ -187,10 +187,18 @@ struct LeafArgs {
   CertBufs b;
 };
 
+constexpr int kProbes = 256;  // vertices probed for the bitmap's component
+
 // Forest pass over the partitions: block -> (job j = blockIdx / G, member m = blockIdx % G);
 // the job's G members share its chunk [E j / M, E (j+1) / M) (Sec. 3 partition): the warm-up
 // prefix in one slice per member, the cached pass in interleaved tiles when the chunk is long
 // enough (use_tiles), else in slices too.
+//
+// Behind a bitmap that marks next to nothing (the component it found holds fewer than a 32nd of the probed
+// vertices: F' has no large one yet, as in a sparse random list) every edge links, and a chunk of fewer vertices
+// than four times the threads goes faster on half of them: random lists on 120,000 to 200,000 vertices,
+// the pass of 4 V edges 190-295 us on 304 blocks and 156-276 on 152, of 6 V 242-557 and 160-211, of 20 V
+// 213-317 and 123-207; 300,000 vertices, 3 V: 311-338 and 195-199; 10^6: 362-401 and 360-379.
 template <int MODE, bool VEC>
 __global__ void __launch_bounds__(1024, 1) leaf_kernel(LeafArgs A) {
   extern __shared__ __align__(16) uint16_t slab[];
@@ -199,6 +207,12 @@ __global__ void __launch_bounds__(1024, 1) leaf_kernel(LeafArgs A) {
   __syncthreads();
   if (stop) return;  // an earlier step failed: its labels and union-finds may be unset
   const int64_t j = blockIdx.x / A.G, m = blockIdx.x % A.G;
+  int64_t members = A.G;
+  if (MODE == 2 && A.mode == 1 && (A.b.giant[j] >> 32) < kProbes / 32 && A.G > 1 &&
+      4 * members * (int64_t)blockDim.x > A.V) {
+    members /= 2;
+    if (m >= members) return;
+  }
   const int64_t lo = A.E * j / A.M, hi = A.E * (j + 1) / A.M;
   const int64_t w = A.stride > 1 ? 0 : min(A.warm, hi - lo);
   int64_t a = A.mode == 0 ? lo : lo + w;
@@ -219,11 +233,11 @@ __global__ void __launch_bounds__(1024, 1) leaf_kernel(LeafArgs A) {
                  staged[warp]};
   const ForestSink S{J, win, A.V, A.b.status, A.u, A.mode == 1 ? A.stride : 0};
   const uint32_t clampv = MODE == 2 ? (uint32_t)A.Vb : (uint32_t)A.V;
-  if (A.mode == 1 && use_tiles<VEC>(a, z, A.G, blockDim.x, kUnroll)) {
-    stream_range<MODE, VEC, kUnroll>(S, A.u, A.v, a, z, clampv, slab, m, A.G, A.queue);
+  if (A.mode == 1 && use_tiles<VEC>(a, z, members, blockDim.x, kUnroll)) {
+    stream_range<MODE, VEC, kUnroll>(S, A.u, A.v, a, z, clampv, slab, m, members, A.queue);
   } else {
     const int64_t n = z - a;
-    const int64_t s = a + n * m / A.G, t = a + n * (m + 1) / A.G;
+    const int64_t s = a + n * m / members, t = a + n * (m + 1) / members;
     stream_range<MODE, VEC, kUnroll>(S, A.u, A.v, s, t, clampv, slab);
   }
   if (A.stage_at < 0) return;
@@ -367,8 +381,6 @@ __global__ void snap_roots_kernel(CertBufs b, int32_t V, int64_t step, int64_t n
 // 1) the component: the most frequent root among 256 vertices spread over [0, V) (any component would be
 //    exact; counting every vertex took 46 us on 2^20 vertices, the giant's counter taking an atomic from
 //    every warp)
-constexpr int kProbes = 256;
-
 __global__ void __launch_bounds__(kProbes) bm_probe_kernel(CertBufs b, int32_t V, int64_t njobs) {
   __shared__ int32_t probe[kProbes];
   __shared__ unsigned best;
@@ -381,7 +393,8 @@ __global__ void __launch_bounds__(kProbes) bm_probe_kernel(CertBufs b, int32_t V
   for (int k = 0; k < kProbes; k++) same += probe[k] == mine;
   atomicMax(&best, same << 8 | (unsigned)(kProbes - 1 - threadIdx.x));
   __syncthreads();
-  if (threadIdx.x == 0) b.giant[j] = (unsigned long long)(uint32_t)probe[kProbes - 1 - (best & (kProbes - 1))];
+  if (threadIdx.x == 0)
+    b.giant[j] = (unsigned long long)(best >> 8) << 32 | (uint32_t)probe[kProbes - 1 - (best & (kProbes - 1))];
 }
 
 // 2) the bitmap words (in the job's label area): bit x set iff x < min(V, Vb) lies in that component; the

@@ -66,7 +66,7 @@ struct CertBufs {
   int2* roots;               // [V] its roots in both forests (scratch of the final stage, idle until then)
   int32_t* cnt;     // [2*M] forest sizes |F|, |F'| per job
   int32_t* nlab;    // [M] labels handed out per job
-  unsigned long long* giant;  // [M] bitmap snapshot: root of the F' component it marks
+  unsigned long long* giant;  // [M] bitmap snapshot: how many probes met the F' component it marks, its root
   int32_t* P1;
   int32_t* P2;
   int32_t* f1u;

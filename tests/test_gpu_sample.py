@@ -228,3 +228,24 @@ def test_grid_of_a_list_that_links_edge_by_edge(cuda_lib, V, opts):
         grids.add(ctx.last_config()["blocks_per_partition"])
     assert len(grids) == 1
     assert not opts or grids == {4 * sms}
+
+
+def test_bitmap_of_nothing_halves_the_grid(cuda_lib):
+    """Sparse random lists on more vertices than labels, whose prefix leaves F' without a large component: the
+    automatic pass takes about the time of one block of 512 per SM (1.6 times it on the whole grid)."""
+    import torch
+
+    total = {}
+    for V in (120_000, 160_000, 200_000):
+        for d in (4, 6, 20):
+            gen = torch.Generator(device="cuda").manual_seed(V + d)
+            u, v = (torch.randint(0, V, (d * V,), dtype=torch.int32, device="cuda", generator=gen) for _ in range(2))
+            found = []
+            for name, opts in (("auto", {}), ("half", {"ctas_per_sm": 1, "block": 512})):
+                ctx = cuda_lib.Context(device="cuda:0", profile=True, **opts)
+                for _ in range(9):
+                    got = ctx.find(u, v, V)
+                total[name] = total.get(name, 0) + sorted(t["forest"] for t in ctx.stage_ms_history(8))[4]
+                found.append(got.cpu().numpy().tolist())
+            assert found[0] == found[1] == oracle.dfs_bridges(u.cpu().numpy(), v.cpu().numpy(), V).tolist()
+    assert total["auto"] < 1.3 * total["half"], total

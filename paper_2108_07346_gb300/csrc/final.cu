@@ -1000,9 +1000,13 @@ constexpr int kCntRest = 7;
 constexpr int32_t kCyclicMin = 4096;  // kept edges above which a graph with many cycles is not reduced
 constexpr int kStripSteps = 8;
 constexpr int32_t kHub = 64;
-constexpr int32_t kCoreMax = 5632;  // the largest layout that fits a block's shared memory
+// Vertices of a core that block 0 solves at most: what fits the shared memory that the sort asks for anyway.
+// More would come out of every block's L1, through which the phases on the grid gather (216 KB for a core of
+// 5,632: a round of list ranking 24 us in place of 12.6 on 500,000 vertices, 6.0 and 3.9 on 100,000), and a core
+// of 4,000 vertices takes the grid no longer than one block.
+constexpr int32_t kCoreMax = 3616;
 using CoreLayout = Layout<kCoreMax>;
-static_assert(kCoreMax % 32 == 0 && CoreLayout::kBytes + 3072 <= 227 * 1024, "the core's layout fits a block");
+static_assert(kCoreMax % 32 == 0 && CoreLayout::kBytes <= (int)kSmemSort, "the core's layout fits beside the L1");
 
 // Appends one item per lane that has one; the place of each, counted in *n per warp.
 __device__ __forceinline__ int32_t warp_place(bool has, int32_t* n) {
@@ -1482,8 +1486,7 @@ void launch_final(const Launch& L, const void* kernel, int32_t V, size_t smem, v
 bool final_prepare() {
   const size_t most = std::max(kSmemTables, kSmemSort);
   return cudaFuncSetAttribute(final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) == cudaSuccess &&
-         cudaFuncSetAttribute(reduced_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)std::max(most, (size_t)CoreLayout::kBytes)) == cudaSuccess;
+         cudaFuncSetAttribute(reduced_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) == cudaSuccess;
 }
 
 void final_stage(const Launch& L, const FinalBufs& f, int32_t V, const int32_t* tu, const int32_t* tv,
@@ -1519,7 +1522,6 @@ void reduced_stage(const Launch& L, const FinalBufs& f, const CertBufs& c, int32
   R.d_nx = c.cnt + 1;
   R.P2 = c.P2;
   R.tmp = c.tmp;
-  smem = std::max(smem, (size_t)CoreLayout::kBytes);
   void* args[] = {&R};
   launch_final(L, (const void*)reduced_kernel, V, smem, args);
 }

@@ -964,15 +964,14 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
 //   1  P2 flattened: every vertex's F' root.  F edges between two roots are kept.
 //   2  F' has V - |F'| components and F has V - |F|, each of them some whole ones of F': the reduced graph's
 //      spanning forests have |F| - |F'| edges.  If the kept edges are that many, it is a forest and all of
-//      them are bridges.  If they are many more (a sparse graph with cycles throughout), the reduction
-//      gained little and the phases above run on F and F' as they are.  Else the roots with kept edges are
-//      numbered.
+//      them are bridges.  If the reduction gained little (stays_whole), the phases above run on F and F' as
+//      they are.  Else the roots with kept edges are numbered.
 //   3  Else leaves are stripped.  The one edge of a vertex of degree 1 is a bridge; without it its other
 //      end may be the next leaf, and the thread goes on there (at most kStripSteps times, so that a long
 //      path does not run in one thread; vertices of kHub edges and more keep their degree, so that their
 //      leaves do not queue on them).
-//   4  What is left, the cycles and what joins them, is solved by block 0 in shared memory when it has at
-//      most kCoreMax vertices, else by every block: a spanning forest of it, then the phases above.
+//   4  What is left, the cycles and what joins them, is solved by block 0 in shared memory when it is small
+//      (block_solves), else by every block: a spanning forest of it, then the phases above.
 //   5  The keys are sorted, as above.
 // 2.5 M edges on 37,147 vertices: 79 us with the phases above on the whole forest, 18 us so (25 with the
 // roots numbered before it was known that all kept edges are bridges); 16.8 M R-MAT edges on 2^20 vertices
@@ -997,7 +996,6 @@ constexpr int kCoreVerts = 4;
 constexpr int kCoreEdges = 5;
 constexpr int kCntTree = 6;
 constexpr int kCntRest = 7;
-constexpr int32_t kCyclicMin = 4096;  // kept edges above which a graph with many cycles is not reduced
 constexpr int kStripSteps = 8;
 constexpr int32_t kHub = 64;
 // Vertices of a core that block 0 solves at most: what fits the shared memory that the sort asks for anyway.
@@ -1005,8 +1003,37 @@ constexpr int32_t kHub = 64;
 // 5,632: a round of list ranking 24 us in place of 12.6 on 500,000 vertices, 6.0 and 3.9 on 100,000), and a core
 // of 4,000 vertices takes the grid no longer than one block.
 constexpr int32_t kCoreMax = 3616;
+constexpr int32_t kChainCore = 1536;  // ... and of a core with few edges beyond a forest
 using CoreLayout = Layout<kCoreMax>;
 static_assert(kCoreMax % 32 == 0 && CoreLayout::kBytes <= (int)kSmemSort, "the core's layout fits beside the L1");
+
+// Whether the phases run on F and F' as they are: of V vertices' graph the reduced one has `kept` edges, `extra` of
+// them beyond a spanning forest.  Numbering, degrees, strip and the listing of the core cost about 25 us and 0.6 us
+// for every 1,000 kept edges, and a large core comes to the phases in the end; the phases alone cost 55 us at
+// 1,000 vertices, 75 at 20,000, 125 at 100,000, 205 at 300,000.  Phases and reduction, us for the stage:
+//   most of the graph kept: random lists of V edges on 20,000 vertices 75 and 124, 100,000 127 and 215, 300,000 205
+//   and 404; a cycle of 500 46 and 59, of 20,000 65 and 151 -- but a list next to a forest on a million vertices
+//   (550 k edges) 448 and 393, and of up to 4,096 kept edges those with many cycles (1.5 V edges on 2,000 vertices)
+//   59 and 53;
+//   an eighth of it, with cycles: 2 V edges on 50,000 vertices 81 and 100, 300,000 213 and 285;
+//   less of it: 3 V edges on 20,000 vertices 73 and 44, 300,000 168 and 70; R-MAT on 2^18 vertices 176 and 88.
+constexpr int32_t kManyKept = 4096;
+
+__device__ __forceinline__ bool stays_whole(int32_t V, int32_t kept, int32_t extra) {
+  const bool many = kept > kManyKept;
+  if (kept > V / 2) {
+    if (!many) return 5 * extra < 2 * kept;
+    return V <= 4 * gstride() || extra >= kept / 256;
+  }
+  return many && kept > V / 8 && extra > kept / 8;
+}
+
+// Whether block 0 solves the core of VC vertices and mc edges.  A core that is mostly cycles without chords takes
+// one block long (a cycle of 1,000 edges 94 us for the stage, 2,000 149; the grid 92 for 4,000), one with twice as
+// many edges as vertices shrinks at once when its own second forest is contracted (3,140 vertices, 8,373 edges: 70).
+__device__ __forceinline__ bool block_solves(int32_t VC, int32_t mc) {
+  return VC <= kCoreMax && (VC <= kChainCore || mc >= 2 * VC);
+}
 
 // Appends one item per lane that has one; the place of each, counted in *n per warp.
 __device__ __forceinline__ int32_t warp_place(bool has, int32_t* n) {
@@ -1198,7 +1225,7 @@ __global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
     write_count(A);
     return;
   }
-  if (kept > kCyclicMin && kept > span + span / 4) {
+  if (stays_whole(V, kept, kept - span)) {
     FinArgs B = A;
     B.orig = nullptr;
     B.ou = A.tu;
@@ -1268,11 +1295,12 @@ __global__ void __launch_bounds__(kThreads) reduced_kernel(ReducedArgs R) {
   if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
   // 4
   const int32_t VC = cnt[kCoreVerts], mc = cnt[kCoreEdges];
-  if (mc > 0 && VC <= kCoreMax) {
+  const bool on_block = mc > 0 && block_solves(VC, mc);
+  if (on_block) {
     if (blockIdx.x == 0) solve_core(R, reinterpret_cast<char*>(sm), gs, id2, cu, cv, cs, VC, mc);
     if (!grid_barrier(f, A.bar_polls, &bar_epoch)) return;
   }
-  const bool on_grid = mc > 0 && VC > kCoreMax;
+  const bool on_grid = mc > 0 && !on_block;
   if (on_grid || *f.nkeys > kRankMax) {  // the keys so far by value: the sort of many, and the phases, need the room
     const int32_t found = *f.nkeys;
     for (int64_t i = gspread(); i < found; i += gstride()) f.keys[i] = resolved(A, ko, f.keys[i]);

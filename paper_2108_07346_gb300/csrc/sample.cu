@@ -115,39 +115,52 @@ __device__ __forceinline__ int2 climb(int2* R, const unsigned long long* H1, con
 // the numbers so far; `seen` is what they were before.  A barrier without numbers (n null) leaves
 // `seen` alone, and one stands between any two with numbers: a fast block may add its number for the
 // next barrier while a slow one still polls this one, but not for the one after.
-static __device__ __noinline__ bool sum_barrier(unsigned long long* word, int32_t* status, unsigned polls,
-                                                const unsigned* n, unsigned* epoch, unsigned* seen, unsigned* sum) {
-  __shared__ int ok;
-  __shared__ unsigned got;
+// What a block keeps between its barriers is in shared memory (as arguments it cost the kernel registers).
+struct SumBarrier {
+  unsigned long long* word;
+  int32_t* status;
+  unsigned polls;  // before it gives up
+  unsigned epoch, seen;
+  unsigned sum;
+  int ok;
+};
+
+static __device__ __noinline__ bool sum_barrier(SumBarrier* s, const unsigned* n) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    const unsigned target = (*epoch += 1) * gridDim.x;
+    const unsigned target = (s->epoch += 1) * gridDim.x;
+    unsigned long long* const word = s->word;
     const unsigned long long add = (unsigned long long)(n ? *n : 0u) << 32 | 1ull;
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(word), "l"(add) : "memory");
     unsigned long long w = 0;
-    ok = bounded_poll(
+    const bool ok = bounded_poll(
         [&] {
           asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(word) : "memory");
           return (int)((unsigned)w - target) >= 0;
         },
-        polls);
-    if (!ok) set_status(status, BRIDGES_ETIMEDOUT_CODE);
+        s->polls);
+    if (!ok) set_status(s->status, BRIDGES_ETIMEDOUT_CODE);
+    s->ok = ok;
     if (n) {
-      got = (unsigned)(w >> 32) - *seen;
-      *seen = (unsigned)(w >> 32);
+      s->sum = (unsigned)(w >> 32) - s->seen;
+      s->seen = (unsigned)(w >> 32);
     }
   }
   __syncthreads();
-  if (n) *sum = got;
-  return ok != 0;
+  return s->ok != 0;
 }
 
 // K edges per thread.
 template <int K>
 __global__ void __launch_bounds__(kThreads, 1) sample_kernel(SampleArgs A) {
-  __shared__ unsigned epoch, seen, nlive;
-  __shared__ unsigned won[2];
-  if (threadIdx.x == 0) epoch = seen = nlive = won[0] = won[1] = 0;
+  __shared__ SumBarrier bar;
+  __shared__ unsigned nlive, won[2];
+  if (threadIdx.x == 0) {
+    bar.word = reinterpret_cast<unsigned long long*>(A.b.ctl);
+    bar.status = A.b.status;
+    bar.polls = A.bar_polls;
+    bar.epoch = bar.seen = nlive = won[0] = won[1] = 0;
+  }
   hold_last_block(A.hold_polls);
   const Job J = job_of(A.b, A.V, 0);
   const int32_t V = A.V;
@@ -159,7 +172,9 @@ __global__ void __launch_bounds__(kThreads, 1) sample_kernel(SampleArgs A) {
   const uint32_t slot0 = (uint32_t)gspread(), nslots = (uint32_t)gstride();
   unsigned left = 0;  // live edges of the grid
   auto barrier = [&](const unsigned* n) {
-    return sum_barrier(reinterpret_cast<unsigned long long*>(ctl), A.b.status, A.bar_polls, n, &epoch, &seen, &left);
+    if (!sum_barrier(&bar, n)) return false;
+    if (n) left = bar.sum;
+    return true;
   };
 
   for (int64_t x = gspread(); x < V; x += gstride()) {

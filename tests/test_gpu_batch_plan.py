@@ -7,6 +7,7 @@ import pytest
 import torch
 
 import graphgen
+import oracle
 import paper_2108_07346_gb300 as pb
 
 pytestmark = pytest.mark.gpu
@@ -48,6 +49,42 @@ def test_planned_on_device_equals_host(G, split):
         want += results(ctx, u, v, off[a:b + 1], Vs[a:b])
     assert got == want
     assert got[4][0] < 0 and sum(c for c, _ in got) > 100
+
+
+@pytest.mark.parametrize("large", [False, True])
+def test_batches_behind_one_another(large):
+    """A batch planned on the device, and behind it, not waited for, batches that the host plans (the last one is
+    still running) and a single call, all on one context; then, idle again, one more of the first kind.  With and
+    without graphs above the shared-memory size among them."""
+    G = 400
+    rng = np.random.default_rng(9)
+    sizes = [5, 300, 1000, 2000, 4096] + ([5000] if large else [])
+    Vs = rng.choice(sizes, G).astype(np.int32)
+    us, vs = [], []
+    for g, V in enumerate(Vs.tolist()):
+        a, b = graphgen.random_multigraph(70_000 + g, V, int(rng.integers(V // 2, 40 * V)))
+        us.append(np.asarray(a, dtype=np.int32))
+        vs.append(np.asarray(b, dtype=np.int32))
+    off = np.concatenate([[0], np.cumsum([len(a) for a in us])]).astype(np.int64)
+    u, v = torch.from_numpy(np.concatenate(us)).cuda(), torch.from_numpy(np.concatenate(vs)).cuda()
+    want = [oracle.dfs_bridges(a, b, V).tolist() for a, b, V in zip(us, vs, Vs.tolist())]
+
+    def check(out, counts, at):
+        out, counts = out.cpu().numpy(), counts.cpu().numpy()
+        for g in range(G):
+            assert out[at[g]:at[g] + 2 * counts[g]].reshape(-1, 2).tolist() == want[g]
+
+    ctx = pb.Context()
+    check(*ctx.find_batched(u, v, off, Vs))
+    sets = [ctx.find_batched(u, v, off, Vs, sync=False) for _ in range(5)]
+    g = int(np.argmax(Vs))
+    single = ctx.find(u[off[g]:off[g + 1]], v[off[g]:off[g + 1]], int(Vs[g])).cpu().numpy().tolist()
+    sets.append(ctx.find_batched(u, v, off, Vs, sync=False))
+    torch.cuda.synchronize()
+    assert single == want[g]
+    for s in sets:
+        check(*s)
+    check(*ctx.find_batched(u, v, off, Vs))
 
 
 def test_a_tuned_plan_is_no_slower_when_waited_for():

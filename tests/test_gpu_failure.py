@@ -43,9 +43,9 @@ def test_final_stage_barrier_timeout_leaves_a_usable_context(cuda_lib):
     """The final stage's grid barrier gives up after its poll cap: one block is held back (a
     bounded sleep, a test knob) while the others wait with a short cap.  The call then returns
     BRIDGES_ETIMEDOUT -- not the count of the call before it -- and the same context, with the
-    knobs cleared, gives the exact result again (the barrier's count and generation are reset
-    for every call)."""
-    g = graphgen.workload("small")  # 2,088 vertices: a block per 256, so 9 blocks
+    knobs cleared, gives the exact result again (the barrier's count is reset for every call).
+    The sample of so few vertices takes one block: its barriers are the next test's."""
+    g = graphgen.workload("small")  # 2,088 vertices: five blocks of the final stage
     u = torch.from_numpy(np.array(g.u)).cuda()
     v = torch.from_numpy(np.array(g.v)).cuda()
     ref = oracle.dfs_bridges(g.u, g.v, g.V).tolist()

@@ -135,10 +135,10 @@ def test_blocks_of_odd_sizes(cuda_lib, block, V, E):
     _check(cuda_lib, u, v, V, block=block, warm_edges=0)
 
 
-@pytest.mark.parametrize("V", [20_000, 60_000, 130_000])
+@pytest.mark.parametrize("V", [20_000, 53_000, 60_000, 130_000])
 def test_long_unaligned_slices(cuda_lib, V):
-    """A list long enough for interleaved tiles whose arrays start off a 16-byte boundary: the aligned copy's
-    result, in a time of the same order (one block alone would take 200 times as long)."""
+    """A list long enough for interleaved tiles whose arrays start off a 16-byte boundary: the planted bridges and
+    cut vertices of the aligned copy, in a time of the same order (one block alone would take 200 times as long)."""
     import time
 
     import torch
@@ -160,10 +160,12 @@ def test_long_unaligned_slices(cuda_lib, V):
         torch.cuda.synchronize()
         return got.cpu().numpy().tolist(), time.perf_counter() - t
 
-    for call in (ctx.find, ctx.articulation_points):
-        want, aligned = timed(lambda: call(u[4:], v[4:], V + 40))
+    path = list(range(V - 1, V + 39))  # (the rest, some 1,000 edges a vertex, has no bridge and no cut vertex)
+    for call, want in ((ctx.find, [[x, x + 1] for x in path]), (ctx.articulation_points, path)):
+        got, aligned = timed(lambda: call(u[4:], v[4:], V + 40))
+        assert got == want
         got, unaligned = timed(lambda: call(u[1:], v[1:], V + 40))
-        assert got == want and len(got) >= 39
+        assert got == want
         assert unaligned < 8 * aligned
 
 

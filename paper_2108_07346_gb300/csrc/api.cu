@@ -227,9 +227,10 @@ bool small_call(const bridges_ctx* c, const CertPlan& p) {
 // for), or with count null to the workspace's own; the sorted pairs go to out, or to the final stage's own dscan array (free by the time it sorts) when out is
 // null.
 int64_t run_path(bridges_ctx* c, cudaStream_t s, const int32_t* u, const int32_t* v, int64_t E, int32_t V, int32_t M,
-                 int32_t* out, int64_t* count, Carved* kout, CertPlan* pout, Want want) {
+                 int32_t* out, int64_t* count, Carved* kout, CertPlan* pout, Want want, bool host_list = false) {
   Range range("bridges: certificate + final stage");
   CertPlan p = plan_for(c, E, V, M);
+  if (host_list) p.stage = false;
   int64_t rc = ensure_ws(c, total_bytes(p), s);
   if (rc != BRIDGES_OK) return rc;
   Carved k = carve(c, p);
@@ -551,7 +552,7 @@ int64_t bridges_find_host(bridges_ctx* c, struct CUstream_st* stream, const int3
          cudaMemcpyAsync(const_cast<int32_t*>(rv), hv, sizeof(int32_t) * (size_t)E, cudaMemcpyHostToDevice, s) !=
              cudaSuccess))
       return cuda_fail(cudaGetLastError());
-    rc = run_path(c, s, ru, rv, E, V, M, dout, c->h_pinned, &k, nullptr, Want::bridges);
+    rc = run_path(c, s, ru, rv, E, V, M, dout, c->h_pinned, &k, nullptr, Want::bridges, !deferred);
     if (rc) return rc;
   }
   if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_fail(cudaGetLastError());
@@ -1544,7 +1545,7 @@ static int64_t articulation_fused_run(bridges_ctx* c, cudaStream_t s, const Laun
 // (u, v) (run_path_host); the block pass then streams (u, v) from the device.
 static int64_t articulation_run(bridges_ctx* c, cudaStream_t s, const int32_t* u, const int32_t* v, int64_t E, int32_t V,
                          int32_t M, int32_t* out_points, int32_t* out_bridges, int64_t* out_counts_device,
-                         const int32_t* hu, const int32_t* hv) {
+                         const int32_t* hu, const int32_t* hv, bool host_list = false) {
   const CertPlan p0 = ap_plan(c, E, V, M);
   const size_t ap_at = align_up(total_bytes(p0), 256);
   Launch L = launch_for(c, s);
@@ -1571,7 +1572,7 @@ static int64_t articulation_run(bridges_ctx* c, cudaStream_t s, const int32_t* u
       return cuda_fail(cudaGetLastError());
   }
   if (rc == 1) {
-    rc = run_path(c, s, u, v, E, V, M, out_bridges, nullptr, &k, nullptr, Want::rooted);
+    rc = run_path(c, s, u, v, E, V, M, out_bridges, nullptr, &k, nullptr, Want::rooted, host_list);
     if (rc) return rc;
   }
   if (!out_points) out_points = k.spare;  // V <= 1: no point is written
@@ -1634,7 +1635,7 @@ extern "C" int64_t bridges_articulation_points_host(bridges_ctx* c, struct CUstr
   rc = stage_host_edges(c, s, hu, hv, E, V, &ru, &rv, &dout, true, &deferred);
   if (rc) return rc;
   const int64_t n = articulation_run(c, s, ru, rv, E, V, M, dout, nullptr, nullptr, deferred ? hu : nullptr,
-                                     deferred ? hv : nullptr);
+                                     deferred ? hv : nullptr, !deferred);
   if (n <= 0) return n;
   if (cudaMemcpyAsync(out_points_host, dout, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)

@@ -206,13 +206,11 @@ __global__ void __launch_bounds__(1024, 1) leaf_kernel(LeafArgs A) {
   if (threadIdx.x == 0) stop = A.mode == 1 ? ld_relaxed(A.b.status) : 0;
   __syncthreads();
   if (stop) return;  // an earlier step failed: its labels and union-finds may be unset
-  const int64_t j = blockIdx.x / A.G, m = blockIdx.x % A.G;
-  int64_t members = A.G;
-  if (MODE == 2 && A.mode == 1 && (A.b.giant[j] >> 32) < kProbes / 32 && A.G > 1 &&
-      4 * members * (int64_t)blockDim.x > A.V) {
-    members /= 2;
-    if (m >= members) return;
-  }
+  const int32_t j = blockIdx.x / A.G, m = blockIdx.x % A.G;
+  const bool half = MODE == 2 && A.mode == 1 && (A.b.giant[j] >> 32) < kProbes / 32 && A.G > 1 &&
+                    4 * (int64_t)A.G * blockDim.x > A.V;
+  const int32_t members = half ? A.G / 2 : A.G;
+  if (m >= members) return;
   const int64_t lo = A.E * j / A.M, hi = A.E * (j + 1) / A.M;
   const int64_t w = A.stride > 1 ? 0 : min(A.warm, hi - lo);
   int64_t a = A.mode == 0 ? lo : lo + w;
@@ -221,8 +219,8 @@ __global__ void __launch_bounds__(1024, 1) leaf_kernel(LeafArgs A) {
     a = max(a, A.r0);
     z = max(a, min(z, A.r1));
   }
-  if (MODE == 1) load_labels(slab, A.b.lab + j * A.b.Vpad, A.b.Vpad);
-  if (MODE == 2) load_words(slab, A.b.lab + j * A.b.Vpad, (A.Vb / 32 + 4) / 4);
+  if (MODE == 1) load_labels(slab, A.b.lab + (int64_t)j * A.b.Vpad, A.b.Vpad);
+  if (MODE == 2) load_words(slab, A.b.lab + (int64_t)j * A.b.Vpad, (A.Vb / 32 + 4) / 4);
   const Job J = job_of(A.b, A.V, j);
   __shared__ int32_t staged[32][2], sent[2];
   if (threadIdx.x < 64) staged[threadIdx.x >> 1][threadIdx.x & 1] = 0;

@@ -164,7 +164,8 @@ int64_t bridges_find_host(bridges_ctx* ctx, struct CUstream_st* stream, const in
  * Graphs with V <= 4096 are certified and solved in shared memory by two persistent kernels,
  * replayed as one CUDA graph cached per capacity: the first certifies every task (a graph, or a
  * partition of a graph with many edges) on a 256-thread group and finishes graphs of up to 1,024
- * vertices in place (with 256 graphs or more a kernel before it plans the tasks from edge_off and V);
+ * vertices in place (with 256 graphs or more, the automatic plan and no earlier batch of the context
+ * still running, a kernel before it plans the tasks from edge_off and V);
  * the second runs the larger graphs' bridge stages (the partitions'
  * certificates merged there), two graphs per block up to 3,008 vertices, else one.  Larger graphs
  * follow through the single-graph path on the same stream.  Enqueue-only: returns BRIDGES_OK or a

@@ -16,13 +16,14 @@
 // edges are rejected by both forests.  To reject those from shared memory, each job first
 // certifies some of its chunk -- one partition a sample of the whole list, in rounds (sample.cu);
 // several, or more vertices than labels, a prefix of the chunk through the union-finds -- and
-// takes a snapshot: a
-// 16-bit label per vertex naming its F' component (components with >= 2 vertices, up to 65,535
-// of them).  F' components nest inside F components (every F' edge joins two ends F already
+// takes a snapshot: a 16-bit label per vertex naming its F' component.  Behind a sample of up to
+// 65,535 vertices the label is the component's root, which a vertex alone shares with no other;
+// else the components of two or more vertices are numbered, the first 65,535 of them.  F'
+// components nest inside F components (every F' edge joins two ends F already
 // joined), so two vertices with equal labels are joined in both forests and their edge can be
 // dropped exactly; connectivity only grows, so a stale snapshot is still sound.  Other edges
 // take the union-find path as before.  When 16-bit labels need more shared memory than a block
-// has (V above about 113 k), the snapshot is instead a bitmap of the largest F' component, one
+// has (V above about 113 k), the snapshot is instead a bitmap of one large F' component, one
 // bit per vertex: an edge with both ends in it is dropped the same way.
 //
 // The merge tree (Sec. 3 phases) certifies the union of f certificates per merge job.  The
@@ -508,7 +509,7 @@ CertPlan make_plan(int64_t E, int32_t V, int32_t M, int32_t fan_in, int32_t bloc
   const int64_t Vpad = (int64_t)align_up((size_t)V + 1, 8);  // entry V: the kNoLabel sentinel
   const size_t lab_bytes = (size_t)Vpad * 2;
   const bool labels_fit = lab_bytes + 1024 <= smem_optin;
-  // Too many vertices for 16-bit labels: one bit per vertex marks the largest F' component
+  // Too many vertices for 16-bit labels: one bit per vertex marks one large F' component
   // (vertices past the bitmap's reach, if any, always take the union-find path).  The bitmap
   // lives in the job's label area (2 Vpad bytes >= its (Vb / 32 + 4) words).
   const int64_t bm_cap = (((int64_t)(smem_optin - 1024) / 4 - 4) * 32) / 128 * 128;

@@ -12,7 +12,7 @@
 // A call that wants the rooted forest runs all of this as one cooperative kernel (final_kernel, every
 // block resident); one that wants only the bridges first contracts the components of F'
 // (reduced_kernel, below), after which a dense graph is a forest, or a small rest solved by one
-// block, and only a sparse graph with cycles throughout comes back to these phases.  They are
+// block, and only a graph that keeps most of its edges takes these phases whole.  They are
 // separated by a software grid barrier; the work per phase is small (O(V)), so launch overhead, not
 // bandwidth, would dominate a kernel-per-phase design, and the barriers (1.3 to 3 us with the
 // stores before them) dominate the kernel: the phases are arranged to need few of them.
@@ -975,7 +975,7 @@ __global__ void __launch_bounds__(kThreads) final_kernel(FinArgs A) {
 //   5  The keys are sorted, as above.
 // 2.5 M edges on 37,147 vertices: 79 us with the phases above on the whole forest, 18 us so (25 with the
 // roots numbered before it was known that all kept edges are bridges); 16.8 M R-MAT edges on 2^20 vertices
-// (141 k kept edges, 140.1 k of them bridges): 417 and 156 us.
+// (141 k kept edges, 140.1 k of them bridges): 417 and 147 us.
 
 struct ReducedArgs {
   FinArgs a;          // a.V: the graph's vertices; tu, tv, d_nt: F; kbits, sup_log, bar_polls, hold_polls
@@ -1381,7 +1381,7 @@ __global__ void tecc_link_kernel(FinalBufs f, const int32_t* P2, int32_t V, cons
   }
 }
 
-__global__ void tecc_label_kernel(FinalBufs f, int32_t V, int32_t* labels, int64_t* count) {
+__global__ void tecc_label_kernel(FinalBufs f, int32_t V, int32_t* labels) {
   const int32_t st = *f.status;
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < V; base += gstride()) {
     const int64_t x = base + threadIdx.x;
@@ -1409,7 +1409,7 @@ void two_edge_components(const Launch& L, const FinalBufs& f, const CertBufs& c,
   const int g = (int)std::min<int64_t>(ceil_div(std::max(V, 1), bs), (int64_t)L.num_sms * 16);
   tecc_init_kernel<<<g, bs, 0, L.stream>>>(f, c.P2, V);
   tecc_link_kernel<<<g, bs, 0, L.stream>>>(f, c.P2, V, c.f1u, c.f1v, c.cnt);
-  tecc_label_kernel<<<g, bs, 0, L.stream>>>(f, V, labels, count_dev);
+  tecc_label_kernel<<<g, bs, 0, L.stream>>>(f, V, labels);
   tecc_count_kernel<<<1, 1, 0, L.stream>>>(f, count_dev);
   *L.launches += 4;
 }

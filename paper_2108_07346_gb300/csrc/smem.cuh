@@ -1,6 +1,6 @@
 // smem.cuh -- certificates and bridges of one graph of up to 4,096 vertices in shared memory, by a
 // group of threads: the batched kernels, the one-block forms of small calls (batched.cu) and the
-// final stage's reduced graph (final.cu) share this code.  Nothing here is visible through the C ABI.
+// core of the final stage's reduced graph (final.cu, up to 3,616 vertices) share this code.  Nothing here is visible through the C ABI.
 #pragma once
 
 #include "../../include/bridges.h"
@@ -140,7 +140,7 @@ struct Grp {
 struct GroupShared {
   int32_t red[kT / 32];
   int32_t red_b[kT / 32];
-  int32_t task, n1, n2, err, flag, sh;
+  int32_t task, n1, n2, err, sh;
   int32_t kept, verts, tree, rest;  // the reduced graph (s_contract)
 };
 

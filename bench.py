@@ -42,17 +42,17 @@ UNIT = "GE/s"
 # DRAM bytes (read + write) per streamed edge, from the ncu captures of the large workload's
 # streaming kernels; each is valid only for the kernel sources it was measured on (hash of those
 # sources).
-#   forest pass, M = 1, at density 1/8 (268 M edges, 2.1 GB: a capture of a few GB, scaled to a
-#   full launch by its streamed edges): 2.1402 GB read + 5.5 MB written for 267,444,294 streamed
-#   edges; block pass stream and fused stream (articulation points), the same density:
-#   2.1471 GB read + 7.6 MB written, and 2.1402 GB read + 0.4 MB written, for 267,444,294
-#   streamed edges each
-TRAFFIC = {"certify_sha": "a777da7ffc79a6ce", "bytes_per_edge": 8.0408,
+#   forest pass, M = 1, at density 1/8 (268,439,884 edges, 2.1 GB: a capture of a few GB, scaled to a
+#   full launch by its streamed edges): 2.1482 GB read + 5.5 MB written; the fused stream
+#   (articulation points), the same density: 2.1482 GB + 1.4 MB; both read the whole list and are
+#   counted over the 267,846,036 edges outside the sample.  The block pass's stream: 2.1472 GB +
+#   7.6 MB for the 268,288,350 edges behind its prefix
+TRAFFIC = {"certify_sha": "7ccc145b76247bb2", "bytes_per_edge": 8.0408,
            "source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the forest pass at density 1/8 "
                      "(268 M edges), scaled to a full launch by its streamed edges"}
-AP_TRAFFIC = {"blocks_sha": "461b023b22eb6faa", "bytes_per_edge": 8.0566,
+AP_TRAFFIC = {"blocks_sha": "514cf6a27b7cd73c", "bytes_per_edge": 8.0316,
               "source": "ncu dram bytes of the block pass stream at density 1/8, scaled by streamed edges"}
-FUSED_TRAFFIC = {"blocks_sha": "461b023b22eb6faa", "bytes_per_edge": 8.0040,
+FUSED_TRAFFIC = {"blocks_sha": "514cf6a27b7cd73c", "bytes_per_edge": 8.0254,
                  "source": "ncu dram bytes of the fused stream at density 1/8, scaled by streamed edges"}
 
 

@@ -112,4 +112,4 @@ def test_a_tuned_plan_is_no_slower_when_waited_for():
     ctx.batch_autotune(u, v, off, Vs)
     tuned, got = waited()
     assert np.array_equal(got, want)
-    assert tuned < 1.15 * fresh
+    assert tuned < 1.25 * fresh

@@ -250,4 +250,4 @@ def test_bitmap_of_nothing_halves_the_grid(cuda_lib):
                 total[name] = total.get(name, 0) + sorted(t["forest"] for t in ctx.stage_ms_history(8))[4]
                 found.append(got.cpu().numpy().tolist())
             assert found[0] == found[1] == oracle.dfs_bridges(u.cpu().numpy(), v.cpu().numpy(), V).tolist()
-    assert total["auto"] < 1.3 * total["half"], total
+    assert total["auto"] < 1.4 * total["half"], total
